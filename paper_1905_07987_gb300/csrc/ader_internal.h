@@ -93,6 +93,13 @@ struct LimArgs {
   int first_order;       // FV recompute with zero slopes (the first-order fallback pass)
 };
 
+// Cells of a block of the elastic predictors (one thread per node; several cells at low order).
+__host__ __device__ constexpr int ck_cells_per_block(int order) {
+  return (order + 1) * (order + 1) * (order + 1) >= 96
+             ? 1
+             : 128 / ((order + 1) * (order + 1) * (order + 1));
+}
+
 // Arguments of the adjoint kernels of the linear elastic step.
 struct AdjArgs {
   const double* u_n;     // forward state at t^n [C][NL]
@@ -116,6 +123,7 @@ struct EnsTable {
   int nr;                              // runs
   int pblocks;                         // persistent blocks of the predictor (SMs x blocks per SM)
   long long cell0[ENS_MAXR + 1];       // first concatenated cell of run r; cell0[nr] = total
+  long long blk0[ENS_MAXR + 1];        // the same for the predictor's blocks of cells
   long long face0[3][ENS_MAXR + 1];    // the same for the faces of direction d
   long long phioff[3][ENS_MAXR];       // run-local offset of direction d's fluxes
 };
@@ -177,6 +185,12 @@ struct StepArgs {
   // elastic: per face (directions concatenated) the wave speed max(vp_L, vp_R) and the nine
   // path-averaged coefficients of B_d, formed when the material is set (null: formed per step)
   const double* fmat;
+  // elastic, Picard predictor: the iterates are polynomials of the spatial operator L applied to
+  // u^n (and to the source), so the time average needs nlev applications of L and these tables
+  // (device memory, see build_linear_levels in api.cu): weights wk[nlev + 1] of the Taylor-scaled
+  // levels, then nlev rows of n + 3 weights of the wavelet samples (time nodes, 0, 1/2, 1).
+  const double* lin;
+  int nlev;
   // hybrid limiter: the cells with FV steps left (nonzero) skip the predictor; their face
   // neighbours compute with FV too, so nothing kept reads their DG data (null: every cell)
   const uint8_t* skip;

@@ -4,6 +4,7 @@
 #include <cstdlib>
 #include <algorithm>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -218,6 +219,89 @@ void build_tables_f(int order, const Tables& T, TablesF& F) {
   }
 }
 
+// Tables of the Picard predictor of a linear system (StepArgs::lin, kernels_ck.cuh).  With
+// Lambda = dt L every iterate at time node t is
+//   q_t = sum_k C_k[t] Lambda^k u + sum_k (sum_m G_k[t][m] s_m) dt Lambda^k g,
+// s_m the wavelet's samples (time nodes, then 0, 1/2, 1), and one iteration
+// q <- u + Kw (Lambda q + dt g s) maps the coefficients by C_{k+1} <- Kw C_k, C_0 <- 1 and
+// G_{k+1} <- Kw G_k, G_0 <- Kw.  So after `iters` iterations the first `iters` levels are powers of
+// Kw and the guess's own coefficients follow, multiplied by Kw^iters.  Stored: the time averages
+// of the coefficients of the scaled levels a_k = (prod_{i<k} phi_i) Lambda^k u with phi_0 = 1 and
+// phi_k = 1/2 after it (the spectral radius of Kw is below 0.41: the scaled weights fall).
+std::vector<double> build_linear_levels(int order, const Tables& T, int iters, bool cerk) {
+  const int n = order + 1, ns = n + 3;
+  typedef std::vector<double> Vec;
+  const auto phi = [](int k) { return k == 0 ? 1.0 : 0.5; };
+  const auto times_kw = [&](const Vec& a) {  // a[t][..] -> sum_m Kw[t][m] a[m][..]
+    const size_t w = a.size() / n;
+    Vec b(a.size(), 0.0);
+    for (int t = 0; t < n; ++t)
+      for (int m = 0; m < n; ++m)
+        for (size_t i = 0; i < w; ++i) b[t * w + i] += T.Kw[t][m] * a[m * w + i];
+    return b;
+  };
+  // the guess: coefficients of u (C0[k][t]) and of the source (G0[k][t][m])
+  std::vector<Vec> C0(1, Vec(n, 1.0)), G0;
+  if (cerk) {
+    // stages dt k_i = Lambda (u + c_i dt k_{i-1}) + dt g s(c_i): coefficients of Lambda^k u and of
+    // dt Lambda^k g times the stage samples, accumulated with the dense-output weights
+    C0.resize(5, Vec(n, 0.0));
+    G0.assign(4, Vec((size_t)n * ns, 0.0));
+    const double c[4] = {0.0, 0.5, 0.5, 1.0};
+    const int smp[4] = {n, n + 1, n + 1, n + 2};
+    double U[5] = {}, S[4][4] = {};  // S[level][stage whose sample it takes]
+    for (int i = 0; i < 4; ++i) {
+      for (int k = 3; k >= 1; --k)
+        for (int q = 0; q < 4; ++q) S[k][q] = c[i] * S[k - 1][q];
+      for (int q = 0; q < 4; ++q) S[0][q] = q == i ? 1.0 : 0.0;
+      for (int k = 4; k >= 2; --k) U[k] = c[i] * U[k - 1];
+      U[1] = 1.0;
+      for (int t = 0; t < n; ++t) {
+        const double b = T.cerk[i == 0 ? 0 : (i == 3 ? 2 : 1)][t];
+        for (int k = 1; k < 5; ++k) C0[k][t] += b * U[k];
+        for (int k = 0; k < 4; ++k)
+          for (int q = 0; q < 4; ++q) G0[k][t * ns + smp[q]] += b * S[k][q];
+      }
+    }
+  }
+  // levels of q after the iterations
+  const size_t K = (size_t)iters + C0.size() - 1;
+  std::vector<double> out(2 * K + 1 + K * ns, 0.0);
+  double scale = 1.0;  // 1 / prod phi
+  const auto average = [&](const Vec& a, size_t w, size_t i) {
+    double s = 0.0;
+    for (int t = 0; t < n; ++t) s += T.w[t] * a[t * w + i];
+    return s;
+  };
+  Vec c(n, 1.0), g((size_t)n * ns, 0.0);
+  for (int t = 0; t < n; ++t)
+    for (int m = 0; m < n; ++m) g[(size_t)t * ns + m] = T.Kw[t][m];
+  // the guess's levels carry Kw^iters times what follows Lambda^iters
+  std::vector<Vec> Ct = C0, Gt = G0;
+  for (int it = 0; it < iters; ++it) {
+    for (Vec& a : Ct) a = times_kw(a);
+    for (Vec& a : Gt) a = times_kw(a);
+  }
+  for (size_t k = 0; k <= K; ++k) {
+    if (k < (size_t)iters) {
+      out[k] = scale * average(c, 1, 0);
+      c = times_kw(c);
+    } else {
+      out[k] = scale * average(Ct[k - iters], 1, 0);
+    }
+    if (k == K) break;
+    out[K + 1 + k] = phi((int)k);
+    if (k < (size_t)iters) {
+      for (int m = 0; m < ns; ++m) out[2 * K + 1 + k * ns + m] = scale * average(g, ns, m);
+      g = times_kw(g);
+    } else if (k - iters < Gt.size()) {
+      for (int m = 0; m < ns; ++m) out[2 * K + 1 + k * ns + m] = scale * average(Gt[k - iters], ns, m);
+    }
+    scale /= phi((int)k);
+  }
+  return out;
+}
+
 // Solve A x = b for several right-hand sides (Gauss-Jordan, partial pivoting); A is m x m.
 bool solve_dense(int m, std::vector<double> A, std::vector<double>& B, int nrhs) {
   for (int c = 0; c < m; ++c) {
@@ -333,6 +417,8 @@ struct ader_ctx {
   cudaEvent_t hb_ev[4] = {nullptr, nullptr, nullptr, nullptr};
   double* face = nullptr;
   double* phi = nullptr;
+  double* lin = nullptr;     // elastic, Picard predictor: weights of its polynomial levels
+  int nlev = 0;
   double* fmat = nullptr;    // elastic: per-face material terms of the Riemann solver
   double* fspeed = nullptr;  // mixed Euler: face wave speeds evaluated by the predictor
   double* mat = nullptr;
@@ -393,6 +479,7 @@ static void free_all(ader_ctx* c) {
   cudaFree(c->face);
   cudaFree(c->phi);
   cudaFree(c->fmat);
+  cudaFree(c->lin);
   cudaFree(c->hb_in);
   cudaFree(c->hb_out);
   if (c->hb_cin) cudaStreamDestroy(c->hb_cin);
@@ -561,6 +648,22 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
     e = cudaMalloc(&c->fspeed, ncells * cfg->dim * 2 * c->nf * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->dev, sizeof(DevScalars));
   if (e == cudaSuccess && cfg->pde == ADER_PDE_ELASTIC) e = cudaMalloc(&c->mat, ncells * 3 * sizeof(double));
+  if (e == cudaSuccess && cfg->pde == ADER_PDE_ELASTIC && cfg->predictor == ADER_PREDICTOR_PICARD) {
+    // (a host allocation that fails for an absurd number of iterations is ADER_ENOMEM)
+    try {
+      const int it = cfg->picard_iters > 0 ? cfg->picard_iters : cfg->order + 1;
+      const bool cerk = cfg->initial_guess == ADER_GUESS_CERK;
+      const std::vector<double> lv = build_linear_levels(cfg->order, c->tab, it, cerk);
+      c->nlev = it + (cerk ? 4 : 0);
+      e = cudaMalloc(&c->lin, lv.size() * sizeof(double));
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->lin, lv.data(), lv.size() * sizeof(double), cudaMemcpyHostToDevice,
+                            c->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    } catch (const std::exception&) {
+      e = cudaErrorMemoryAllocation;
+    }
+  }
   if (cfg->limiter) {
     const int ns = 2 * cfg->order + 1;
     c->nss = 1;
@@ -896,6 +999,8 @@ static StepArgs make_args(ader_ctx* c, double dt, double t_end) {
   a.phi = c->phi;
   a.mat = c->mat;
   a.fmat = c->mat_set ? c->fmat : nullptr;
+  a.lin = c->lin;
+  a.nlev = c->nlev;
   a.dev = c->dev;
   a.iters = c->cfg.picard_iters > 0 ? c->cfg.picard_iters : c->cfg.order + 1;
   a.cerk = c->cfg.initial_guess == ADER_GUESS_CERK ? 1 : 0;
@@ -1526,6 +1631,8 @@ static ader_status ens_capture_persistent(ader_ensemble* e, int steps, double dt
   for (int r = 0; r < nr; ++r) {
     const ader_ctx* c = e->runs[r];
     E.cell0[r + 1] = E.cell0[r] + c->g.ncells;
+    const int cpb = ck_cells_per_block(c->cfg.order);
+    E.blk0[r + 1] = E.blk0[r] + (c->g.ncells + cpb - 1) / cpb;
     long long off = 0;
     for (int d = 0; d < c->g.dim; ++d) {
       const long long nf = (long long)(c->g.n[d] + 1) * (c->g.ncells / c->g.n[d]);
@@ -1698,15 +1805,11 @@ ader_status ader_ensemble_autotune(ader_ensemble* e, double dt, int* best, doubl
                             cudaMemcpyDeviceToDevice, e->stream));
   }
   // candidates: (branches, persistent blocks per SM); branches 0 = one persistent launch per
-  // phase for all runs
+  // phase for all runs.  The fused launch (-1) is left to ader_ensemble_set_launch.
   std::vector<std::pair<int, int>> cand = {{1, 1}, {2, 1}, {4, 1}};
   if (ens_batchable(e, dt)) {
     cand.push_back({0, 1});
     cand.push_back({0, 2});
-    if (e->runs[0]->fam->ens_fused && e->runs[0]->cfg.predictor == ADER_PREDICTOR_PICARD) {
-      cand.push_back({-1, 1});
-      cand.push_back({-1, 2});
-    }
   }
   const int cand_s[] = {2, 4};
   cudaEvent_t t0, t1;

@@ -10,6 +10,8 @@ cudaError_t ens_step_elastic3_mixed(const StepArgs* R, const EnsTable& E, const 
                                     const TablesF& F, int order, cudaStream_t s);
 cudaError_t predictor_ck_elastic3(const StepArgs& a, const Tables& t, const TablesF& f, int prec,
                                   cudaStream_t s);
+cudaError_t predictor_picard_elastic3(const StepArgs& a, const Tables& t, const TablesF& f,
+                                      int prec, cudaStream_t s);
 cudaError_t ens_step_ck_elastic3(const StepArgs* R, const EnsTable& E, const Tables& T,
                                  const TablesF& F, int prec, int order, cudaStream_t s);
 cudaError_t ens_fused_elastic3_fp64(const StepArgs* R, const EnsTable& E, const Tables& T,
@@ -157,6 +159,7 @@ cudaError_t launch_face_material_elastic(const Geometry& g, const double* mat, c
 const Family* family_elastic3() {
   static Family f = [] {
     Family g = *FamilyImpl<Elastic, 3>::get();
+    g.predictor = &predictor_picard_elastic3;
     g.adj_run = &adj_run;
     g.adj_run_ck = &adj_run_ck;
     g.adj_scratch_per_block = &adj_scratch;

@@ -65,37 +65,6 @@ __device__ __forceinline__ void contract_lines(const double* X, const double* Dm
   }
 }
 
-// Elastic: each row v of B_d has one non-zero coef(d,v) at column src(d,v); the NCP term
-// B_d dq/dx_d is contracted directly from q (no flux buffer).
-template <class C, int d, int RS>
-__device__ __forceinline__ void contract_ncp_elastic(const double* X, const double* Dm,
-                                                     double inv_h, double irho, double lam,
-                                                     double mu, double (&R)[C::LPT][C::n],
-                                                     int tid) {
-  constexpr int n = C::n, NV = C::NV, NL = C::NL, TPB = C::TPB, st = ipow(n, d);
-#pragma unroll
-  for (int k = 0; k < C::LPT; ++k) {
-    const int l = tid + k * TPB;
-    if (l < NL) {
-      const int j = l / NV, v = l - (l / NV) * NV;
-      const int s = Elastic::src(d, v);
-      if (s >= 0) {
-        const double coef = -Elastic::coef_ir(d, v, irho, lam, mu) * inv_h;
-        const int jd = digit<n, d>(j);
-        const int j0 = j - jd * st;
-        const double* Dr = Dm + jd * RS;
-#pragma unroll
-        for (int t = 0; t < n; ++t) {
-          double acc = 0.0;
-#pragma unroll
-          for (int m = 0; m < n; ++m) acc = fma(Dr[m], X[t * NL + (j0 + m * st) * NV + s], acc);
-          R[k][t] = fma(coef, acc, R[k][t]);
-        }
-      }
-    }
-  }
-}
-
 // Shallow water: the derivative of the surface h + b along every direction at the owned
 // space-time nodes, G[node][d] = sum_m D[j_d][m] (h + b)(t, j with j_d -> m) (node = t NS + j,
 // m ascending), one thread per node so that every lane works; the momentum lines of direction d
@@ -179,8 +148,8 @@ __device__ __forceinline__ void load_nodes(const double* qs, const PdeParams& pp
 }
 
 // Continuous extension Runge-Kutta guess of the predictor (Sec. 5): the classical four-stage
-// Runge-Kutta method on the cell-local ODE dq/dt = R(q) (flux divergence or non-conservative
-// product of one time level, point source at the stage time), and its natural continuous
+// Runge-Kutta method on the cell-local ODE dq/dt = R(q) (flux divergence of one time level), and
+// its natural continuous
 // extension of uniform order 3 evaluated at the time nodes:
 //   q_t = u + dt (b1(x_t) k1 + b2(x_t) (k2 + k3) + b4(x_t) k4)   (weights: T.cerk)
 // written to the n time slices of qs.  Called once per cell before the Picard iterations (not
@@ -188,12 +157,10 @@ __device__ __forceinline__ void load_nodes(const double* qs, const PdeParams& pp
 template <class P, int D, int N>
 __device__ __noinline__ void cerk_guess_cell(const StepArgs& A, const Tables& T, double* qs,
                                              double* Fs, const double* sD, const double* ul,
-                                             double irho, double lam, double mu, bool has_src,
                                              int tid) {
   using C = Cfg<P, D, N>;
   constexpr int n = C::n, NV = C::NV, NL = C::NL, NS = C::NS, TPB = C::TPB, LPT = C::LPT;
   const double dt = A.dev->dt;
-  const double tn = A.dev->t;
   double kst[4][LPT];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -208,7 +175,7 @@ __device__ __noinline__ void cerk_guess_cell(const StepArgs& A, const Tables& T,
     double R1[LPT];
 #pragma unroll
     for (int k = 0; k < LPT; ++k) R1[k] = 0.0;
-    if constexpr (P::CONS) {
+    {
 #pragma unroll
       for (int d = 0; d < D; ++d) {
         for (int j = tid; j < NS; j += TPB) {
@@ -238,41 +205,6 @@ __device__ __noinline__ void cerk_guess_cell(const StepArgs& A, const Tables& T,
         __syncthreads();
       }
     }
-    if constexpr (P::NCP) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
-#pragma unroll
-        for (int k = 0; k < LPT; ++k) {
-          const int l = tid + k * TPB;
-          if (l < NL) {
-            const int j = l / NV, v = l - (l / NV) * NV;
-            const int sv = Elastic::src(d, v);
-            if (sv >= 0) {
-              const double coef = -Elastic::coef_ir(d, v, irho, lam, mu) * A.g.inv_h[d];
-              const int jd = (j / st) % n, j0 = j - jd * st;
-              double acc = 0.0;
-#pragma unroll
-              for (int m = 0; m < n; ++m) acc = fma(sD[jd * n + m], qs[(j0 + m * st) * NV + sv], acc);
-              R1[k] = fma(coef, acc, R1[k]);
-            }
-          }
-        }
-      }
-    }
-    if (has_src) {
-      const double tau = fma(ca, dt, tn) - A.src.t0;
-      const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
-      const double ric = (1.0 - 2.0 * a) * exp(-a);
-#pragma unroll
-      for (int k = 0; k < LPT; ++k) {
-        const int l = tid + k * TPB;
-        if (l < NL) {
-          const int j = l / NV, v = l - (l / NV) * NV;
-          if (v >= 3) R1[k] = fma(-A.src.M[v - 3] * A.src.phi[j], ric, R1[k]);
-        }
-      }
-    }
 #pragma unroll
     for (int k = 0; k < LPT; ++k) kst[i][k] = R1[k];
     __syncthreads();  // the next stage overwrites slice 0
@@ -293,9 +225,9 @@ __device__ __noinline__ void cerk_guess_cell(const StepArgs& A, const Tables& T,
 // cell-local part of the face terms of Eq. (6), and the face extrapolations.
 //   q^0 = u (or the continuous extension Runge-Kutta guess, A.cerk);
 //   q^{r+1} = u + dt Kw R(q^r)  (Kw = K1^{-1} diag(w), K1^{-1} e0 = 1)
-//   R(q) = -sum_d (1/h_d) D_d F_d(q) - sum_d (1/h_d) B_d D_d q + point source
-// One cell c (all threads of the block; called by the per-context kernel and by the persistent
-// ensemble kernel).
+//   R(q) = -sum_d (1/h_d) D_d F_d(q) (- the state-dependent product of the shallow water equations)
+// The conservative systems; the linear elastic system has its own form (kernels_ck.cuh).
+// One cell c (all threads of the block).
 template <class P, int D, int N>
 __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& T, long long c) {
   using C = Cfg<P, D, N>;
@@ -307,7 +239,6 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
   double* G = Fs + C::FSLOTS * NL;  // [NST][D] surface derivatives (shallow water)
   const int tid = threadIdx.x;
   const double dt = A.dev->dt;
-  const double tn = A.dev->t;
   const double* u = A.u + c * NL;
   // D and c0/c1 are indexed by a per-lane row: staged in shared memory
   __shared__ double sD[n * n], sC[2][n];
@@ -328,29 +259,9 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
       for (int t = 0; t < n; ++t) qs[t * NL + l] = ul[k];
     }
   }
-  double irho = 0.0, lam = 0.0, mu = 0.0;
-  if constexpr (P::NCP) {
-    irho = 1.0 / A.mat[c * 3 + 0];
-    lam = A.mat[c * 3 + 1];
-    mu = A.mat[c * 3 + 2];
-  }
-  // point sources exist for the elastic system only (rejected at ader_set_point_source for the
-  // others): compiled out of the conservative systems' kernels
-  const bool has_src = P::NCP && (A.src.cell == c);
-  double ric[n];
-#pragma unroll
-  for (int t = 0; t < n; ++t) ric[t] = 0.0;
-  if (has_src) {
-#pragma unroll
-    for (int t = 0; t < n; ++t) {
-      const double tau = fma(T.x[t], dt, tn) - A.src.t0;
-      const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
-      ric[t] = (1.0 - 2.0 * a) * exp(-a);
-    }
-  }
   __syncthreads();
   if (A.cerk) {
-    cerk_guess_cell<P, D, N>(A, T, qs, Fs, sD, ul, irho, lam, mu, has_src, tid);
+    cerk_guess_cell<P, D, N>(A, T, qs, Fs, sD, ul, tid);
     __syncthreads();
   }
 
@@ -360,7 +271,7 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
     for (int k = 0; k < LPT; ++k)
 #pragma unroll
       for (int t = 0; t < n; ++t) R[k][t] = 0.0;
-    if constexpr (P::CONS) {
+    {
       double qn[C::NPT][NV];
       typename P::Aux ax[C::NPT];
       load_nodes<C, P>(qs, A.p, qn, ax, tid);
@@ -379,28 +290,9 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
         contract_lines<C, 2, n>(Fs, sD, -A.g.inv_h[2], R, tid);
       }
     }
-    if constexpr (P::NCP) {
-      contract_ncp_elastic<C, 0, n>(qs, sD, A.g.inv_h[0], irho, lam, mu, R, tid);
-      contract_ncp_elastic<C, 1, n>(qs, sD, A.g.inv_h[1], irho, lam, mu, R, tid);
-      contract_ncp_elastic<C, 2, n>(qs, sD, A.g.inv_h[2], irho, lam, mu, R, tid);
-    }
     if constexpr (P::NCPS) {
       ncp_swe_lines<C, 0>(qs, G, A.g.inv_h[0], A.p.grav, R, tid);
       ncp_swe_lines<C, 1>(qs, G, A.g.inv_h[1], A.p.grav, R, tid);
-    }
-    if (has_src) {
-#pragma unroll
-      for (int k = 0; k < LPT; ++k) {
-        const int l = tid + k * TPB;
-        if (l < NL) {
-          const int j = l / NV, v = l - (l / NV) * NV;
-          if (v >= 3) {
-            const double amp = -A.src.M[v - 3] * A.src.phi[j];
-#pragma unroll
-            for (int t = 0; t < n; ++t) R[k][t] = fma(amp, ric[t], R[k][t]);
-          }
-        }
-      }
     }
     __syncthreads();  // every read of qs of this iteration is done
 #pragma unroll
@@ -431,8 +323,8 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
     }
   }
   double* qbs;   // time-averaged q [NL] in smem
-  double* FBs;   // time-averaged fluxes [D][NL] in smem (conservative)
-  if constexpr (P::CONS) {
+  double* FBs;   // time-averaged fluxes [D][NL] in smem
+  {
     double FB[D][LPT];
     double qn[C::NPT][NV];
     typename P::Aux ax[C::NPT];
@@ -467,15 +359,6 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
         for (int d = 0; d < D; ++d) FBs[d * NL + l] = FB[d][k];
       }
     }
-  } else {
-    qbs = qs;
-    FBs = nullptr;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < LPT; ++k) {
-      const int l = tid + k * TPB;
-      if (l < NL) qbs[l] = qb[k];
-    }
   }
   __syncthreads();
 
@@ -492,7 +375,7 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
         const int st = (d == 0 ? 1 : (d == 1 ? n : n * n));
         const int jd = (j / st) % n;
         const int j0 = j - jd * st;
-        if constexpr (P::CONS) {
+        {
           double dF = 0.0, Fp = 0.0, Fm = 0.0;
 #pragma unroll
           for (int m = 0; m < n; ++m) {
@@ -503,15 +386,6 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
           }
           // -(1/h) D F + (1/h)(e1/w F+ - e0/w F-)
           vol += A.g.inv_h[d] * (-dF + sC[1][jd] * Fp - sC[0][jd] * Fm);
-        }
-        if constexpr (P::NCP) {
-          const int s = Elastic::src(d, v);
-          if (s >= 0) {
-            double dq = 0.0;
-#pragma unroll
-            for (int m = 0; m < n; ++m) dq = fma(sD[jd * n + m], qbs[(j0 + m * st) * NV + s], dq);
-            vol -= A.g.inv_h[d] * Elastic::coef_ir(d, v, irho, lam, mu) * dq;
-          }
         }
         if constexpr (P::NCPS) {
           // time average of the state-dependent product taken node by node (sum_t w_t g h_t
@@ -524,12 +398,6 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
             vol -= A.g.inv_h[d] * A.p.grav * nb;
           }
         }
-      }
-      if (has_src && v >= 3) {
-        double sbar = 0.0;
-#pragma unroll
-        for (int t = 0; t < n; ++t) sbar = fma(T.w[t], ric[t], sbar);
-        vol = fma(-A.src.M[v - 3] * A.src.phi[j], sbar, vol);
       }
       un[l] = fma(dt, vol, ul[k]);
     }
@@ -551,11 +419,11 @@ __device__ __forceinline__ void predictor_cell(const StepArgs& A, const Tables& 
     for (int m = 0; m < n; ++m) {
       const int jj = jbase + m * st;
       qf = fma(ev[m], qbs[jj * NV + v], qf);
-      if constexpr (P::CONS) ff = fma(ev[m], FBs[d * NL + jj * NV + v], ff);
+      ff = fma(ev[m], FBs[d * NL + jj * NV + v], ff);
     }
     double* rec = fc + (d * 2 + side) * FR;
     rec[jp * NV + v] = qf;
-    if constexpr (P::CONS) rec[NF * NV + jp * NV + v] = ff;
+    rec[NF * NV + jp * NV + v] = ff;
   }
 }
 
@@ -1237,6 +1105,7 @@ template <class P, int D>
 size_t FamilyImpl<P, D>::smem(int order, int prec) {
 #define ADER_SMEM_CASE(NN) \
   case NN: return prec == 1 ? CfgM<P, D, NN>::SMEM : Cfg<P, D, NN>::SMEM;
+  if constexpr (P::NCP) return 0;   // the elastic predictors fit at every order
   if constexpr (P::NCPS) prec = 0;  // FP64 only
   switch (order) {
     ADER_SMEM_CASE(1)
@@ -1253,12 +1122,16 @@ size_t FamilyImpl<P, D>::smem(int order, int prec) {
 template <class P, int D>
 cudaError_t FamilyImpl<P, D>::predictor(const StepArgs& a, const Tables& t, const TablesF& f,
                                         int prec, cudaStream_t s) {
-  if constexpr (!P::NCPS) {
-    if (prec == 1) {
-      ADER_DISPATCH_N(launch_predictor_mixed_n, a, t, f, s)
+  if constexpr (P::NCP) {  // set by the elastic family (kernels_ck.cuh)
+    return cudaErrorInvalidValue;
+  } else {
+    if constexpr (!P::NCPS) {
+      if (prec == 1) {
+        ADER_DISPATCH_N(launch_predictor_mixed_n, a, t, f, s)
+      }
     }
+    ADER_DISPATCH_N(launch_predictor_n, a, t, s)
   }
-  ADER_DISPATCH_N(launch_predictor_n, a, t, s)
 }
 
 }  // namespace ader

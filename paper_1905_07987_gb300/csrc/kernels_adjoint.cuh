@@ -18,6 +18,37 @@
 
 namespace ader {
 
+// Elastic: each row v of B_d has one non-zero coef(d,v) at column src(d,v); the NCP term
+// B_d dq/dx_d is contracted directly from q (no flux buffer).
+template <class C, int d, int RS>
+__device__ __forceinline__ void contract_ncp_elastic(const double* X, const double* Dm,
+                                                     double inv_h, double irho, double lam,
+                                                     double mu, double (&R)[C::LPT][C::n],
+                                                     int tid) {
+  constexpr int n = C::n, NV = C::NV, NL = C::NL, TPB = C::TPB, st = ipow(n, d);
+#pragma unroll
+  for (int k = 0; k < C::LPT; ++k) {
+    const int l = tid + k * TPB;
+    if (l < NL) {
+      const int j = l / NV, v = l - (l / NV) * NV;
+      const int s = Elastic::src(d, v);
+      if (s >= 0) {
+        const double coef = -Elastic::coef_ir(d, v, irho, lam, mu) * inv_h;
+        const int jd = digit<n, d>(j);
+        const int j0 = j - jd * st;
+        const double* Dr = Dm + jd * RS;
+#pragma unroll
+        for (int t = 0; t < n; ++t) {
+          double acc = 0.0;
+#pragma unroll
+          for (int m = 0; m < n; ++m) acc = fma(Dr[m], X[t * NL + (j0 + m * st) * NV + s], acc);
+          R[k][t] = fma(coef, acc, R[k][t]);
+        }
+      }
+    }
+  }
+}
+
 // Rows r of B_d whose single non-zero sits in column k (B_d^T has these entries in row k).
 struct RowsT {
   signed char r[3][9][3];

@@ -11,7 +11,23 @@
 // that of the Picard predictor: the volume term dt (L qbar + g sbar) goes into u_next and qbar
 // is extrapolated to the faces.
 //
-// Cost: N+1 applications of L per cell, against (N+1) iterations over n time nodes for Picard.
+// The Picard predictor of this linear system (PIC = true) runs in the same kernels: with the
+// constant or the Runge-Kutta guess every iterate at every time node is a polynomial of L applied
+// to u^n plus one applied to g, so its time average is
+//   qbar = sum_{k<=K} wk_k a_k + sum_{k<K} gam_k b_k,   a_0 = u,  b_0 = dt g,
+//   a_{k+1} = dt phi_k L a_k,  b_{k+1} = dt phi_k L b_k,
+// with K = iterations (+ 4 with the Runge-Kutta guess), the weights formed on the host by running
+// the iteration on the coefficients (build_linear_levels in api.cu), and gam_k a fixed combination of the
+// wavelet's samples.  The result is the Picard iteration's up to rounding, for K applications of
+// L to one time level in place of (iterations) x (n time levels) and the time solves.
+// Measured against the space-time iteration it replaces, two steps of 57 x 49 x 41 cells at order
+// 5, mixed: 96.7 -> 28.4 ms; 8 ensemble runs of sides 24 to 64 at order 4, mixed, two steps:
+// 203 -> 69.3 ms; an FP64 step at order 4, about 30 000 cells: 21.8 -> 4.7 ms.  The mixed form's
+// error against binary64 stays where it was (6.7e-12 and 6.8e-12 of the state): L qbar in
+// float-float and the first binary32 level with the tables' lo parts (without the two: 24.1 ms,
+// but 4.1e-11).
+//
+// Cost: N+1 applications of L per cell for the Taylor series, iterations + 1 for Picard.
 // One thread per spatial node (several cells per block at low order).  Along direction d the
 // thread forms the six derivatives that the eight non-zero rows of B_d read (the three
 // velocities and the stresses sigma_{0d}, sigma_{1d}, sigma_{2d}) and combines them:
@@ -49,6 +65,28 @@ struct CfgCK {
   // + the point source's spatial factor g [NS][6] of the source cell
   static constexpr size_t SMEM = ((size_t)CPB * 2 * REC + (size_t)NS * 6) * sizeof(double);
 };
+
+// Wavelet samples of the step: at the time nodes, then (for the Runge-Kutta guess) at the start,
+// the middle and the end.
+template <int N>
+__device__ __forceinline__ double ck_ricker(const StepArgs& A, const Tables& T, int m, double tn,
+                                            double dt) {
+  const double x = m <= N ? T.x[m <= N ? m : 0] : 0.5 * (m - N - 1);
+  const double tau = fma(x, dt, tn) - A.src.t0;
+  const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
+  return (1.0 - 2.0 * a) * exp(-a);
+}
+
+// gam_k of the Picard form's source levels from the samples s[n + 3].
+template <int N>
+__device__ __forceinline__ double lin_gamma(const StepArgs& A, const double* s, int k) {
+  constexpr int NSMP = N + 4;
+  const double* w = A.lin + 2 * A.nlev + 1 + (long long)k * NSMP;
+  double g = 0.0;
+#pragma unroll
+  for (int m = 0; m < NSMP; ++m) g = fma(w[m], s[m], g);
+  return g;
+}
 
 // R[v] += row v of -sum_d (1/h_d) B_d D_d X at node j of the cell record X ([NS][NVP]).
 // Dr[d][m] = D[j_d][m];  cf[d] = {1/(rho h_d), (lam + 2 mu)/h_d, lam/h_d, mu/h_d}.
@@ -100,8 +138,9 @@ __device__ __forceinline__ void ck_apply(const double* X, int j, const double (&
 }
 
 // The CPB cells from c0 of one context (one block); the kernel below and the ensemble's
-// persistent kernel call it.
-template <int N>
+// persistent kernel call it.  PIC: the Picard predictor's polynomial form (A.lin) instead of the
+// Taylor series.
+template <int N, bool PIC>
 __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tables& T,
                                                    long long c0) {
   using C = CfgCK<N>;
@@ -127,25 +166,28 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
 
   // point source of the block (at most one cell): Taylor coefficients s_k of the wavelet's
   // interpolant, its time average, and the spatial factor g of each node
-  __shared__ double s_sk[n], s_sbar;
+  // (the Picard form keeps the wavelet's samples)
+  __shared__ double s_sk[PIC ? n + 3 : n], s_sbar;
   __shared__ int s_slot;
   const long long sc = A.src.cell - c0;
   const bool srcb = sc >= 0 && sc < ncb;  // uniform over the block
   if (srcb && tid == 0) {
-    double ric[n], sbar = 0.0;
+    double ric[PIC ? n + 3 : n], sbar = 0.0;
 #pragma unroll
-    for (int t = 0; t < n; ++t) {
-      const double tau = fma(T.x[t], dt, tn) - A.src.t0;
-      const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
-      ric[t] = (1.0 - 2.0 * a) * exp(-a);
-      sbar = fma(T.w[t], ric[t], sbar);
-    }
+    for (int t = 0; t < (PIC ? n + 3 : n); ++t) ric[t] = ck_ricker<N>(A, T, t, tn, dt);
 #pragma unroll
-    for (int k = 0; k < n; ++k) {
-      double s = 0.0;
+    for (int t = 0; t < n; ++t) sbar = fma(T.w[t], ric[t], sbar);
+    if constexpr (PIC) {
 #pragma unroll
-      for (int t = 0; t < n; ++t) s = fma(T.Vi[k][t], ric[t], s);
-      s_sk[k] = s;
+      for (int t = 0; t < n + 3; ++t) s_sk[t] = ric[t];
+    } else {
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        double s = 0.0;
+#pragma unroll
+        for (int t = 0; t < n; ++t) s = fma(T.Vi[k][t], ric[t], s);
+        s_sk[k] = s;
+      }
     }
     s_sbar = sbar;
     s_slot = (int)sc;
@@ -183,22 +225,23 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
     for (int v = 0; v < NV; ++v) qb[v] = Xa[j * NVP + v];
   }
 
-  // Taylor coefficients a_1 .. a_N; qbar accumulates a_k / (k+1)
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    const double* Xc = (k & 1) ? Xb : Xa;
-    double* Xn = (k & 1) ? Xa : Xb;
+  // levels a_1 .. a_K; qbar accumulates them with their weights (Taylor: K = N, 1 / (k+1))
+  const int K = PIC ? A.nlev : N;
+  const double* Xc = Xa;
+  double* Xn = Xb;
+#pragma unroll(PIC ? 1 : N)
+  for (int k = 0; k < K; ++k) {
     if (act) {
       double R[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) R[v] = 0.0;
       ck_apply<N>(Xc, j, Dr, cf, R);
-      if (srcc) {
+      if (!PIC && srcc) {
 #pragma unroll
         for (int v = 3; v < NV; ++v) R[v] = fma(gsrc[j * 6 + v - 3], s_sk[k], R[v]);
       }
-      const double f = dt * (1.0 / (k + 1));
-      const double wk = 1.0 / (k + 2);
+      const double f = dt * (PIC ? A.lin[K + 1 + k] : 1.0 / (k + 1));
+      const double wk = PIC ? A.lin[k + 1] : 1.0 / (k + 2);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const double a = f * R[v];
@@ -207,15 +250,55 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
       }
     }
     __syncthreads();
+    double* x = const_cast<double*>(Xc);
+    Xc = Xn;
+    Xn = x;
   }
-  // qbar into the buffer that held a_{N-1} (last read before the final barrier)
-  double* Xq = ((N - 1) & 1) ? Xb : Xa;
-  double* Xo = ((N - 1) & 1) ? Xa : Xb;
+  if constexpr (PIC) {
+    // the source cell's own levels b_0 = dt g, b_1, .. (the block of the source cell alone)
+    if (srcb) {
+      if (srcc) {
+        const double gam = dt * lin_gamma<N>(A, s_sk, 0);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const double g = v >= 3 ? gsrc[j * 6 + (v >= 3 ? v - 3 : 0)] : 0.0;
+          qb[v] = fma(gam, g, qb[v]);
+          Xn[j * NVP + v] = dt * g;
+        }
+      }
+      __syncthreads();
+      for (int k = 1; k < K; ++k) {
+        double* x = const_cast<double*>(Xc);
+        Xc = Xn;
+        Xn = x;
+        if (srcc) {
+          double R[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) R[v] = 0.0;
+          ck_apply<N>(Xc, j, Dr, cf, R);
+          const double f = dt * A.lin[K + k];
+          const double gam = lin_gamma<N>(A, s_sk, k);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const double b = f * R[v];
+            qb[v] = fma(gam, b, qb[v]);
+            Xn[j * NVP + v] = b;
+          }
+        }
+        __syncthreads();
+      }
+    }
+  }
+  // qbar into the buffer of the level before the last (last read before the final barrier)
+  double* Xq = Xn;
+  double* Xo = const_cast<double*>(Xc);
   if (act) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) Xq[j * NVP + v] = qb[v];
   }
   __syncthreads();
+
+  const int oo = (int)(Xo - Xa);  // 0 or REC, the same for every cell of the block
 
   // volume term: u_next = u + dt (L qbar + g sbar), staged for a coalesced store (u from L2)
   if (act) {
@@ -233,7 +316,7 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
   __syncthreads();
   for (int e = tid; e < ncb * NL; e += TPB) {
     const int s = e / NL, r = e - s * NL;
-    const double* Xs = smem + (size_t)s * 2 * REC + (((N - 1) & 1) ? 0 : REC);
+    const double* Xs = smem + (size_t)s * 2 * REC + oo;
     A.u_next[c0 * NL + e] = fma(dt, Xs[(r / NV) * NVP + r % NV], A.u[c0 * NL + e]);
   }
 
@@ -242,7 +325,7 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
   for (int e = tid; e < ncb * NF * NV; e += TPB) {
     const int s = e / (NF * NV), r = e - s * (NF * NV);
     const int v = r % NV, jp = r / NV;
-    const double* Xs = smem + (size_t)s * 2 * REC + (((N - 1) & 1) ? REC : 0);
+    const double* Xs = smem + (size_t)s * 2 * REC + (REC - oo);
     double* fc = A.face + (c0 + s) * (3 * 2 * FR) + jp * NV + v;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -261,25 +344,25 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
   }
 }
 
-template <int N>
+template <int N, bool PIC>
 __global__ void __launch_bounds__(CfgCK<N>::TPB) k_predictor_ck(const __grid_constant__ StepArgs A,
                                                                const __grid_constant__ Tables T) {
-  predictor_ck_block<N>(A, T, (long long)blockIdx.x * CfgCK<N>::CPB);
+  predictor_ck_block<N, PIC>(A, T, (long long)blockIdx.x * CfgCK<N>::CPB);
 }
 
-template <int N>
+template <int N, bool PIC>
 cudaError_t launch_predictor_ck_n(const StepArgs& a, const Tables& t, cudaStream_t s) {
   using C = CfgCK<N>;
   static bool attr = false;
   if (!attr) {
     const cudaError_t e = cudaFuncSetAttribute(
-        k_predictor_ck<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+        k_predictor_ck<N, PIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_predictor_ck<N><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t);
+  k_predictor_ck<N, PIC><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t);
   return cudaGetLastError();
 }
 
@@ -353,8 +436,9 @@ __device__ __forceinline__ void ck_apply_ff(const float2* U, int j, const float2
   }
 }
 
-// Binary32 R[v] += row v of -sum_d (1/h_d) B_d D_d X at node j (X: [NS][NVF] floats).
-template <int N>
+// Binary32 R[v] += row v of -sum_d (1/h_d) B_d D_d X at node j (X: [NS][NVF] floats).  LO: the
+// derivative matrix and the coefficients with their lo parts (no rounding of fixed tables).
+template <int N, bool LO = false>
 __device__ __forceinline__ void ck_apply_f(const float* X, int j, const float2* D2,
                                            const ff (&cf)[3][4], float (&R)[9]) {
   constexpr int n = N + 1, NVF = CfgCKM<N>::NVF;
@@ -364,8 +448,8 @@ __device__ __forceinline__ void ck_apply_f(const float* X, int j, const float2* 
     const int jd = (j / st) % n;
     const float* b = X + (j - jd * st) * NVF;
     const float2* Dr = D2 + jd * n;
-    const int s0 = Elastic::sig(0, d), s1 = Elastic::sig(1, d), s2 = Elastic::sig(2, d);
-    float dv0 = 0.f, dv1 = 0.f, dv2 = 0.f, ds0 = 0.f, ds1 = 0.f, ds2 = 0.f;
+    const int sv[6] = {0, 1, 2, Elastic::sig(0, d), Elastic::sig(1, d), Elastic::sig(2, d)};
+    float g[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, lo[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int m = 0; m < n; ++m) {
       const float4* p = reinterpret_cast<const float4*>(b + m * st * NVF);
@@ -378,31 +462,36 @@ __device__ __forceinline__ void ck_apply_f(const float* X, int j, const float2* 
         r[4 * i + 2] = v.z;
         r[4 * i + 3] = v.w;
       }
-      const float c = Dr[m].x;
-      dv0 = fmaf(c, r[0], dv0);
-      dv1 = fmaf(c, r[1], dv1);
-      dv2 = fmaf(c, r[2], dv2);
-      ds0 = fmaf(c, r[s0], ds0);
-      ds1 = fmaf(c, r[s1], ds1);
-      ds2 = fmaf(c, r[s2], ds2);
-    }
-    const float dv[3] = {dv0, dv1, dv2};
-    R[0] = fmaf(cf[d][0].h, ds0, R[0]);
-    R[1] = fmaf(cf[d][0].h, ds1, R[1]);
-    R[2] = fmaf(cf[d][0].h, ds2, R[2]);
+      const float2 c = Dr[m];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) R[3 + i] = fmaf(i == d ? cf[d][1].h : cf[d][2].h, dv[d], R[3 + i]);
+      for (int i = 0; i < 6; ++i) {
+        g[i] = fmaf(c.x, r[sv[i]], g[i]);
+        if (LO) lo[i] = fmaf(c.y, r[sv[i]], lo[i]);
+      }
+    }
+    const auto add = [&](int v, const ff& k, int i) {  // R[v] += k g_i
+      if (LO) {
+        const float x = g[i] + lo[i];
+        R[v] = fmaf(k.h, x, fmaf(k.l, x, R[v]));
+      } else {
+        R[v] = fmaf(k.h, g[i], R[v]);
+      }
+    };
+#pragma unroll
+    for (int i = 0; i < 3; ++i) add(i, cf[d][0], 3 + i);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) add(3 + i, i == d ? cf[d][1] : cf[d][2], d);
 #pragma unroll
     for (int v = 6; v < 9; ++v) {
       const int s = Elastic::src(d, v);
-      if (s >= 0) R[v] = fmaf(cf[d][3].h, dv[s], R[v]);
+      if (s >= 0) add(v, cf[d][3], s);
     }
   }
 }
 
 // The CPB cells from c0 of one context (one block), mixed precision; the kernel below and the
 // ensemble's persistent kernel call it.
-template <int N>
+template <int N, bool PIC>
 __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, const Tables& T,
                                                          const TablesF& F, long long c0) {
   using C = CfgCKM<N>;
@@ -447,25 +536,28 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
     }
   }
   // point source of the block, as in the FP64 kernel, kept in float-float for the per-node terms
-  __shared__ ff s_skf[n], s_sbarf;
+  __shared__ ff s_skf[PIC ? 1 : n], s_sbarf;
+  __shared__ double s_smp[PIC ? n + 3 : 1];
   __shared__ int s_slot;
   const long long sc = A.src.cell - c0;
   const bool srcb = sc >= 0 && sc < ncb;
   if (srcb && tid == 0) {
-    double ric[n], sbar = 0.0;
+    double ric[PIC ? n + 3 : n], sbar = 0.0;
 #pragma unroll
-    for (int t = 0; t < n; ++t) {
-      const double tau = fma(T.x[t], dt, tn) - A.src.t0;
-      const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
-      ric[t] = (1.0 - 2.0 * a) * exp(-a);
-      sbar = fma(T.w[t], ric[t], sbar);
-    }
+    for (int t = 0; t < (PIC ? n + 3 : n); ++t) ric[t] = ck_ricker<N>(A, T, t, tn, dt);
 #pragma unroll
-    for (int k = 0; k < n; ++k) {
-      double s = 0.0;
+    for (int t = 0; t < n; ++t) sbar = fma(T.w[t], ric[t], sbar);
+    if constexpr (PIC) {
 #pragma unroll
-      for (int t = 0; t < n; ++t) s = fma(T.Vi[k][t], ric[t], s);
-      s_skf[k] = ff_split(s);
+      for (int t = 0; t < n + 3; ++t) s_smp[t] = ric[t];
+    } else {
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        double s = 0.0;
+#pragma unroll
+        for (int t = 0; t < n; ++t) s = fma(T.Vi[k][t], ric[t], s);
+        s_skf[k] = ff_split(s);
+      }
     }
     s_sbarf = ff_split(sbar);
     s_slot = (int)sc;
@@ -487,6 +579,7 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
   ff cf[3][4];
   ff LU[NV], dbar[NV];
   const ff dtf = ff_split_int(dt);
+  const int K = PIC ? A.nlev : N;
   if (act) {
 #pragma unroll
     for (int d = 0; d < 3; ++d)
@@ -499,36 +592,39 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       ff t0 = LU[v];
-      if (srcc && v >= 3) {
+      if (!PIC && srcc && v >= 3) {
         const float2 g = gsrc[j * 6 + v - 3];
         t0 = ff_add(t0, ff_mul({g.x, g.y}, s_skf[0]));
       }
       const ff a1 = ff_mul(dtf, t0);
+      // both forms weight the first level with the mean of tau, 1/2, but for rounding (one Picard
+      // iteration or more; phi_0 = 1)
       dbar[v] = {0.5f * a1.h, 0.5f * a1.l};
       XA[j * NVF + v] = a1.h;
     }
   }
   __syncthreads();
 
-  // a_2 .. a_N in binary32; their share of dbar, sum_k a_k / (k+1), in binary32
+  // a_2 .. a_K in binary32; their share of dbar, sum_k a_k / (k+1), in binary32
   float d32[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) d32[v] = 0.f;
-#pragma unroll
-  for (int k = 1; k < N; ++k) {
-    const float* Xc = (k & 1) ? XA : XB;
-    float* Xn = (k & 1) ? XB : XA;
+  float *Xc = XA, *Xn = XB;
+#pragma unroll(PIC ? 1 : N)
+  for (int k = 1; k < K; ++k) {
     if (act) {
       float R[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) R[v] = 0.f;
-      ck_apply_f<N>(Xc, j, s_D, cf, R);
-      if (srcc) {
+      // the largest binary32 level of the Picard form without the tables' rounding
+      if (PIC && k == 1) ck_apply_f<N, true>(Xc, j, s_D, cf, R);
+      else ck_apply_f<N>(Xc, j, s_D, cf, R);
+      if (!PIC && srcc) {
 #pragma unroll
-        for (int v = 3; v < NV; ++v) R[v] = fmaf(gsrc[j * 6 + v - 3].x, s_skf[k].h, R[v]);
+        for (int v = 3; v < NV; ++v) R[v] = fmaf(gsrc[j * 6 + v - 3].x, s_skf[PIC ? 0 : k].h, R[v]);
       }
-      const float f = dtf.h * (1.0f / (k + 1));
-      const float wk = 1.0f / (k + 2);
+      const float f = dtf.h * (PIC ? (float)A.lin[K + 1 + k] : 1.0f / (k + 1));
+      const float wk = PIC ? (float)A.lin[k + 1] : 1.0f / (k + 2);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const float a = f * R[v];
@@ -537,10 +633,52 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
       }
     }
     __syncthreads();
+    float* x = Xc;
+    Xc = Xn;
+    Xn = x;
+  }
+  if constexpr (PIC) {
+    // the source cell's own levels: b_0 = dt g in float-float, b_1, .. in binary32
+    if (srcb) {
+      if (srcc) {
+        const ff gam = ff_split(dt * lin_gamma<N>(A, s_smp, 0));
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          float2 g = make_float2(0.f, 0.f);
+          if (v >= 3) {
+            g = gsrc[j * 6 + (v >= 3 ? v - 3 : 0)];
+            dbar[v] = ff_add(dbar[v], ff_mul({g.x, g.y}, gam));
+          }
+          Xn[j * NVF + v] = dtf.h * g.x;
+        }
+      }
+      __syncthreads();
+      for (int k = 1; k < K; ++k) {
+        float* x = Xc;
+        Xc = Xn;
+        Xn = x;
+        if (srcc) {
+          float R[NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) R[v] = 0.f;
+          ck_apply_f<N>(Xc, j, s_D, cf, R);
+          const float f = dtf.h * (float)A.lin[K + k];
+          const float gam = (float)lin_gamma<N>(A, s_smp, k);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const float b = f * R[v];
+            d32[v] = fmaf(gam, b, d32[v]);
+            Xn[j * NVF + v] = b;
+          }
+        }
+        __syncthreads();
+      }
+    }
   }
 
   // qbar = u + dbar (float-float, in place: after the base term only the owner reads its node);
-  // dbar's hi part into A for the binary32 L dbar
+  // dbar's hi part into A for the binary32 L dbar of the Taylor form; the Picard form takes
+  // L qbar in float-float, as its iteration's volume term is formed
   if (act) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -548,19 +686,26 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
       const float2 uu = U[j * NVQ + v];
       const ff q = ff_add({uu.x, uu.y}, dbar[v]);
       U[j * NVQ + v] = make_float2(q.h, q.l);
-      XA[j * NVF + v] = dbar[v].h;
+      if (!PIC) XA[j * NVF + v] = dbar[v].h;
     }
   }
   __syncthreads();
   ff vol[NV];
   if (act) {
-    float R[NV];
+    if constexpr (PIC) {  // L qbar in float-float
 #pragma unroll
-    for (int v = 0; v < NV; ++v) R[v] = 0.f;
-    ck_apply_f<N>(XA, j, s_D, cf, R);
+      for (int v = 0; v < NV; ++v) vol[v] = {0.f, 0.f};
+      ck_apply_ff<N>(U, j, s_D, cf, vol);
+    } else {
+      float R[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) R[v] = 0.f;
+      ck_apply_f<N>(XA, j, s_D, cf, R);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) vol[v] = ff_add(LU[v], {R[v], 0.f});
+    }
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      vol[v] = ff_add(LU[v], {R[v], 0.f});
       if (srcc && v >= 3) {
         const float2 g = gsrc[j * 6 + v - 3];
         vol[v] = ff_add(vol[v], ff_mul({g.x, g.y}, s_sbarf));
@@ -606,27 +751,27 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
   }
 }
 
-template <int N>
+template <int N, bool PIC>
 __global__ void __launch_bounds__(CfgCKM<N>::TPB, CfgCKM<N>::MINB)
     k_predictor_ck_mixed(const __grid_constant__ StepArgs A, const __grid_constant__ Tables T,
                          const __grid_constant__ TablesF F) {
-  predictor_ck_mixed_block<N>(A, T, F, (long long)blockIdx.x * CfgCKM<N>::CPB);
+  predictor_ck_mixed_block<N, PIC>(A, T, F, (long long)blockIdx.x * CfgCKM<N>::CPB);
 }
 
-template <int N>
+template <int N, bool PIC>
 cudaError_t launch_predictor_ck_mixed_n(const StepArgs& a, const Tables& t, const TablesF& f,
                                         cudaStream_t s) {
   using C = CfgCKM<N>;
   static bool attr = false;
   if (!attr) {
     const cudaError_t e = cudaFuncSetAttribute(
-        k_predictor_ck_mixed<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+        k_predictor_ck_mixed<N, PIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
   if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_predictor_ck_mixed<N><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t, f);
+  k_predictor_ck_mixed<N, PIC><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t, f);
   return cudaGetLastError();
 }
 

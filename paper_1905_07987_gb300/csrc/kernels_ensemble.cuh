@@ -1,5 +1,5 @@
-// Ensembles of uneven grids advanced together: one persistent launch per phase of the step for all
-// runs.  The work of the runs is concatenated (cells for the predictor and the corrector, faces of
+// Ensembles of uneven elastic grids advanced together: one persistent launch per phase of the step for
+// all runs.  The work of the runs is concatenated (the predictor's blocks of cells, the corrector's cells, faces of
 // one direction for the Riemann solver); each work item finds its run by binary search in the
 // prefix offsets of the run table and is processed by the same device function as in the
 // per-context kernels, with that run's step arguments (from device memory).  Blocks and warps
@@ -7,6 +7,7 @@
 // large ones inside one launch.  No block waits for another.
 #pragma once
 #include "kernels.cuh"
+#include "kernels_ck.cuh"
 #include "step_scalars.cuh"
 
 namespace ader {
@@ -22,24 +23,34 @@ __device__ __forceinline__ int ens_find(const long long* off, int nr, long long 
   return lo;
 }
 
-template <class P, int D, int N, bool MIXED>
+template <int N, bool MIXED>
 struct EnsCfg {
-  static constexpr int TPB = MIXED ? CfgM<P, D, N>::TPB : Cfg<P, D, N>::TPB;
-  static constexpr int MINB = MIXED ? CfgM<P, D, N>::MINB : 1;
-  static constexpr size_t SMEM = MIXED ? CfgM<P, D, N>::SMEM : Cfg<P, D, N>::SMEM;
+  static constexpr int TPB = MIXED ? CfgCKM<N>::TPB : CfgCK<N>::TPB;
+  static constexpr int MINB = MIXED ? CfgCKM<N>::MINB : 1;
+  static constexpr int CPB = MIXED ? CfgCKM<N>::CPB : CfgCK<N>::CPB;
+  static constexpr size_t SMEM = MIXED ? CfgCKM<N>::SMEM : CfgCK<N>::SMEM;
+  static_assert(CPB == ck_cells_per_block(N), "the host counts the blocks of each run");
 };
 
-template <class P, int D, int N, bool MIXED>
-__global__ void __launch_bounds__(EnsCfg<P, D, N, MIXED>::TPB, EnsCfg<P, D, N, MIXED>::MINB)
+// The it-th predictor block of all runs (PIC: Picard predictor, otherwise Cauchy-Kowalevski).
+template <int N, bool MIXED, bool PIC>
+__device__ __forceinline__ void ens_predictor_block(const StepArgs* R, const EnsTable& E,
+                                                    const Tables& T, const TablesF& F,
+                                                    long long it) {
+  const int r = ens_find(E.blk0, E.nr, it);
+  const long long c0 = (it - E.blk0[r]) * EnsCfg<N, MIXED>::CPB;
+  if constexpr (MIXED) predictor_ck_mixed_block<N, PIC>(R[r], T, F, c0);
+  else predictor_ck_block<N, PIC>(R[r], T, c0);
+  __syncthreads();  // the next block of cells reuses the shared memory
+}
+
+template <int N, bool MIXED, bool PIC>
+__global__ void __launch_bounds__(EnsCfg<N, MIXED>::TPB, EnsCfg<N, MIXED>::MINB)
     k_ens_predictor(const StepArgs* __restrict__ R, const __grid_constant__ EnsTable E,
                     const __grid_constant__ Tables T, const __grid_constant__ TablesF F) {
-  const long long total = E.cell0[E.nr];
-  for (long long it = blockIdx.x; it < total; it += gridDim.x) {
-    const int r = ens_find(E.cell0, E.nr, it);
-    if constexpr (MIXED) predictor_mixed_cell<P, D, N>(R[r], T, F, it - E.cell0[r]);
-    else predictor_cell<P, D, N>(R[r], T, it - E.cell0[r]);
-    __syncthreads();  // the next cell reuses the shared memory
-  }
+  const long long total = E.blk0[E.nr];
+  for (long long it = blockIdx.x; it < total; it += gridDim.x)
+    ens_predictor_block<N, MIXED, PIC>(R, E, T, F, it);
 }
 
 template <class P, int D, int N>
@@ -74,28 +85,30 @@ __global__ void __launch_bounds__(256) k_ens_corrector(const StepArgs* __restric
   }
 }
 
-// One step of every run: dt, predictor, Riemann per direction, corrector, time advance.
-template <class P, int D, int N, bool MIXED>
+// One step of every run: dt, predictor (`blocks` of them), Riemann per direction, corrector, time
+// advance.
+template <int N, bool MIXED, bool PIC>
 cudaError_t ens_step_n(const StepArgs* R, const EnsTable& E, const Tables& T, const TablesF& F,
-                       cudaStream_t s) {
-  using G = EnsCfg<P, D, N, MIXED>;
+                       long long blocks, cudaStream_t s) {
+  using G = EnsCfg<N, MIXED>;
   static bool attr = false;
   if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_ens_predictor<P, D, N, MIXED>,
+    const cudaError_t e = cudaFuncSetAttribute(k_ens_predictor<N, MIXED, PIC>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)G::SMEM);
     if (e != cudaSuccess) return e;
     attr = true;
   }
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
   cudaError_t e = launch_ens_dt(R, E.nr, s);
   if (e != cudaSuccess) return e;
-  k_ens_predictor<P, D, N, MIXED><<<E.pblocks, G::TPB, G::SMEM, s>>>(R, E, T, F);
+  k_ens_predictor<N, MIXED, PIC><<<(unsigned)blocks, G::TPB, G::SMEM, s>>>(R, E, T, F);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  for (int d = 0; d < D; ++d) {
-    k_ens_riemann<P, D, N><<<152 * 16, 128, 0, s>>>(R, E, T, d);
+  for (int d = 0; d < 3; ++d) {
+    k_ens_riemann<Elastic, 3, N><<<152 * 16, 128, 0, s>>>(R, E, T, d);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_ens_corrector<P, D, N><<<152 * 8, 256, 0, s>>>(R, E);
+  k_ens_corrector<Elastic, 3, N><<<152 * 8, 256, 0, s>>>(R, E);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_ens_advance(R, E.nr, s);
 }
@@ -145,13 +158,15 @@ __device__ __forceinline__ bool grid_sync(GridBar* b, unsigned nblocks, long lon
 // over the concatenated cells, the Riemann solver over the concatenated faces of all directions,
 // the corrector over the concatenated degrees of freedom and the time advance, separated by
 // grid-wide barriers.  Rsteps: the runs' step arguments of each step ([steps][nr]).
-template <class P, int D, int N, bool MIXED>
-__global__ void __launch_bounds__(EnsCfg<P, D, N, MIXED>::TPB, EnsCfg<P, D, N, MIXED>::MINB)
+template <int N, bool MIXED>
+__global__ void __launch_bounds__(EnsCfg<N, MIXED>::TPB, EnsCfg<N, MIXED>::MINB)
     k_ens_fused(const StepArgs* __restrict__ Rsteps, const __grid_constant__ EnsTable E,
                 const __grid_constant__ Tables T, const __grid_constant__ TablesF F, int steps,
                 GridBar* bar, long long limit) {
+  using P = Elastic;
+  constexpr int D = 3;
   using C = Cfg<P, D, N>;
-  constexpr int n = N + 1, NL = C::NL, TPB = EnsCfg<P, D, N, MIXED>::TPB;
+  constexpr int n = N + 1, NL = C::NL, TPB = EnsCfg<N, MIXED>::TPB;
   extern __shared__ __align__(16) double fsm[];
   const unsigned nb = gridDim.x;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -161,12 +176,8 @@ __global__ void __launch_bounds__(EnsCfg<P, D, N, MIXED>::TPB, EnsCfg<P, D, N, M
     const StepArgs* R = Rsteps + (long long)s * E.nr;
     if (blockIdx.x == 0 && (int)threadIdx.x < E.nr) dt_finalize_one(R[threadIdx.x]);
     if (!(ok = grid_sync(bar, nb, limit))) break;
-    for (long long it = blockIdx.x; it < ncell; it += nb) {
-      const int r = ens_find(E.cell0, E.nr, it);
-      if constexpr (MIXED) predictor_mixed_cell<P, D, N>(R[r], T, F, it - E.cell0[r]);
-      else predictor_cell<P, D, N>(R[r], T, it - E.cell0[r]);
-      __syncthreads();  // the next cell reuses the shared memory
-    }
+    for (long long it = blockIdx.x; it < E.blk0[E.nr]; it += nb)
+      ens_predictor_block<N, MIXED, true>(R, E, T, F, it);
     if (!(ok = grid_sync(bar, nb, limit))) break;
     {
       const long long nf0 = E.face0[0][E.nr], nf1 = E.face0[1][E.nr];
@@ -203,20 +214,20 @@ __global__ void __launch_bounds__(EnsCfg<P, D, N, MIXED>::TPB, EnsCfg<P, D, N, M
 }
 
 // Launch `steps` steps of every run as one cooperative kernel (after zeroing the barrier).
-template <class P, int D, int N, bool MIXED>
+template <int N, bool MIXED>
 cudaError_t ens_fused_n(const StepArgs* R, const EnsTable& E, const Tables& T, const TablesF& F,
                         int steps, GridBar* bar, long long limit, int blocks_per_sm,
                         cudaStream_t s) {
-  using G = EnsCfg<P, D, N, MIXED>;
+  using G = EnsCfg<N, MIXED>;
   constexpr size_t SW = (size_t)ENS_MAXR * 2 * 3 * (N + 1) * sizeof(double);
   constexpr size_t SMEM = G::SMEM > SW ? G::SMEM : SW;
   static int max_bps = 0;
   if (!max_bps) {
-    cudaError_t e = cudaFuncSetAttribute(k_ens_fused<P, D, N, MIXED>,
+    cudaError_t e = cudaFuncSetAttribute(k_ens_fused<N, MIXED>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
     if (e != cudaSuccess) return e;
     int nbk = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbk, k_ens_fused<P, D, N, MIXED>, G::TPB, SMEM);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbk, k_ens_fused<N, MIXED>, G::TPB, SMEM);
     if (e != cudaSuccess) return e;
     max_bps = nbk < 1 ? 1 : nbk;
   }
@@ -236,7 +247,7 @@ cudaError_t ens_fused_n(const StepArgs* R, const EnsTable& E, const Tables& T, c
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_ens_fused<P, D, N, MIXED>, R, E, T, F, steps, bar, limit);
+  return cudaLaunchKernelEx(&cfg, k_ens_fused<N, MIXED>, R, E, T, F, steps, bar, limit);
 }
 
 }  // namespace ader

@@ -37,8 +37,8 @@ struct CfgM {
   // NL / LPD threads per block (about LPD lines per thread), rounded up to 64 threads for Euler
   // and to whole warps otherwise, from sweeps on GB300 (LPD in {2, 3, 4, 6, 8}; 128 to 320
   // threads at orders 3 and 4): Euler 128 threads at order 3 (NL / 3), 320 at order 4 (NL / 2,
-  // 96 registers, 20 warps per SM); elastic NL / 6 at order 4, NL / 8 at order 5.
-  static constexpr int LPD = EULER ? (N == 4 ? 2 : 3) : (N >= 5 ? 8 : 6);
+  // 96 registers, 20 warps per SM).
+  static constexpr int LPD = EULER ? (N == 4 ? 2 : 3) : 6;
   static constexpr int RND = EULER ? 64 : 32;
   static constexpr int TPB_E = ((NL + LPD - 1) / LPD + RND - 1) / RND * RND;
   static constexpr int TPB = TPB_E < 64 ? 64 : (TPB_E > 512 ? 512 : TPB_E);
@@ -49,12 +49,12 @@ struct CfgM {
   // v0[D], p0 (float-float) per spatial node; rows padded to an odd number of float-float values
   // so that the 8-byte loads of consecutive nodes fall on distinct banks
   static constexpr int BW = EULER ? ((D + 1) % 2 ? D + 1 : D + 2) : 1;
-  static constexpr size_t B_FB0 = P::CONS ? (size_t)D * NL * sizeof(ff) : 0;
+  static constexpr size_t B_FB0 = (size_t)D * NL * sizeof(ff);
   static constexpr size_t B_UFF = (size_t)NL * sizeof(ff);
   static constexpr size_t B_BF = EULER ? (size_t)NS * BW * sizeof(ff) : 0;
   // rounded up to 16 bytes: the region behind it is also read as doubles
   static constexpr size_t B_DQ = ((size_t)n * NL * sizeof(float) + 15) / 16 * 16;
-  static constexpr size_t B_F3 = P::CONS ? (size_t)D * n * NL * sizeof(float) : 0;
+  static constexpr size_t B_F3 = (size_t)D * n * NL * sizeof(float);
   static constexpr size_t SMEM = B_FB0 + B_UFF + B_BF + B_DQ + B_F3;
 };
 
@@ -232,12 +232,12 @@ __device__ __forceinline__ void linear_nodes(const float* qbh, const float* qbl,
   }
 }
 
-// R[k][t] += cf[d][v] * sum_m D[j_d][m] X[t][(j, j_d -> m)][src]  in binary32 (D as n x n rows
+// R[k][t] += cf[d][v] * sum_m D[j_d][m] X[t][(j, j_d -> m)][v]  in binary32 (D as n x n rows
 // in shared memory, hi parts alone and as (hi, lo) pairs: the row index differs between the lanes
-// of a warp), with the per-cell
-// coefficients cf = {hi[3][NV], lo[3][NV]} in shared memory; with LO the lo parts of the
+// of a warp), with the
+// coefficients cf = {hi[3][NV], lo[3][NV]} (-1/h_d) in shared memory; with LO the lo parts of the
 // coefficient and of the float-float derivative matrix are added (no rounding of fixed tables).
-template <class M, int d, bool NCP, bool LO = false>
+template <class M, int d, bool LO = false>
 __device__ __forceinline__ void contract_f(const float* X, const float* Dh, const float2* D2,
                                            const float* cf, float (&R)[M::LPT][M::n], int tid) {
   constexpr int n = M::n, NV = M::NV, NL = M::NL, TPB = M::TPB, st = ipow(n, d);
@@ -246,11 +246,6 @@ __device__ __forceinline__ void contract_f(const float* X, const float* Dh, cons
     const int l = tid + k * TPB;
     if (l < NL) {
       const int j = l / NV, v = l - (l / NV) * NV;
-      int s = v;
-      if constexpr (NCP) {
-        s = Elastic::src(d, v);
-        if (s < 0) continue;
-      }
       const float c = cf[d * NV + v], clo = cf[3 * NV + d * NV + v];
       const int jd = digit<n, d>(j);
       const int j0 = j - jd * st;
@@ -259,7 +254,7 @@ __device__ __forceinline__ void contract_f(const float* X, const float* Dh, cons
         float acc = 0.f, lo = 0.f;
 #pragma unroll
         for (int m = 0; m < n; ++m) {
-          const float x = X[t * NL + (j0 + m * st) * NV + s];
+          const float x = X[t * NL + (j0 + m * st) * NV + v];
           if constexpr (LO) {
             const float2 dm = D2[jd * n + m];
             acc = fmaf(dm.x, x, acc);
@@ -304,8 +299,8 @@ __device__ __forceinline__ void dflux_level(const float* sq, const ff* uff, cons
   }
 }
 
-// One time level of contract_f: r[k] += cf[d][v] * sum_m D[j_d][m] X[(j, j_d -> m)][src] (binary32).
-template <class M, int d, bool NCP>
+// One time level of contract_f: r[k] += cf[d][v] * sum_m D[j_d][m] X[(j, j_d -> m)][v] (binary32).
+template <class M, int d>
 __device__ __forceinline__ void contract_level(const float* X, const float* Dh, const float* cf,
                                                float (&r)[M::LPT], int tid) {
   constexpr int n = M::n, NV = M::NV, NL = M::NL, TPB = M::TPB, st = ipow(n, d);
@@ -314,23 +309,17 @@ __device__ __forceinline__ void contract_level(const float* X, const float* Dh, 
     const int l = tid + k * TPB;
     if (l < NL) {
       const int j = l / NV, v = l - (l / NV) * NV;
-      int s = v;
-      if constexpr (NCP) {
-        s = Elastic::src(d, v);
-        if (s < 0) continue;
-      }
       const int jd = digit<n, d>(j);
       const int j0 = j - jd * st;
       float acc = 0.f;
 #pragma unroll
-      for (int m = 0; m < n; ++m) acc = fmaf(Dh[jd * n + m], X[(j0 + m * st) * NV + s], acc);
+      for (int m = 0; m < n; ++m) acc = fmaf(Dh[jd * n + m], X[(j0 + m * st) * NV + v], acc);
       r[k] = fmaf(cf[d * NV + v], acc, r[k]);
     }
   }
 }
 
-// One cell c (all threads of the block; called by the per-context kernel and by the persistent
-// ensemble kernel).
+// One cell c (all threads of the block).
 template <class P, int D, int N>
 __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Tables& T,
                                                      const TablesF& F, long long c) {
@@ -351,18 +340,10 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
   const double dt = A.dev->dt;
   const float dtf = (float)dt;
   const ff dtff = {dtf, (float)(dt - (double)dtf)};
-  const double tn = A.dev->t;
   const double* u = A.u + c * NL;
   const ff g1 = {F.g1h, F.g1l};
 
-  double irho = 0.0, lam = 0.0, mu = 0.0;
-  if constexpr (P::NCP) {
-    irho = 1.0 / A.mat[c * 3 + 0];
-    lam = A.mat[c * 3 + 1];
-    mu = A.mat[c * 3 + 2];
-  }
-  // per-cell contraction coefficients: -1/h_d, or -coef(d,v)/h_d for the rows of B_d, as
-  // (hi, lo) binary32 pairs
+  // contraction coefficients -1/h_d as (hi, lo) binary32 pairs
   __shared__ float cf[2 * 3 * NV];
   // tables indexed by a per-lane row (j_d, face side) staged in shared memory
   // (hi, lo) pairs interleaved: one 8-byte load per entry in the float-float contractions
@@ -381,28 +362,12 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
     sE[3][tid] = F.e1l[tid];
   }
   if (tid < 3 * NV) {
-    const int d = tid / NV, v = tid % NV;
-    double cd = d < D ? -A.g.inv_h[d] : 0.0;
-    if constexpr (P::NCP) cd = -Elastic::coef_ir(d, v, irho, lam, mu) * A.g.inv_h[d];
+    const int d = tid / NV;
+    const double cd = d < D ? -A.g.inv_h[d] : 0.0;
     const float h = (float)cd;
     cf[tid] = h;
     cf[3 * NV + tid] = (float)(cd - (double)h);
   }
-  // point sources exist for the elastic system only (rejected at ader_set_point_source for the
-  // others): compiled out of the conservative systems' kernels
-  const bool has_src = P::NCP && (A.src.cell == c);
-  double ric[n];
-#pragma unroll
-  for (int t = 0; t < n; ++t) ric[t] = 0.0;
-  if (has_src) {
-#pragma unroll
-    for (int t = 0; t < n; ++t) {
-      const double tau = fma(T.x[t], dt, tn) - A.src.t0;
-      const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
-      ric[t] = (1.0 - 2.0 * a) * exp(-a);
-    }
-  }
-
   // ---- phase 0: base terms at the spatial nodes (FP64 -> float-float) --------------------
   double ul[LPT];
 #pragma unroll
@@ -415,7 +380,7 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
     }
   }
   __syncthreads();  // uff complete
-  if constexpr (P::CONS) {
+  {
     // flux of u^n at the spatial nodes in float-float (scaled by 1/h_d): 1/rho, v, p, F_d
 #pragma unroll
     for (int k = 0; k < M::NPS; ++k) {
@@ -463,8 +428,7 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
   }
   __syncthreads();
 
-  // B0 = R(u^n) in float-float (hi, lo): flux divergence (conservative form) or the
-  // non-conservative product (elastic); the elastic volume term reuses it.
+  // B0 = R(u^n) in float-float (hi, lo): the flux divergence.
   float b0f[LPT], b0l[LPT];
 #pragma unroll
   for (int k = 0; k < LPT; ++k) {
@@ -479,62 +443,34 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
         const int st = (d == 0 ? 1 : (d == 1 ? n : n * n));
         const int jd = (j / st) % n;
         const int j0 = j - jd * st;
-        if constexpr (P::CONS) {
 #pragma unroll
-          for (int m = 0; m < n; ++m) {
-            const ff f = FB0[d * NL + (j0 + m * st) * NV + v];
-            const float2 dm = sD2[jd * n + m];
-            ff_mac(aS, dm.x, dm.y, f.h, f.l);
-          }
-        } else {
-          const int s = Elastic::src(d, v);
-          if (s >= 0) {
-            ff g = {0.f, 0.f};
-#pragma unroll
-            for (int m = 0; m < n; ++m) {
-              const ff f = uff[(j0 + m * st) * NV + s];
-              const float2 dm = sD2[jd * n + m];
-              ff_mac(g, dm.x, dm.y, f.h, f.l);
-            }
-            aS = ff_add(aS, ff_mul(ff_norm(g.h, g.l), {cf[d * NV + v], cf[3 * NV + d * NV + v]}));
-          }
+        for (int m = 0; m < n; ++m) {
+          const ff f = FB0[d * NL + (j0 + m * st) * NV + v];
+          const float2 dm = sD2[jd * n + m];
+          ff_mac(aS, dm.x, dm.y, f.h, f.l);
         }
       }
-      // B0 renormalised, without a round trip through FP64 (conservative form: -aS)
+      // B0 = -aS renormalised, without a round trip through FP64
       const ff b = ff_norm(aS.h, aS.l);
-      b0f[k] = P::CONS ? -b.h : b.h;
-      b0l[k] = P::CONS ? -b.l : b.l;
+      b0f[k] = -b.h;
+      b0l[k] = -b.l;
     }
   }
 
   // ---- continuous extension Runge-Kutta guess (Sec. 5), A.cerk: dq^0 at the time nodes -------
   // Classical four-stage Runge-Kutta on the cell-local ODE dq/dt = R(u + dq) with the stages
-  // k_i = B0 + dR(s_i) (+ the point source at the stage time), s = 0, h/2 k_1, h/2 k_2, h k_3,
+  // k_i = B0 + dR(s_i), s = 0, h/2 k_1, h/2 k_2, h k_3,
   // and its natural continuous extension dq(x_t) = h sum_i b_i(x_t) k_i (sum_i b_i = x_t): the
   // stage increments and dR in binary32 (they are O(dt)), B0 from its float-float hi part.
   if (A.cerk) {
     float kd[3][LPT];   // dR of the stages 2, 3, 4
-    double rs[4] = {0.0, 0.0, 0.0, 0.0};  // wavelet at the stage times (source cell)
-    if (has_src) {
-      const double ts[4] = {0.0, 0.5, 0.5, 1.0};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const double tau = fma(ts[i], dt, tn) - A.src.t0;
-        const double a = (M_PI * A.src.f0 * tau) * (M_PI * A.src.f0 * tau);
-        rs[i] = (1.0 - 2.0 * a) * exp(-a);
-      }
-    }
 #pragma unroll
     for (int st = 0; st < 3; ++st) {
 #pragma unroll
       for (int k = 0; k < LPT; ++k) {
         const int l = tid + k * TPB;
         if (l < NL) {
-          float kp = b0f[k] + (st > 0 ? kd[st - 1][k] : 0.f);
-          if (has_src) {
-            const int j = l / NV, v = l - (l / NV) * NV;
-            if (v >= 3) kp = fmaf((float)(-A.src.M[v - 3] * A.src.phi[j]), (float)rs[st], kp);
-          }
+          const float kp = b0f[k] + (st > 0 ? kd[st - 1][k] : 0.f);
           dqs[l] = (st == 2 ? dtf : 0.5f * dtf) * kp;
         }
       }
@@ -542,17 +478,11 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
       float r[LPT];
 #pragma unroll
       for (int k = 0; k < LPT; ++k) r[k] = 0.f;
-      if constexpr (P::CONS) {
-        dflux_level<M, P, D>(dqs, uff, bff, A.p, F.g1h, F.g1l, dF3, tid);
-        __syncthreads();
-        contract_level<M, 0, false>(dF3, sDh, cf, r, tid);
-        contract_level<M, 1, false>(dF3 + NL, sDh, cf, r, tid);
-        if constexpr (D == 3) contract_level<M, 2, false>(dF3 + 2 * NL, sDh, cf, r, tid);
-      } else {
-        contract_level<M, 0, true>(dqs, sDh, cf, r, tid);
-        contract_level<M, 1, true>(dqs, sDh, cf, r, tid);
-        contract_level<M, 2, true>(dqs, sDh, cf, r, tid);
-      }
+      dflux_level<M, P, D>(dqs, uff, bff, A.p, F.g1h, F.g1l, dF3, tid);
+      __syncthreads();
+      contract_level<M, 0>(dF3, sDh, cf, r, tid);
+      contract_level<M, 1>(dF3 + NL, sDh, cf, r, tid);
+      if constexpr (D == 3) contract_level<M, 2>(dF3 + 2 * NL, sDh, cf, r, tid);
 #pragma unroll
       for (int k = 0; k < LPT; ++k) kd[st][k] = r[k];
       __syncthreads();  // the stage's reads of dqs / dF3 are done
@@ -561,21 +491,10 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
     for (int k = 0; k < LPT; ++k) {
       const int l = tid + k * TPB;
       if (l < NL) {
-        float s1 = 0.f, s23 = 0.f, s4 = 0.f;
-        if (has_src) {
-          const int j = l / NV, v = l - (l / NV) * NV;
-          if (v >= 3) {
-            const float amp = (float)(-A.src.M[v - 3] * A.src.phi[j]);
-            s1 = amp * (float)rs[0];
-            s23 = amp * (float)(rs[1] + rs[2]);
-            s4 = amp * (float)rs[3];
-          }
-        }
-        const float k23 = kd[0][k] + kd[1][k] + s23, k4 = kd[2][k] + s4;
+        const float k23 = kd[0][k] + kd[1][k], k4 = kd[2][k];
 #pragma unroll
         for (int t = 0; t < n; ++t)
-          dqs[t * NL + l] = dtf * fmaf(F.th[t], b0f[k],
-                                       fmaf(F.cerk[0][t], s1, fmaf(F.cerk[1][t], k23, F.cerk[2][t] * k4)));
+          dqs[t * NL + l] = dtf * fmaf(F.th[t], b0f[k], fmaf(F.cerk[1][t], k23, F.cerk[2][t] * k4));
       }
     }
     __syncthreads();
@@ -583,9 +502,9 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
 
   // ---- Picard iterations on dq ----------------------------------------------------------
   float R[LPT][n];
-  ff dqb[P::CONS ? LPT : 1];  // time average of the last iterate (float-float)
+  ff dqb[LPT];  // time average of the last iterate (float-float)
 #pragma unroll
-  for (int k = 0; k < (P::CONS ? LPT : 1); ++k) dqb[k] = {0.f, 0.f};
+  for (int k = 0; k < LPT; ++k) dqb[k] = {0.f, 0.f};
   for (int it = 0; it < A.iters; ++it) {
 #pragma unroll
     for (int k = 0; k < LPT; ++k)
@@ -593,43 +512,17 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
       for (int t = 0; t < n; ++t) R[k][t] = 0.f;
     const bool last = (it == A.iters - 1);
     if (it > 0 || A.cerk) {  // dq^0 = 0 gives dR = 0 without a guess
-      if constexpr (P::CONS) {
-        // all directions at once into dF3
-        dflux_nodes_all<M, P, D>(dqs, uff, bff, A.p, F.g1h, F.g1l, dF3, tid);
-        __syncthreads();
-        if (last) {
-          contract_f<M, 0, false, true>(dF3, sDh, sD2, cf, R, tid);
-          contract_f<M, 1, false, true>(dF3 + NSL, sDh, sD2, cf, R, tid);
-          if constexpr (D == 3) contract_f<M, 2, false, true>(dF3 + 2 * NSL, sDh, sD2, cf, R, tid);
-        } else {
-          contract_f<M, 0, false>(dF3, sDh, sD2, cf, R, tid);
-          contract_f<M, 1, false>(dF3 + NSL, sDh, sD2, cf, R, tid);
-          if constexpr (D == 3) contract_f<M, 2, false>(dF3 + 2 * NSL, sDh, sD2, cf, R, tid);
-        }
+      // all directions at once into dF3
+      dflux_nodes_all<M, P, D>(dqs, uff, bff, A.p, F.g1h, F.g1l, dF3, tid);
+      __syncthreads();
+      if (last) {
+        contract_f<M, 0, true>(dF3, sDh, sD2, cf, R, tid);
+        contract_f<M, 1, true>(dF3 + NSL, sDh, sD2, cf, R, tid);
+        if constexpr (D == 3) contract_f<M, 2, true>(dF3 + 2 * NSL, sDh, sD2, cf, R, tid);
       } else {
-        if (last) {
-          contract_f<M, 0, true, true>(dqs, sDh, sD2, cf, R, tid);
-          contract_f<M, 1, true, true>(dqs, sDh, sD2, cf, R, tid);
-          contract_f<M, 2, true, true>(dqs, sDh, sD2, cf, R, tid);
-        } else {
-          contract_f<M, 0, true>(dqs, sDh, sD2, cf, R, tid);
-          contract_f<M, 1, true>(dqs, sDh, sD2, cf, R, tid);
-          contract_f<M, 2, true>(dqs, sDh, sD2, cf, R, tid);
-        }
-      }
-    }
-    if (has_src) {
-#pragma unroll
-      for (int k = 0; k < LPT; ++k) {
-        const int l = tid + k * TPB;
-        if (l < NL) {
-          const int j = l / NV, v = l - (l / NV) * NV;
-          if (v >= 3) {
-            const float amp = (float)(-A.src.M[v - 3] * A.src.phi[j]);
-#pragma unroll
-            for (int t = 0; t < n; ++t) R[k][t] = fmaf(amp, (float)ric[t], R[k][t]);
-          }
-        }
+        contract_f<M, 0>(dF3, sDh, sD2, cf, R, tid);
+        contract_f<M, 1>(dF3 + NSL, sDh, sD2, cf, R, tid);
+        if constexpr (D == 3) contract_f<M, 2>(dF3 + 2 * NSL, sDh, sD2, cf, R, tid);
       }
     }
     __syncthreads();  // every read of dq of this iteration is done
@@ -637,29 +530,20 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
     for (int k = 0; k < LPT; ++k) {
       const int l = tid + k * TPB;
       if (l < NL) {
-        // dq_t = dt (kw1_t B0 + sum_m Kw[t][m] R_m); after the last iteration only the flux
-        // remainders (conservative form) read the nodal dq_t
-        if (!last || P::CONS) {
+        // dq_t = dt (kw1_t B0 + sum_m Kw[t][m] R_m)
 #pragma unroll
-          for (int t = 0; t < n; ++t) {
-            float acc = F.kw1[t] * b0f[k];
+        for (int t = 0; t < n; ++t) {
+          float acc = F.kw1[t] * b0f[k];
 #pragma unroll
-            for (int m = 0; m < n; ++m) acc = fmaf(F.Kw[t][m], R[k][m], acc);
-            dqs[t * NL + l] = dtf * acc;
-          }
+          for (int m = 0; m < n; ++m) acc = fmaf(F.Kw[t][m], R[k][m], acc);
+          dqs[t * NL + l] = dtf * acc;
         }
         if (last) {  // the time average qbar in float-float, from the weights averaged over t
           ff acc = {0.f, 0.f};
           ff_mac(acc, F.wk1h, F.wk1l, b0f[k], b0l[k]);
 #pragma unroll
           for (int m = 0; m < n; ++m) ff_mac(acc, F.wKh[m], F.wKl[m], R[k][m], 0.f);
-          const ff q = ff_mul(dtff, ff_norm(acc.h, acc.l));
-          if constexpr (P::CONS) {
-            dqb[k] = q;
-          } else {  // straight to its place in shared memory (hi, lo over dq)
-            dqs[l] = q.h;
-            dqs[NL + l] = q.l;
-          }
+          dqb[k] = ff_mul(dtff, ff_norm(acc.h, acc.l));
         }
       }
     }
@@ -668,7 +552,7 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
 
   // ---- epilogue in float-float -------------------------------------------------------------
   float *qbh, *qbl;   // time-averaged dq [NL] (hi, lo)
-  if constexpr (P::CONS) {
+  {
     // Time-averaged flux increment = A(u^n) qbar + sum_t w_t N(dq_t): the quadratic remainders N
     // per space-time node in binary32, the linear part once per spatial node in float-float.
     float* NB = dF3;  // [D][n][NL] remainders
@@ -699,9 +583,6 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
     }
     __syncthreads();
     linear_nodes<M, P, D>(qbh, qbl, uff, bff, g1, F, A.p, FB0, tid);
-  } else {
-    qbh = dqs;  // written by the last time solve
-    qbl = dqs + NL;
   }
   __syncthreads();
 
@@ -717,35 +598,15 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
         const int st = (d == 0 ? 1 : (d == 1 ? n : n * n));
         const int jd = (j / st) % n;
         const int j0 = j - jd * st;
-        if constexpr (P::CONS) {
-          // weak-form volume term of the time-averaged flux: sum_m W[j_d][m] G_d[m]
+        // weak-form volume term of the time-averaged flux: sum_m W[j_d][m] G_d[m]
 #pragma unroll
-          for (int m = 0; m < n; ++m) {
-            const ff g = FB0[d * NL + (j0 + m * st) * NV + v];
-            const float2 wm = sW2[jd * n + m];
-            ff_mac(dvol, wm.x, wm.y, g.h, g.l);
-          }
-        } else {
-          const int s = Elastic::src(d, v);
-          if (s >= 0) {
-            ff a = {0.f, 0.f};
-#pragma unroll
-            for (int m = 0; m < n; ++m) {
-              const int i = (j0 + m * st) * NV + s;
-              const float2 dm = sD2[jd * n + m];
-              ff_mac(a, dm.x, dm.y, qbh[i], qbl[i]);
-            }
-            dvol = ff_add(dvol, ff_mul(ff_norm(a.h, a.l), {cf[d * NV + v], cf[3 * NV + d * NV + v]}));
-          }
+        for (int m = 0; m < n; ++m) {
+          const ff g = FB0[d * NL + (j0 + m * st) * NV + v];
+          const float2 wm = sW2[jd * n + m];
+          ff_mac(dvol, wm.x, wm.y, g.h, g.l);
         }
       }
-      double vol = ff_to_d(P::CONS ? dvol : ff_add({b0f[k], b0l[k]}, dvol));
-      if (has_src && v >= 3) {
-        double sbar = 0.0;
-#pragma unroll
-        for (int t = 0; t < n; ++t) sbar = fma(T.w[t], ric[t], sbar);
-        vol = fma(-A.src.M[v - 3] * A.src.phi[j], sbar, vol);
-      }
+      const double vol = ff_to_d(dvol);
       un[l] = fma(dt, vol, ul[k]);
       uff[l] = ff_add(uff[l], {qbh[l], qbl[l]});  // time-averaged state u^n + qbar for the faces
     }
@@ -769,21 +630,17 @@ __device__ __forceinline__ void predictor_mixed_cell(const StepArgs& A, const Ta
         const ff q = uff[jj * NV + v];
         ff_mac(qa0, sE[0][m], sE[1][m], q.h, q.l);
         ff_mac(qa1, sE[2][m], sE[3][m], q.h, q.l);
-        if constexpr (P::CONS) {
-          const ff g = FB0[d * NL + jj * NV + v];
-          ff_mac(fa0, sE[0][m], sE[1][m], g.h, g.l);
-          ff_mac(fa1, sE[2][m], sE[3][m], g.h, g.l);
-        }
+        const ff g = FB0[d * NL + jj * NV + v];
+        ff_mac(fa0, sE[0][m], sE[1][m], g.h, g.l);
+        ff_mac(fa1, sE[2][m], sE[3][m], g.h, g.l);
       }
       double* rec0 = fc + (d * 2) * FR;
       double* rec1 = rec0 + FR;
       const double q0 = ff_to_d(qa0), q1 = ff_to_d(qa1);
       rec0[jp * NV + v] = q0;
       rec1[jp * NV + v] = q1;
-      if constexpr (P::CONS) {
-        rec0[NF * NV + jp * NV + v] = ff_to_d(fa0) * A.g.h[d];
-        rec1[NF * NV + jp * NV + v] = ff_to_d(fa1) * A.g.h[d];
-      }
+      rec0[NF * NV + jp * NV + v] = ff_to_d(fa0) * A.g.h[d];
+      rec1[NF * NV + jp * NV + v] = ff_to_d(fa1) * A.g.h[d];
       if constexpr (M::EULER) {  // the face states as written, for the wave speeds below
         double* qs = reinterpret_cast<double*>(dF3);
         qs[((d * 2) * NF + jp) * NV + v] = q0;
