@@ -47,6 +47,26 @@ struct Tables {
                               // Runge-Kutta guess at the time nodes
 };
 
+// Tables of the FP64 predictor's integer contractions (fx.cuh): entries T 2^p as a signed high word
+// and a signed low word, sum over a row of |entry| < 2^61.
+struct fx2 {
+  int h, l;
+};
+// Bits kept of a contraction's sum (fx_dot: sum / 2^(64 - SH), inputs < 2^60, rows < 2^61): the
+// sums over the directions stay below 2^59, the time averages (weights of sum 1) below 2^60, and
+// what becomes a double below 2^63, one result (SHK) or the sum of three (SHS).
+constexpr int FX_SHD = 0, FX_SHW = 4, FX_SHK = 5, FX_SHS = 4;
+struct TablesX {
+  fx2 D[3][MAXN][MAXN];  // D[i][m] (1/h_d) / max_d (1/h_d)
+  fx2 S[3][MAXN][MAXN + 2];  // volume and cell-local face terms: -D, then -c0 and c1 (the factors
+                             // of the two face values), alike
+  fx2 Kw[MAXN][MAXN];
+  fx2 w[MAXN];           // time weights
+  fx2 e[2][MAXN];        // e0, e1
+  int kR, kV, kS, kw, ke;  // results r of D, S, of Kw on results of D, of w, of e: r 2^(E + k)
+  double mih;            // -max_d (1/h_d)
+};
+
 // Single-precision and float-float copies of the tables for the mixed-precision predictor.
 // A float-float value is hi + lo with hi = fl32(x), lo = fl32(x - hi).
 struct TablesF {
@@ -62,6 +82,7 @@ struct TablesF {
   float e0h[MAXN], e0l[MAXN], e1h[MAXN], e1l[MAXN];
   float th[MAXN];                          // time nodes x_t
   float cerk[3][MAXN];                     // dense-output weights b1, b2 (= b3), b4 at x_t
+  TablesX x;                               // the FP64 predictor's integer tables
 };
 
 // Subcell tables of the limiter (Sec. 3.5).

@@ -219,6 +219,58 @@ void build_tables_f(int order, const Tables& T, TablesF& F) {
   }
 }
 
+// t 2^p rounded, as a signed high and a signed low word.
+fx2 fx_entry(double t, int p) {
+  const long long v = std::llround(std::ldexp(t, p));
+  const uint32_t l = (uint32_t)v;
+  return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
+}
+
+// Largest p with sum_m |M[i][m]| 2^p < 2^61 (and room for the rounding) for each of `rows` rows.
+int fx_scale(int rows, int n, const double* M, int stride) {
+  double big = 0.0;
+  for (int i = 0; i < rows; ++i) {
+    double s = 0.0;
+    for (int m = 0; m < n; ++m) s += std::fabs(M[i * stride + m]);
+    big = std::max(big, s);
+  }
+  return 60 - std::ilogb(big * 1.0000001);
+}
+
+void build_tables_x(int order, int dim, const Tables& T, const Geometry& g, TablesX& X) {
+  std::memset(&X, 0, sizeof(X));
+  const int n = order + 1;
+  double S[MAXN][MAXN + 2] = {};
+  for (int i = 0; i < n; ++i) {
+    for (int m = 0; m < n; ++m) S[i][m] = -T.D[i][m];
+    S[i][n] = -T.c0[i];
+    S[i][n + 1] = T.c1[i];
+  }
+  const int pD = fx_scale(n, n, T.D[0], MAXN), pS = fx_scale(n, n + 2, S[0], MAXN + 2);
+  const int pK = fx_scale(n, n, T.Kw[0], MAXN), pw = fx_scale(1, n, T.w, MAXN);
+  const int pe = std::min(fx_scale(1, n, T.e0, MAXN), fx_scale(1, n, T.e1, MAXN));
+  double mih = 0.0;
+  for (int d = 0; d < dim; ++d) mih = std::max(mih, g.inv_h[d]);
+  for (int i = 0; i < n; ++i) {
+    for (int m = 0; m < n; ++m) {
+      for (int d = 0; d < dim; ++d) X.D[d][i][m] = fx_entry(T.D[i][m] * (g.inv_h[d] / mih), pD);
+      X.Kw[i][m] = fx_entry(T.Kw[i][m], pK);
+    }
+    X.w[i] = fx_entry(T.w[i], pw);
+    X.e[0][i] = fx_entry(T.e0[i], pe);
+    X.e[1][i] = fx_entry(T.e1[i], pe);
+    for (int m = 0; m < n + 2; ++m)
+      for (int d = 0; d < dim; ++d) X.S[d][i][m] = fx_entry(S[i][m] * (g.inv_h[d] / mih), pS);
+  }
+  // inputs are x 2^(1082 - E), results sum / 2^(64 - SH)
+  X.kR = 64 - FX_SHD - pD - 1082;
+  X.kV = 64 - FX_SHS - pS - 1082;
+  X.kS = X.kR + 64 - FX_SHK - pK;
+  X.kw = 64 - FX_SHW - pw - 1082;
+  X.ke = 64 - FX_SHK - pe - 1082;
+  X.mih = -mih;
+}
+
 // Tables of the Picard predictor of a linear system (StepArgs::lin, kernels_ck.cuh).  With
 // Lambda = dt L every iterate at time node t is
 //   q_t = sum_k C_k[t] Lambda^k u + sum_k (sum_m G_k[t][m] s_m) dt Lambda^k g,
@@ -627,6 +679,7 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
   }
   build_tables_f(cfg->order, c->tab, c->tabf);
   for (int d = 0; d < 3; ++d) split_f(c->g.inv_h[d], c->tabf.ihh[d], c->tabf.ihl[d]);
+  build_tables_x(cfg->order, cfg->dim, c->tab, c->g, c->tabf.x);
   split_f(c->p.gamma - 1.0, c->tabf.g1h, c->tabf.g1l);
   const int n = cfg->order + 1;
   c->nodes = 1;

@@ -24,14 +24,23 @@ struct Cfg {
   static constexpr int NF = ipow(n, D - 1);     // nodes per face
   static constexpr int FR = NF * NV * (P::CONS ? 2 : 1);  // doubles per face record
   static constexpr int NPHI = (P::NCP || P::NCPS) ? 2 : 1;  // numerical fluxes per face node and variable
-  static constexpr int TPB_RAW = ((NL + 5) / 6 + 31) / 32 * 32;
-  static constexpr int TPB = TPB_RAW < 64 ? 64 : (TPB_RAW > 512 ? 512 : TPB_RAW);
-  static constexpr int LPT = (NL + TPB - 1) / TPB;   // lines per thread
-  static constexpr int NPT = (NST + TPB - 1) / TPB;  // space-time nodes per thread
   static constexpr int FSLOTS = P::CONS ? cmax(n, D + 1) : 0;
   // shallow water: the surface derivatives d(h + b)/dx_d at every space-time node [NST][D]
   static constexpr int GSLOTS = P::NCPS ? NST * D : 0;
-  static constexpr size_t SMEM = ((size_t)(n + FSLOTS) * NL + GSLOTS) * sizeof(double);
+  static constexpr size_t SMEM_F = ((size_t)(n + FSLOTS) * NL + GSLOTS) * sizeof(double);
+  // the integer form of the FP64 predictor (kernels_fx.cuh): q, velocities, sums (and the surface
+  // derivatives); all nonlinear
+  // conservative systems whose cell fits a block's shared memory (not 3-D Euler at order 6)
+  static constexpr size_t SMEM_X = ((size_t)(n + FSLOTS) * NL + (size_t)NST * D + GSLOTS) * sizeof(double);
+  static constexpr bool FX = P::CONS && !P::LINEAR && SMEM_X <= 228352;
+  static constexpr size_t SMEM = FX && SMEM_X > SMEM_F ? SMEM_X : SMEM_F;
+  // lines per thread aimed at (integer form: one or two rounds of tasks per phase)
+  static constexpr int LPD = !FX ? 6 : (NL > 1024 ? 3 : 2);
+  static constexpr int TPB_RAW = ((NL + LPD - 1) / LPD + 31) / 32 * 32;
+  static constexpr int TPB = TPB_RAW < 64 ? 64 : (TPB_RAW > 512 ? 512 : TPB_RAW);
+  static constexpr int MINB = FX && TPB <= 480 ? 960 / TPB : 1;  // 30 warps per SM
+  static constexpr int LPT = (NL + TPB - 1) / TPB;   // lines per thread
+  static constexpr int NPT = (NST + TPB - 1) / TPB;  // space-time nodes per thread
 };
 
 template <int n, int d>
@@ -998,21 +1007,6 @@ __global__ void __launch_bounds__(256) k_cfl(const __grid_constant__ StepArgs A)
 
 // ---- launchers ----------------------------------------------------------------------------
 template <class P, int D, int N>
-cudaError_t launch_predictor_n(const StepArgs& a, const Tables& t, cudaStream_t s) {
-  using C = Cfg<P, D, N>;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_predictor<P, D, N>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  if (a.g.ncells > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_predictor<P, D, N><<<(unsigned)a.g.ncells, C::TPB, C::SMEM, s>>>(a, t);
-  return cudaGetLastError();
-}
-
-template <class P, int D, int N>
 cudaError_t launch_riemann_n(const StepArgs& a, const Tables& t, cudaStream_t s) {
   using C = Cfg<P, D, N>;
   long long off = 0;
@@ -1098,8 +1092,31 @@ struct FamilyImpl {
 };
 
 }  // namespace ader
+#include "kernels_fx.cuh"
 #include "kernels_mixed.cuh"
 namespace ader {
+
+template <class P, int D, int N>
+cudaError_t launch_predictor_n(const StepArgs& a, const Tables& t, const TablesF& f, cudaStream_t s) {
+  using C = Cfg<P, D, N>;
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e;
+    if constexpr (C::FX)
+      e = cudaFuncSetAttribute(k_predictor_fx<P, D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)C::SMEM);
+    else
+      e = cudaFuncSetAttribute(k_predictor<P, D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)C::SMEM);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  if (a.g.ncells > 0x7fffffffLL) return cudaErrorInvalidValue;
+  if constexpr (C::FX) k_predictor_fx<P, D, N><<<(unsigned)a.g.ncells, C::TPB, C::SMEM, s>>>(a, t, f.x);
+  else k_predictor<P, D, N><<<(unsigned)a.g.ncells, C::TPB, C::SMEM, s>>>(a, t);
+  return cudaGetLastError();
+}
+
 
 template <class P, int D>
 size_t FamilyImpl<P, D>::smem(int order, int prec) {
@@ -1130,7 +1147,7 @@ cudaError_t FamilyImpl<P, D>::predictor(const StepArgs& a, const Tables& t, cons
         ADER_DISPATCH_N(launch_predictor_mixed_n, a, t, f, s)
       }
     }
-    ADER_DISPATCH_N(launch_predictor_n, a, t, s)
+    ADER_DISPATCH_N(launch_predictor_n, a, t, f, s)
   }
 }
 
