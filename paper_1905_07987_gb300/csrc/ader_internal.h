@@ -241,6 +241,10 @@ struct Family {
   // mixed-precision adjoint of a mixed forward step)
   cudaError_t (*adj_run_ck)(const StepArgs&, const AdjArgs&, const Tables&, const TablesF&,
                             int prec, cudaStream_t);
+  // adjoint of the step with the Picard predictor in its polynomial form (StepArgs::lin), and
+  // whether that many levels fit (otherwise adj_run)
+  cudaError_t (*adj_run_lin)(const StepArgs&, const AdjArgs&, const Tables&, cudaStream_t);
+  bool (*adj_lin_fits)(int order, int nlev);
   // one step of every run of an ensemble (fixed dt, no limiter, no receivers); runs: the runs'
   // step arguments of this step in device memory; null when the family has no batched path
   cudaError_t (*ens_step)(const StepArgs* runs, const EnsTable& E, const Tables& t,

@@ -16,6 +16,12 @@ cudaError_t adj_run_ck_n<2>(const StepArgs& a, const AdjArgs& j, const Tables& t
   return AdjLaunchCK<2>::run(a, j, t, s);
 }
 template <>
+cudaError_t adj_run_lin_n<2>(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s) {
+  return AdjLaunchCK<2>::run_lin(a, j, t, s);
+}
+template <>
+bool adj_lin_fits_n<2>(int nlev) { return AdjLaunchCK<2>::fits(nlev); }
+template <>
 cudaError_t adj_run_ck_mixed_n<2>(const StepArgs& a, const AdjArgs& j, const Tables& t,
                                   const TablesF& f, cudaStream_t s) {
   return AdjLaunchCKM<2>::run(a, j, t, f, s);

@@ -1209,21 +1209,23 @@ ader_status ader_adjoint_step(ader_ctx* c, double t_n, double dt, const double* 
   if (!adjoint_supported(c)) return ADER_EUNSUPPORTED;
   if (!c->mat_set) return ADER_ESTATE;
   const bool ck = c->cfg.predictor == ADER_PREDICTOR_CK;
+  // levels: the adjoint of a polynomial of L (Cauchy-Kowalevski, or Picard when its levels fit)
+  const bool levels = ck || c->fam->adj_lin_fits(c->cfg.order, c->nlev);
   const int iters = c->cfg.picard_iters > 0 ? c->cfg.picard_iters : c->cfg.order + 1;
   if (!c->dev_adj) {
     int dev = 0, sms = 0;
     CUDA_OK(cudaGetDevice(&dev));
     CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // the Cauchy-Kowalevski adjoint keeps its cell in shared memory: no iterate slabs
-    c->adj_blocks = ck ? 0 : sms * c->fam->adj_blocks_per_sm(c->cfg.order);
-    c->adj_spb = ck ? 0 : c->fam->adj_scratch_per_block(c->cfg.order, iters);
+    // the adjoint of the levels keeps its cell in shared memory: no iterate slabs
+    c->adj_blocks = levels ? 0 : sms * c->fam->adj_blocks_per_sm(c->cfg.order);
+    c->adj_spb = levels ? 0 : c->fam->adj_scratch_per_block(c->cfg.order, iters);
     long long nfaces = 0;
     for (int d = 0; d < 3; ++d) nfaces += (long long)(c->g.n[d] + 1) * (c->g.ncells / c->g.n[d]);
     cudaError_t e = cudaMalloc(&c->dev_adj, sizeof(DevScalars));
     if (e == cudaSuccess) e = cudaMalloc(&c->adjf, (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&c->gface, (size_t)nfaces * 6 * sizeof(double));
-    // Picard: the iterate slabs; Cauchy-Kowalevski: lambda's projections onto the cells' faces
-    const size_t scratch = ck ? (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar
+    // lambda's projections onto the cells' faces, or the iterate slabs
+    const size_t scratch = levels ? (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar
                               : (size_t)c->adj_blocks * c->adj_spb;
     if (e == cudaSuccess) e = cudaMalloc(&c->adj_scratch, scratch * sizeof(double));
     if (e != cudaSuccess) {
@@ -1243,10 +1245,11 @@ ader_status ader_adjoint_step(ader_ctx* c, double t_n, double dt, const double* 
   a.u = u_n;
   a.dev = c->dev_adj;
   a.iters = iters;
-  if (ck) {
+  if (levels) {
     // the adjoint kernels form the forward face data themselves
     AdjArgs j{u_n, lam, dJdu, grad_mat, grad_M, c->adjf, c->gface, nullptr, 0, c->adj_scratch};
-    CUDA_OK(c->fam->adj_run_ck(a, j, c->tab, c->tabf, c->cfg.precision, c->stream));
+    if (ck) CUDA_OK(c->fam->adj_run_ck(a, j, c->tab, c->tabf, c->cfg.precision, c->stream));
+    else CUDA_OK(c->fam->adj_run_lin(a, j, c->tab, c->stream));
   } else {
     // forward face data of the step from u^n (the predictor also writes the scratch next state)
     CUDA_OK(c->fam->predictor(a, c->tab, c->tabf, ADER_PREC_FP64, c->stream));
@@ -1344,22 +1347,25 @@ ader_status ader_adjoint_step_static(ader_ctx* c, double t_n, double dt, const d
   CUDA_OK(cudaGetDevice(&dev));
   void* base = nullptr;
   CUDA_OK(static_array_address(&base));
-  // layout: device scalars | face adjoints | face material gradients | per-block iterate slabs
-  // (Picard) or lambda's face projections (Cauchy-Kowalevski)
+  // layout: device scalars | face adjoints | face material gradients | lambda's face projections, or
+  // per-block iterate slabs (Picard, see below)
   const int iters = c->cfg.picard_iters > 0 ? c->cfg.picard_iters : c->cfg.order + 1;
   long long nfaces = 0;
   for (int d = 0; d < 3; ++d) nfaces += (long long)(c->g.n[d] + 1) * (c->g.ncells / c->g.n[d]);
   const size_t b_dev = round256(sizeof(DevScalars));
   const size_t b_adjf = round256((size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar * sizeof(double));
   const size_t b_gface = round256((size_t)nfaces * 6 * sizeof(double));
-  // Picard: one iterate slab per thread block; Cauchy-Kowalevski: lambda's face projections
-  const long long spb = ck ? 0 : c->fam->adj_scratch_per_block(c->cfg.order, iters);
-  const size_t b_slab = ck ? (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar * sizeof(double)
-                           : (size_t)spb * sizeof(double);
+  // lambda's face projections; a Picard step whose projections (or levels) do not fit: one iterate
+  // slab per thread block
   const size_t fixed = b_dev + b_adjf + b_gface;
+  const size_t b_proj = (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar * sizeof(double);
+  const bool levels = ck || (c->fam->adj_lin_fits(c->cfg.order, c->nlev) &&
+                             fixed + b_proj <= kStaticScratchBytes);
+  const long long spb = levels ? 0 : c->fam->adj_scratch_per_block(c->cfg.order, iters);
+  const size_t b_slab = levels ? b_proj : (size_t)spb * sizeof(double);
   if (fixed + b_slab > kStaticScratchBytes) return ADER_EINVAL;  // grid too large for the array
   long long blocks = 0;
-  if (!ck) {
+  if (!levels) {
     int sms = 0;
     CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     blocks = (long long)sms * c->fam->adj_blocks_per_sm(c->cfg.order);
@@ -1376,9 +1382,10 @@ ader_status ader_adjoint_step_static(ader_ctx* c, double t_n, double dt, const d
   a.u = u_n;
   a.dev = dev_s;
   a.iters = iters;
-  if (ck) {
+  if (levels) {
     AdjArgs j{u_n, lam, dJdu, grad_mat, grad_M, adjf, gface, nullptr, 0, slab};
-    CUDA_OK(c->fam->adj_run_ck(a, j, c->tab, c->tabf, c->cfg.precision, c->stream));
+    if (ck) CUDA_OK(c->fam->adj_run_ck(a, j, c->tab, c->tabf, c->cfg.precision, c->stream));
+    else CUDA_OK(c->fam->adj_run_lin(a, j, c->tab, c->stream));
   } else {
     CUDA_OK(c->fam->predictor(a, c->tab, c->tabf, ADER_PREC_FP64, c->stream));
     AdjArgs j{u_n, lam, dJdu, grad_mat, grad_M, adjf, gface, slab, spb};

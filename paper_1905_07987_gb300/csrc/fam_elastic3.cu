@@ -29,6 +29,10 @@ int adj_bps_n();
 template <int N>
 cudaError_t adj_run_ck_n(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s);
 template <int N>
+cudaError_t adj_run_lin_n(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s);
+template <int N>
+bool adj_lin_fits_n(int nlev);
+template <int N>
 cudaError_t adj_run_ck_mixed_n(const StepArgs& a, const AdjArgs& j, const Tables& t,
                                const TablesF& f, cudaStream_t s);
 namespace {
@@ -63,6 +67,26 @@ cudaError_t adj_run_ck(const StepArgs& a, const AdjArgs& j, const Tables& t, con
     case 5: return adj_run_ck_n<5>(a, j, t, s);
   }
   return cudaErrorInvalidValue;
+}
+cudaError_t adj_run_lin(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s) {
+  switch (a.g.order) {
+    case 1: return adj_run_lin_n<1>(a, j, t, s);
+    case 2: return adj_run_lin_n<2>(a, j, t, s);
+    case 3: return adj_run_lin_n<3>(a, j, t, s);
+    case 4: return adj_run_lin_n<4>(a, j, t, s);
+    case 5: return adj_run_lin_n<5>(a, j, t, s);
+  }
+  return cudaErrorInvalidValue;
+}
+bool adj_lin_fits(int order, int nlev) {
+  switch (order) {
+    case 1: return adj_lin_fits_n<1>(nlev);
+    case 2: return adj_lin_fits_n<2>(nlev);
+    case 3: return adj_lin_fits_n<3>(nlev);
+    case 4: return adj_lin_fits_n<4>(nlev);
+    case 5: return adj_lin_fits_n<5>(nlev);
+  }
+  return false;
 }
 long long adj_scratch(int order, int iters) {
   switch (order) {
@@ -162,6 +186,8 @@ const Family* family_elastic3() {
     g.predictor = &predictor_picard_elastic3;
     g.adj_run = &adj_run;
     g.adj_run_ck = &adj_run_ck;
+    g.adj_run_lin = &adj_run_lin;
+    g.adj_lin_fits = &adj_lin_fits;
     g.adj_scratch_per_block = &adj_scratch;
     g.adj_blocks_per_sm = &adj_bps;
     g.ens_step = &ens_step;

@@ -11,8 +11,9 @@
 //                  predictor (kept in a per-block global scratch slab), then the adjoint of the
 //                  volume term, of the face extrapolation, and of the Picard iteration in reverse.
 // The forward face data q_bar of the step are recomputed by the forward predictor kernel first.
-// With the Cauchy-Kowalevski predictor (kernels_adjoint_ck.cuh) k_adj_riemann runs in two halves
-// around the cell kernel, which forms the forward face data itself.
+// The adjoints of the levels (kernels_adjoint_ck.cuh: the Cauchy-Kowalevski predictor, and the Picard
+// predictor wherever their buffers fit) run k_adj_riemann in two halves around a cell kernel that
+// forms the forward face data itself; k_adj_cell is left with the other Picard steps.
 #pragma once
 #include "kernels.cuh"
 

@@ -403,45 +403,328 @@ __global__ void __launch_bounds__(256) k_adj_face_sum(const __grid_constant__ St
     atomicOr(&A.dev->status, ST_NONFINITE);
 }
 
+// ---- Picard predictor ------------------------------------------------------------------------
+//
+// The Picard predictor's time average is qbar = sum_{k<=K} w_k a_k + sum_{k<K} gam_k b_k with
+// a_0 = u, b_0 = dt g and both advanced by f_k L, f_k = dt phi_k (kernels_ck.cuh).  Its adjoint is
+// the same reverse recursion with those weights, once for the levels of u and, in the source's
+// cell, once for the levels of the source:
+//   ab_k = w_k F + f_k L^T nu_{k+1},   nu_{k+1} = (w_k / phi_k) lambda + ab_{k+1},   ab_{K+1} = 0,
+//   lambda^n = lambda + ab_0 (the levels of u),   material sum_k f_k nu_{k+1}^T (dL/dm) a_k,
+//   moment dt sbar lambda^T (dg/dM) + dt ab_0^T (dg/dM) (the levels of the source).
+// K + 1 applications of L and of L^T replace the recomputation and reversal of K iterations over
+// n time nodes (k_adj_cell, kept for the grids and iteration counts whose buffers do not fit: the
+// K + 2 records of a block's cells in shared memory, lambda's projections in the fixed array of
+// the allocation-free entry point).  Measured, misfit gradient over 4 steps of 19 x 16 x 13 cells
+// at order 3: 33.9 -> 7.1 ms (46.3 with the space-time forward predictor).
+
+// Forward and reverse levels of one sequence whose first level is in the record 0 of `base` ([K + 2]
+// records).  w(k): weight of level k.  Adds sum_k w_k a_k to qb and the material terms to gm; ab
+// returns ab_0.  All threads of the block; act: the thread has a node of the sequence.
+template <int N, class W>
+__device__ __forceinline__ void adj_lin_levels(double* base, int K, bool act, int j, double dt,
+                                               const double* phi, W w, const double (&Dr)[3][N + 1],
+                                               const double (&DT)[3][N + 1],
+                                               const double (&cf)[3][4], double irho, double lam,
+                                               double ik, double imu, const double (&lam_j)[9],
+                                               const double (&Fj)[9], double (&qb)[9],
+                                               double (&gm)[3], double (&ab)[9]) {
+  using C = CfgCKA<N>;
+  constexpr int NV = C::NV, NVP = C::NVP, REC = C::REC;
+  double* const spare = base + (K + 1) * REC;
+#pragma unroll 1
+  for (int k = 0; k <= K; ++k) {
+    if (act) {
+      const double* r = base + k * REC + j * NVP;
+      const double wk = w(k);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) qb[v] = fma(wk, r[v], qb[v]);
+      double R[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) R[v] = 0.0;
+      ck_apply<N>(base + k * REC, j, Dr, cf, R);
+      const double f = dt * (k < K ? phi[k] : 0.5);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) R[v] *= f;
+      if (k < K) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) base[(k + 1) * REC + j * NVP + v] = R[v];
+      } else {
+        // the last level's f_K L a_K (phi_K = 1/2), with nu_{K+1} = 2 w_K lambda
+        double nu[NV];
+        double* o = spare + j * NVP;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) o[v] = nu[v] = 2.0 * wk * lam_j[v];
+        o[9] = nu[3] + nu[4] + nu[5];
+        ck_dmat_R(R, nu, irho, lam, ik, imu, gm);
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll 1
+  for (int k = K; k >= 0; --k) {
+    const double* Yin = ((K - k) & 1) ? base : spare;
+    double* Yout = ((K - k) & 1) ? spare : base;
+    if (act) {
+      double Tt[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Tt[v] = 0.0;
+      ck_apply_T<N>(Yin, j, DT, cf, Tt);
+      const double f = dt * (k < K ? phi[k] : 0.5), wk = w(k);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) ab[v] = fma(f, Tt[v], wk * Fj[v]);
+      if (k > 0) {
+        // nu_k, and its pairing with f_{k-1} L a_{k-1} = a_k
+        const double wl = w(k - 1) / phi[k - 1];
+        double nu[NV], P[NV];
+        double* o = Yout + j * NVP;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          o[v] = nu[v] = fma(wl, lam_j[v], ab[v]);
+          P[v] = base[k * REC + j * NVP + v];
+        }
+        o[9] = nu[3] + nu[4] + nu[5];
+        ck_dmat_R(P, nu, irho, lam, ik, imu, gm);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(CfgCKA<N>::TPB)
+    k_adj_cell_lin(const __grid_constant__ StepArgs A, const __grid_constant__ AdjArgs J,
+                   const __grid_constant__ Tables T) {
+  using C = CfgCKA<N>;
+  constexpr int n = C::n, NS = C::NS, NV = C::NV, NL = C::NL, NVP = C::NVP, CPB = C::CPB;
+  constexpr int TPB = C::TPB, REC = C::REC, NF = C::NF;
+  extern __shared__ __align__(16) double smem[];  // [CPB][K + 2][NS][NVP]
+  __shared__ double s_smp[n + 3], s_sbar;
+  __shared__ double s_sum[CPB][9];  // per-cell gradient sums (3 material, 6 moment)
+  const int tid = threadIdx.x;
+  const int K = A.nlev, NBUF = K + 2;
+  const int slot = tid / NS;
+  const int j = tid - slot * NS;
+  const long long c0 = (long long)blockIdx.x * CPB;
+  const int ncb = (int)(A.g.ncells - c0 < CPB ? A.g.ncells - c0 : CPB);
+  const bool act = slot < ncb;
+  const long long c = c0 + slot;
+  double* base = smem + (size_t)(act ? slot : 0) * NBUF * REC;
+  const double dt = A.dev->dt;
+  const double* phi = A.lin + K + 1;
+
+  // lambda^{n+1} into the record 0, coalesced, then into registers
+  for (int e = tid; e < ncb * NL; e += TPB) {
+    const int s = e / NL, r = e - s * NL;
+    smem[(size_t)s * NBUF * REC + (r / NV) * NVP + r % NV] = J.lam[c0 * NL + e];
+  }
+  const long long sc = A.src.cell - c0;
+  const bool srcb = sc >= 0 && sc < ncb;
+  if (srcb && tid == 0) {
+    double sbar = 0.0;
+    for (int m = 0; m < n + 3; ++m) {
+      s_smp[m] = ck_ricker<N>(A, T, m, A.dev->t, dt);
+      if (m < n) sbar = fma(T.w[m], s_smp[m], sbar);
+    }
+    s_sbar = sbar;
+  }
+  const bool srcc = srcb && act && sc == slot;  // this thread's cell holds the source
+  double Dr[3][n], DT[3][n], cf[3][4];
+  double irho = 0.0, lam = 0.0, ik = 0.0, imu = 0.0;
+  if (act) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int jd = d == 0 ? j % n : (d == 1 ? (j / n) % n : j / (n * n));
+#pragma unroll
+      for (int m = 0; m < n; ++m) {
+        Dr[d][m] = T.D[jd][m];
+        DT[d][m] = T.D[m][jd];
+      }
+    }
+    irho = 1.0 / A.mat[c * 3 + 0];
+    lam = A.mat[c * 3 + 1];
+    const double mu = A.mat[c * 3 + 2];
+    ik = 1.0 / (3.0 * lam + 2.0 * mu);
+    imu = 1.0 / mu;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const double ih = A.g.inv_h[d];
+      cf[d][0] = irho * ih;
+      cf[d][1] = (lam + 2.0 * mu) * ih;
+      cf[d][2] = lam * ih;
+      cf[d][3] = mu * ih;
+    }
+  }
+  __syncthreads();
+  double lam_j[NV], Fj[NV], qb[NV], ab[NV], gm[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int v = 0; v < NV; ++v) lam_j[v] = Fj[v] = qb[v] = ab[v] = 0.0;
+  if (act) {
+    // F: the face adjoints carried back to the nodes (transposed extrapolation)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) lam_j[v] = base[j * NVP + v];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
+      const int jd = (j / st) % n;
+      const int jp = (j % st) + (j / (st * n)) * st;
+      const double* af = J.adjf + (c * 3 + d) * 2 * (long long)(NF * NV) + jp * NV;
+      const double e0 = T.e0[jd], e1 = T.e1[jd];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Fj[v] = fma(e0, af[v], fma(e1, af[NF * NV + v], Fj[v]));
+    }
+  }
+  double gM[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (srcb) {  // the levels of the source (the source's cell alone works)
+    const double ph = srcc ? A.src.phi[j] : 0.0;
+    if (srcc) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) base[j * NVP + v] = v >= 3 ? -dt * A.src.M[v >= 3 ? v - 3 : 0] * ph : 0.0;
+    }
+    __syncthreads();
+    const double* sm = s_smp;
+    adj_lin_levels<N>(base, K - 1, srcc, j, dt, phi, [&](int k) { return lin_gamma<N>(A, sm, k); }, Dr,
+                      DT, cf, irho, lam, ik, imu, lam_j, Fj, qb, gm, ab);
+    if (srcc) {
+#pragma unroll
+      for (int a = 0; a < 6; ++a) gM[a] = -ph * dt * fma(s_sbar, lam_j[3 + a], ab[3 + a]);
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < ncb * NL; e += TPB) {
+    const int s = e / NL, r = e - s * NL;
+    smem[(size_t)s * NBUF * REC + (r / NV) * NVP + r % NV] = J.u_n[c0 * NL + e];
+  }
+  __syncthreads();
+  adj_lin_levels<N>(base, K, act, j, dt, phi, [&](int k) { return A.lin[k]; }, Dr, DT, cf, irho, lam,
+                    ik, imu, lam_j, Fj, qb, gm, ab);
+
+  // qbar (for the forward face data) into record 0, lambda^n = lambda + ab_0 into record 1, the
+  // gradient terms of the nodes into record 2 (K >= 1), for coalesced stores and fixed-order sums
+  double* red = base + 2 * REC;
+  if (act) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      base[j * NVP + v] = qb[v];
+      base[REC + j * NVP + v] = lam_j[v] + ab[v];
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) red[q * NS + j] = gm[q];
+    if (srcc)
+#pragma unroll
+      for (int q = 0; q < 6; ++q) red[(3 + q) * NS + j] = gM[q];
+  }
+  __syncthreads();
+  bool bad = false;
+  for (int e = tid; e < ncb * NL; e += TPB) {
+    const int s = e / NL, r = e - s * NL;
+    double out = smem[(size_t)s * NBUF * REC + REC + (r / NV) * NVP + r % NV];
+    if (J.dJdu) out += J.dJdu[c0 * NL + e];
+    J.lam[c0 * NL + e] = out;
+    bad |= !isfinite(out);
+  }
+  if (bad) atomicOr(&A.dev->status, ST_NONFINITE);
+  for (int e = tid; e < ncb * NF * NV; e += TPB) {
+    const int s = e / (NF * NV), r = e - s * (NF * NV);
+    const int v = r % NV, jp = r / NV;
+    const double* Xs = smem + (size_t)s * NBUF * REC;
+    double* fc = A.face + (c0 + s) * (3 * 2 * NF * NV) + jp * NV + v;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int st = (d == 0 ? 1 : (d == 1 ? n : n * n));
+      const int jbase = (jp % st) + (jp / st) * st * n;
+      double q0 = 0.0, q1 = 0.0;
+#pragma unroll
+      for (int m = 0; m < n; ++m) {
+        const double x = Xs[(jbase + m * st) * NVP + v];
+        q0 = fma(T.e0[m], x, q0);
+        q1 = fma(T.e1[m], x, q1);
+      }
+      fc[(d * 2 + 0) * NF * NV] = q0;
+      fc[(d * 2 + 1) * NF * NV] = q1;
+    }
+  }
+  // component q is summed by the cell's thread q mod NS (order 1 has fewer nodes than sums)
+  for (int q = j; act && q < (srcc ? 9 : 3); q += NS) {
+    double s = 0.0;
+    for (int i = 0; i < NS; ++i) s += red[q * NS + i];
+    s_sum[slot][q] = s;
+  }
+  __syncthreads();
+  // the cell's own material gradient (its faces' share follows in k_adj_face_sum)
+  if (act && j == 0) {
+    for (int q = 0; q < 3; ++q) J.grad_mat[c * 3 + q] += s_sum[slot][q];
+    if (!isfinite(s_sum[slot][0]) || !isfinite(s_sum[slot][1]) || !isfinite(s_sum[slot][2]))
+      atomicOr(&A.dev->status, ST_NONFINITE);
+    if (srcc)
+      for (int q = 0; q < 6; ++q) J.grad_M[q] += s_sum[slot][3 + q];
+  }
+}
+
 template <int N>
 cudaError_t adj_run_ck_n(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s);
+template <int N>
+cudaError_t adj_run_lin_n(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s);
+template <int N>
+bool adj_lin_fits_n(int nlev);
+
+// lambda's projections onto every cell's faces -> face adjoints -> cell kernel (forward face data
+// out) -> face material gradients -> their sums per cell
+template <int N, class Kernel>
+cudaError_t adj_run_levels(Kernel kernel, size_t smem, const StepArgs& a, const AdjArgs& j,
+                           const Tables& t, cudaStream_t s) {
+  using C = CfgCKA<N>;
+  long long offs[3] = {0, 0, 0}, off = 0;
+  for (int d = 0; d < 3; ++d) {
+    offs[d] = off;
+    off += (long long)(a.g.n[d] + 1) * (a.g.ncells / a.g.n[d]);
+  }
+  cudaError_t e = launch_adj_proj<N>(a, j, t, s);
+  if (e != cudaSuccess) return e;
+  for (int d = 0; d < 3; ++d) {
+    e = launch_adj_riemann<N, 1>(a, j, t, d, offs[d], s);
+    if (e != cudaSuccess) return e;
+  }
+  const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  kernel<<<(unsigned)blocks, C::TPB, smem, s>>>(a, j, t);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  for (int d = 0; d < 3; ++d) {
+    e = launch_adj_riemann<N, 2>(a, j, t, d, offs[d], s);
+    if (e != cudaSuccess) return e;
+  }
+  k_adj_face_sum<N><<<(unsigned)((a.g.ncells + 255) / 256), 256, 0, s>>>(a, j, offs[1], offs[2]);
+  return cudaGetLastError();
+}
 
 template <int N>
 struct AdjLaunchCK {
   static cudaError_t run(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s) {
-    using C = CfgCKA<N>;
+    constexpr size_t SMEM = CfgCKA<N>::SMEM;
     static bool attr = false;
     if (!attr) {
-      cudaError_t e = cudaFuncSetAttribute(k_adj_cell_ck<N>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)C::SMEM);
+      const cudaError_t e = cudaFuncSetAttribute(
+          k_adj_cell_ck<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
       if (e != cudaSuccess) return e;
       attr = true;
     }
-    long long offs[3] = {0, 0, 0}, off = 0;
-    for (int d = 0; d < 3; ++d) {
-      offs[d] = off;
-      off += (long long)(a.g.n[d] + 1) * (a.g.ncells / a.g.n[d]);
-    }
-    // lambda's projections onto every cell's faces -> face adjoints -> cell kernel (forward face
-    // data out) -> face material gradients -> their sums per cell
-    cudaError_t e0 = launch_adj_proj<N>(a, j, t, s);
-    if (e0 != cudaSuccess) return e0;
-    for (int d = 0; d < 3; ++d) {
-      cudaError_t e = launch_adj_riemann<N, 1>(a, j, t, d, offs[d], s);
+    return adj_run_levels<N>(k_adj_cell_ck<N>, SMEM, a, j, t, s);
+  }
+  // Picard predictor (a.nlev levels); the records of a block have to fit its shared memory
+  static size_t smem_lin(int nlev) {
+    return (size_t)CfgCKA<N>::CPB * (nlev + 2) * CfgCKA<N>::REC * sizeof(double);
+  }
+  static bool fits(int nlev) { return nlev >= 1 && nlev < 64 && smem_lin(nlev) <= 232448 - 4096; }
+  static cudaError_t run_lin(const StepArgs& a, const AdjArgs& j, const Tables& t, cudaStream_t s) {
+    static bool attr = false;
+    if (!attr) {
+      const cudaError_t e = cudaFuncSetAttribute(
+          k_adj_cell_lin<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 4096);
       if (e != cudaSuccess) return e;
+      attr = true;
     }
-    const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
-    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-    k_adj_cell_ck<N><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, j, t);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    for (int d = 0; d < 3; ++d) {
-      e = launch_adj_riemann<N, 2>(a, j, t, d, offs[d], s);
-      if (e != cudaSuccess) return e;
-    }
-    k_adj_face_sum<N><<<(unsigned)((a.g.ncells + 255) / 256), 256, 0, s>>>(a, j, offs[1], offs[2]);
-    return cudaGetLastError();
+    return adj_run_levels<N>(k_adj_cell_lin<N>, smem_lin(a.nlev), a, j, t, s);
   }
 };
 

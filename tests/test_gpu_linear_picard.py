@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from cases import Case, rel_linf
+from oracle.adjoint import step_vjp
 from paper_1905_07987_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -37,3 +38,49 @@ def test_fp64(order, iters, guess):
 def test_mixed(order, iters, guess):
     out, ref, u = run(order, iters, guess, "mixed")
     assert np.abs(out - ref).max() < 2e-6 * np.abs(ref - u).max()
+
+
+def device(a):
+    return torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).cuda()
+
+
+def adjoint(c, u, lam, dt, t, static):
+    lam_d = device(lam)
+    gm = torch.zeros(c.ctx.cells * 3, dtype=torch.float64, device="cuda")
+    gM = torch.zeros(6, dtype=torch.float64, device="cuda")
+    c.ctx.adjoint_step(t, dt, device(u), lam_d, gm, gM, static=static)
+    c.ctx.sync()
+    return lam_d.cpu().numpy(), gm.cpu().numpy(), gM.cpu().numpy()
+
+
+def close(a, b):
+    return np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+
+
+# 40 iterations: more levels than fit, the adjoint that keeps the iterates
+@pytest.mark.parametrize("static", [False, True])
+@pytest.mark.parametrize("order,iters", [(1, 1), (1, 4), (2, 7), (3, 1), (4, 3), (5, 6), (2, 40)])
+def test_adjoint(order, iters, static):
+    nc = (3, 3, 1) if order < 4 else (2, 1, 2)
+    mat = synth.elastic_material(nc, seed=order)
+    c = Case("elastic", 3, order, nc, hi=tuple(0.5 * k for k in nc), bc="absorbing", material=mat,
+             picard_iters=iters)
+    c.point_source([0.7, 0.2, 0.3], synth.moment_tensor(5), 2.0, 0.4)
+    rng = np.random.default_rng(order)
+    u, lam = rng.standard_normal(c.shape), rng.standard_normal(c.shape)
+    dt = 0.7 * float(c.oracle.cfl_dt(torch.from_numpy(u)))
+    ref = step_vjp(c.oracle, torch.from_numpy(u), torch.from_numpy(lam), dt, 0.35)
+    out = adjoint(c, u, lam, dt, 0.35, static)
+    for a, b in zip(out, ref):
+        assert close(a, b.numpy().reshape(-1))
+
+
+def test_adjoint_static_beyond_the_projections():
+    # 16 x 16 x 16 cells at order 4: the projections do not fit the fixed array, the iterate slabs do
+    nc = (16, 16, 16)
+    mat = synth.elastic_material(nc, seed=2)
+    c = Case("elastic", 3, 4, nc, hi=(8.0,) * 3, bc="periodic", material=mat)
+    rng = np.random.default_rng(1)
+    u, lam = rng.standard_normal(c.shape), rng.standard_normal(c.shape)
+    a, b = (adjoint(c, u, lam, 1e-3, 0.0, s) for s in (False, True))
+    assert close(a[0], b[0]) and close(a[1], b[1])
