@@ -52,19 +52,38 @@ struct Tables {
 struct fx2 {
   int h, l;
 };
+// A table entry: with the upper half of the low word, for the low words' products.
+struct fx3 {
+  int h, l, q;
+};
 // Bits kept of a contraction's sum (fx_dot: sum / 2^(64 - SH), inputs < 2^60, rows < 2^61): the
 // sums over the directions stay below 2^59, the time averages (weights of sum 1) below 2^60, and
 // what becomes a double below 2^63, one result (SHK) or the sum of three (SHS).
 constexpr int FX_SHD = 0, FX_SHW = 4, FX_SHK = 5, FX_SHS = 4;
 struct TablesX {
-  fx2 D[3][MAXN][MAXN];  // D[i][m] (1/h_d) / max_d (1/h_d)
-  fx2 S[3][MAXN][MAXN + 2];  // volume and cell-local face terms: -D, then -c0 and c1 (the factors
+  fx3 D[3][MAXN][MAXN];  // D[i][m] (1/h_d) / max_d (1/h_d)
+  fx3 S[3][MAXN][MAXN + 2];  // volume and cell-local face terms: -D, then -c0 and c1 (the factors
                              // of the two face values), alike
-  fx2 Kw[MAXN][MAXN];
-  fx2 w[MAXN];           // time weights
-  fx2 e[2][MAXN];        // e0, e1
+  fx3 Kw[MAXN][MAXN];
+  fx3 w[MAXN];           // time weights
+  fx3 e[2][MAXN];        // e0, e1
   int kR, kV, kS, kw, ke;  // results r of D, S, of Kw on results of D, of w, of e: r 2^(E + k)
   double mih;            // -max_d (1/h_d)
+};
+
+// Tables of the elastic predictors' integer form (kernels_ck_fx.cuh): the derivative in the parity basis
+// (e_m = x_m + x_{n-1-m}, o_m = x_m - x_{n-1-m}, 2 x_c): even outputs from odd inputs (ev), odd
+// outputs from even inputs and the middle (od), the middle's output (mid); the face values e0, e1.
+// most levels of the integer form (the defaults, with the Runge-Kutta guess too)
+__host__ __device__ constexpr int fxe_levels(int order) { return order + 5; }
+constexpr int FXE_SHG = 4, FXE_SHC = 5;     // bits kept of the derivatives and of the material products
+struct TablesE {
+  fx3 ev[MAXN / 2][MAXN / 2];
+  fx3 od[MAXN / 2][MAXN / 2 + 1];
+  fx3 mid[MAXN / 2];
+  fx3 e[2][MAXN];
+  int kc;                                   // material coefficients are x 2^kc
+  int ke;                                   // face values: r 2^(E + ke)
 };
 
 // Single-precision and float-float copies of the tables for the mixed-precision predictor.
@@ -83,6 +102,7 @@ struct TablesF {
   float th[MAXN];                          // time nodes x_t
   float cerk[3][MAXN];                     // dense-output weights b1, b2 (= b3), b4 at x_t
   TablesX x;                               // the FP64 predictor's integer tables
+  TablesE el;                              // the elastic predictors' integer tables
 };
 
 // Subcell tables of the limiter (Sec. 3.5).
@@ -212,6 +232,11 @@ struct StepArgs {
   // levels, then nlev rows of n + 3 weights of the wavelet samples (time nodes, 0, 1/2, 1).
   const double* lin;
   int nlev;
+  // elastic: factors r_k of the levels b_{k+1} = r_k dt L b_k (b_0 = u^n) whose plain sum is the time
+  // average, for the integer form of the predictors, [nfx + 1] in device memory, the last one 1 (0
+  // levels: the form does not apply)
+  const double* rfx;
+  int nfx;
   // hybrid limiter: the cells with FV steps left (nonzero) skip the predictor; their face
   // neighbours compute with FV too, so nothing kept reads their DG data (null: every cell)
   const uint8_t* skip;

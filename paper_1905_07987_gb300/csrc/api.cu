@@ -219,11 +219,11 @@ void build_tables_f(int order, const Tables& T, TablesF& F) {
   }
 }
 
-// t 2^p rounded, as a signed high and a signed low word.
-fx2 fx_entry(double t, int p) {
+// t 2^p rounded, as a signed high and a signed low word (and the low word's upper half).
+fx3 fx_entry(double t, int p) {
   const long long v = std::llround(std::ldexp(t, p));
   const uint32_t l = (uint32_t)v;
-  return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
+  return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l, (int)l >> 16};
 }
 
 // Largest p with sum_m |M[i][m]| 2^p < 2^61 (and room for the rounding) for each of `rows` rows.
@@ -269,6 +269,35 @@ void build_tables_x(int order, int dim, const Tables& T, const Geometry& g, Tabl
   X.kw = 64 - FX_SHW - pw - 1082;
   X.ke = 64 - FX_SHK - pe - 1082;
   X.mih = -mih;
+}
+
+void build_tables_e(int order, const Tables& T, TablesE& X) {
+  std::memset(&X, 0, sizeof(X));
+  const int n = order + 1, H = n / 2;
+  double P[MAXN + 1][MAXN] = {};  // even rows, odd rows, the middle's
+  for (int i = 0; i < H; ++i)
+    for (int m = 0; m < H; ++m) {
+      P[i][m] = T.D[i][m] - T.D[i][n - 1 - m];
+      P[H + i][m] = T.D[i][m] + T.D[i][n - 1 - m];
+    }
+  if (n % 2)
+    for (int i = 0; i < H; ++i) {
+      P[H + i][H] = T.D[i][H];
+      P[2 * H][i] = 2.0 * T.D[H][i];
+    }
+  const int p = fx_scale(2 * H + 1, H + 1, P[0], MAXN);
+  const int pe = std::min(fx_scale(1, n, T.e0, MAXN), fx_scale(1, n, T.e1, MAXN));
+  for (int i = 0; i < H; ++i) {
+    for (int m = 0; m < H; ++m) X.ev[i][m] = fx_entry(P[i][m], p);
+    for (int m = 0; m <= H; ++m) X.od[i][m] = fx_entry(P[H + i][m], p);
+    X.mid[i] = fx_entry(P[2 * H][i], p);
+  }
+  for (int i = 0; i < n; ++i) {
+    X.e[0][i] = fx_entry(T.e0[i], pe);
+    X.e[1][i] = fx_entry(T.e1[i], pe);
+  }
+  X.kc = 64 - FXE_SHG - p + 64 - FXE_SHC;
+  X.ke = 60 - pe - 1082;
 }
 
 // Tables of the Picard predictor of a linear system (StepArgs::lin, kernels_ck.cuh).  With
@@ -471,6 +500,8 @@ struct ader_ctx {
   double* phi = nullptr;
   double* lin = nullptr;     // elastic, Picard predictor: weights of its polynomial levels
   int nlev = 0;
+  double* rfx = nullptr;     // elastic: factors of the levels in the predictors' integer form
+  int nfx = 0;
   double* fmat = nullptr;    // elastic: per-face material terms of the Riemann solver
   double* fspeed = nullptr;  // mixed Euler: face wave speeds evaluated by the predictor
   double* mat = nullptr;
@@ -532,6 +563,7 @@ static void free_all(ader_ctx* c) {
   cudaFree(c->phi);
   cudaFree(c->fmat);
   cudaFree(c->lin);
+  cudaFree(c->rfx);
   cudaFree(c->hb_in);
   cudaFree(c->hb_out);
   if (c->hb_cin) cudaStreamDestroy(c->hb_cin);
@@ -680,6 +712,7 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
   build_tables_f(cfg->order, c->tab, c->tabf);
   for (int d = 0; d < 3; ++d) split_f(c->g.inv_h[d], c->tabf.ihh[d], c->tabf.ihl[d]);
   build_tables_x(cfg->order, cfg->dim, c->tab, c->g, c->tabf.x);
+  build_tables_e(cfg->order, c->tab, c->tabf.el);
   split_f(c->p.gamma - 1.0, c->tabf.g1h, c->tabf.g1l);
   const int n = cfg->order + 1;
   c->nodes = 1;
@@ -701,6 +734,9 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
     e = cudaMalloc(&c->fspeed, ncells * cfg->dim * 2 * c->nf * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&c->dev, sizeof(DevScalars));
   if (e == cudaSuccess && cfg->pde == ADER_PDE_ELASTIC) e = cudaMalloc(&c->mat, ncells * 3 * sizeof(double));
+  std::vector<double> rfx;  // ratios of the levels' weights
+  if (cfg->pde == ADER_PDE_ELASTIC && cfg->predictor == ADER_PREDICTOR_CK)
+    for (int k = 0; k < cfg->order; ++k) rfx.push_back(1.0 / (k + 2));
   if (e == cudaSuccess && cfg->pde == ADER_PDE_ELASTIC && cfg->predictor == ADER_PREDICTOR_PICARD) {
     // (a host allocation that fails for an absurd number of iterations is ADER_ENOMEM)
     try {
@@ -713,9 +749,21 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
         e = cudaMemcpyAsync(c->lin, lv.data(), lv.size() * sizeof(double), cudaMemcpyHostToDevice,
                             c->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+      for (int k = 0; k < c->nlev && c->nlev <= fxe_levels(cfg->order); ++k)
+        rfx.push_back(lv[k + 1] / lv[k] * lv[c->nlev + 1 + k]);
     } catch (const std::exception&) {
       e = cudaErrorMemoryAllocation;
     }
+  }
+  bool shrink = !rfx.empty();  // no level outgrows the one before it by its factor
+  for (double r : rfx) shrink = shrink && std::fabs(r) <= 1.0;
+  if (e == cudaSuccess && shrink) {
+    c->nfx = (int)rfx.size();
+    rfx.push_back(1.0);
+    e = cudaMalloc(&c->rfx, rfx.size() * sizeof(double));
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(c->rfx, rfx.data(), rfx.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   }
   if (cfg->limiter) {
     const int ns = 2 * cfg->order + 1;
@@ -1054,6 +1102,8 @@ static StepArgs make_args(ader_ctx* c, double dt, double t_end) {
   a.fmat = c->mat_set ? c->fmat : nullptr;
   a.lin = c->lin;
   a.nlev = c->nlev;
+  a.rfx = c->rfx;
+  a.nfx = c->nfx;
   a.dev = c->dev;
   a.iters = c->cfg.picard_iters > 0 ? c->cfg.picard_iters : c->cfg.order + 1;
   a.cerk = c->cfg.initial_guess == ADER_GUESS_CERK ? 1 : 0;

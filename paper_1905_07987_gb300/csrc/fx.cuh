@@ -57,20 +57,30 @@ __device__ __forceinline__ long long fx_mul(fx2 a, fx2 b) {
   return (long long)a.h * b.h + (int)(c >> 32);
 }
 
-// sum_m X[m] T[m] / 2^(64 - SH) for a table row T of n entries (h, l).  LL: with the low words'
-// products (the input's without its last four bits, so that their sum fits).
-template <int n, int SH, bool LL = true>
-__device__ __forceinline__ long long fx_dot(const fx2 (&X)[n], const fx2* T) {
-  long long s1 = 0, s0 = 1ll << (31 - SH), sl = 0;
-#pragma unroll
-  for (int m = 0; m < n; ++m) {
-    s1 += (long long)X[m].h * T[m].h;
-    s0 += (long long)X[m].h * T[m].l;
-    s0 += (long long)X[m].l * T[m].h;
-    if (LL) sl += (long long)(X[m].l >> 4) * T[m].l;
+// Sum of products, sum X T / 2^(64 - SH).  LL: with the low words' products, to 2^-16 of the last place
+// of the high sum, as products of their upper halves.
+template <int SH, bool LL = true>
+struct FxAcc {
+  long long s1 = 0, s0 = 1ll << (31 - SH);
+  __device__ __forceinline__ void mac(fx2 x, fx3 t) {
+    s1 += (long long)x.h * t.h;
+    s0 += (long long)x.h * t.l;
+    s0 += (long long)x.l * t.h;
+    if (LL) s0 += (long long)(x.l >> 16) * t.q;
   }
-  if (LL) s0 += sl >> 28;
-  return SH ? (s1 << SH) + (s0 >> (32 - SH)) : s1 + (int)(s0 >> 32);
+  __device__ __forceinline__ long long get() const {
+    const long long t = s1 + (int)(s0 >> 32);
+    return SH ? (long long)(((unsigned long long)t << SH) | ((unsigned)s0 >> (32 - SH))) : t;
+  }
+};
+
+// The same for a table row T of n entries.
+template <int n, int SH, bool LL = true>
+__device__ __forceinline__ long long fx_dot(const fx2 (&X)[n], const fx3* T) {
+  FxAcc<SH, LL> a;
+#pragma unroll
+  for (int m = 0; m < n; ++m) a.mac(X[m], T[m]);
+  return a.get();
 }
 
 }  // namespace ader

@@ -344,28 +344,6 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
   }
 }
 
-template <int N, bool PIC>
-__global__ void __launch_bounds__(CfgCK<N>::TPB) k_predictor_ck(const __grid_constant__ StepArgs A,
-                                                               const __grid_constant__ Tables T) {
-  predictor_ck_block<N, PIC>(A, T, (long long)blockIdx.x * CfgCK<N>::CPB);
-}
-
-template <int N, bool PIC>
-cudaError_t launch_predictor_ck_n(const StepArgs& a, const Tables& t, cudaStream_t s) {
-  using C = CfgCK<N>;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_predictor_ck<N, PIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
-  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_predictor_ck<N, PIC><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t);
-  return cudaGetLastError();
-}
-
 // ---- mixed precision --------------------------------------------------------------------------
 
 template <int N>

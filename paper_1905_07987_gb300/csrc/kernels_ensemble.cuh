@@ -7,7 +7,7 @@
 // large ones inside one launch.  No block waits for another.
 #pragma once
 #include "kernels.cuh"
-#include "kernels_ck.cuh"
+#include "kernels_ck_fx.cuh"
 #include "step_scalars.cuh"
 
 namespace ader {
@@ -25,10 +25,10 @@ __device__ __forceinline__ int ens_find(const long long* off, int nr, long long 
 
 template <int N, bool MIXED>
 struct EnsCfg {
-  static constexpr int TPB = MIXED ? CfgCKM<N>::TPB : CfgCK<N>::TPB;
-  static constexpr int MINB = MIXED ? CfgCKM<N>::MINB : 1;
-  static constexpr int CPB = MIXED ? CfgCKM<N>::CPB : CfgCK<N>::CPB;
-  static constexpr size_t SMEM = MIXED ? CfgCKM<N>::SMEM : CfgCK<N>::SMEM;
+  static constexpr int TPB = MIXED ? CfgCKM<N>::TPB : CfgE<N>::TPB;
+  static constexpr int MINB = MIXED ? CfgCKM<N>::MINB : CfgE<N>::MINB;
+  static constexpr int CPB = MIXED ? CfgCKM<N>::CPB : CfgE<N>::CPB;
+  static constexpr size_t SMEM = MIXED ? CfgCKM<N>::SMEM : CfgE<N>::SMEM;
   static_assert(CPB == ck_cells_per_block(N), "the host counts the blocks of each run");
 };
 
@@ -40,7 +40,7 @@ __device__ __forceinline__ void ens_predictor_block(const StepArgs* R, const Ens
   const int r = ens_find(E.blk0, E.nr, it);
   const long long c0 = (it - E.blk0[r]) * EnsCfg<N, MIXED>::CPB;
   if constexpr (MIXED) predictor_ck_mixed_block<N, PIC>(R[r], T, F, c0);
-  else predictor_ck_block<N, PIC>(R[r], T, c0);
+  else predictor_elastic_block<N, PIC>(R[r], T, F.el, c0);
   __syncthreads();  // the next block of cells reuses the shared memory
 }
 

@@ -1,6 +1,6 @@
 // Picard predictor of the 3-D elastic family, orders 1-6, FP64 and mixed precision: the linear
 // system's iterates in their polynomial form (kernels_ck.cuh).
-#include "kernels_ck.cuh"
+#include "kernels_ck_fx.cuh"
 
 namespace ader {
 
@@ -19,12 +19,12 @@ cudaError_t predictor_picard_elastic3(const StepArgs& a, const Tables& t, const 
     return cudaErrorInvalidValue;
   }
   switch (a.g.order) {
-    case 1: return launch_predictor_ck_n<1, true>(a, t, s);
-    case 2: return launch_predictor_ck_n<2, true>(a, t, s);
-    case 3: return launch_predictor_ck_n<3, true>(a, t, s);
-    case 4: return launch_predictor_ck_n<4, true>(a, t, s);
-    case 5: return launch_predictor_ck_n<5, true>(a, t, s);
-    case 6: return launch_predictor_ck_n<6, true>(a, t, s);
+    case 1: return launch_predictor_elastic_n<1, true>(a, t, f, s);
+    case 2: return launch_predictor_elastic_n<2, true>(a, t, f, s);
+    case 3: return launch_predictor_elastic_n<3, true>(a, t, f, s);
+    case 4: return launch_predictor_elastic_n<4, true>(a, t, f, s);
+    case 5: return launch_predictor_elastic_n<5, true>(a, t, f, s);
+    case 6: return launch_predictor_elastic_n<6, true>(a, t, f, s);
   }
   return cudaErrorInvalidValue;
 }
