@@ -30,6 +30,7 @@ struct DevScalars {
   long long seismo_row;      // next seismogram row
   int n_troubled;            // troubled cells of the last step
   int fv_retry;              // limiter: a MUSCL-Hancock recompute of this step was inadmissible
+  unsigned cfl_blocks;       // blocks of the CFL kernel that have finished (wraps to 0)
 };
 
 // 1-D reference-element tables, passed by value as a kernel parameter (constant bank).
@@ -237,6 +238,8 @@ struct StepArgs {
   // levels: the form does not apply)
   const double* rfx;
   int nfx;
+  // 1: the corrector advances the time (no receivers read the step's row after it)
+  int advance;
   // hybrid limiter: the cells with FV steps left (nonzero) skip the predictor; their face
   // neighbours compute with FV too, so nothing kept reads their DG data (null: every cell)
   const uint8_t* skip;

@@ -1143,12 +1143,13 @@ static ader_status step_impl(ader_ctx* c, double dt, double t_end) {
   a.fspeed = c->fspeed;  // mixed Euler step: face speeds evaluated by the predictor
   // the filtered CFL maximum pays off from ~2^18 nodes; below, the plain FP64 pass has less latency
   a.cfl_filter = (c->cfg.pde == ADER_PDE_EULER && c->g.ncells * c->nodes >= (1LL << 18)) ? 1 : 0;
+  a.advance = c->rec.nrec > 0 ? 0 : 1;
   cudaStream_t s = c->stream;
   ader_status st;
   if ((st = mark(c, 0)) != ADER_OK) return st;
-  if (!(dt > 0)) CUDA_OK(c->fam->cfl(a, s));
+  if (!(dt > 0)) CUDA_OK(c->fam->cfl(a, s));  // forms dt too
   if ((st = mark(c, 1)) != ADER_OK) return st;
-  CUDA_OK(launch_dt_finalize(a, s));
+  if (dt > 0) CUDA_OK(launch_dt_finalize(a, s));
   if ((st = mark(c, 2)) != ADER_OK) return st;
   if (c->cfg.predictor == ADER_PREDICTOR_CK) {
     CUDA_OK(c->fam->predictor_ck(a, c->tab, c->tabf, c->cfg.precision, s));
@@ -1175,8 +1176,10 @@ static ader_status step_impl(ader_ctx* c, double dt, double t_end) {
     std::swap(c->mm, c->mm_new);
   }
   if ((st = mark(c, 6)) != ADER_OK) return st;
-  if (c->rec.nrec > 0) CUDA_OK(launch_receivers(a, c->rec, (int)c->nodes, (int)c->nvar, s));
-  CUDA_OK(launch_advance_rec(a, c->rec.nrec > 0, s));
+  if (c->rec.nrec > 0) {
+    CUDA_OK(launch_receivers(a, c->rec, (int)c->nodes, (int)c->nvar, s));
+    CUDA_OK(launch_advance_rec(a, 1, s));
+  }
   if ((st = mark(c, 7)) != ADER_OK) return st;
   if (c->timing) c->ev_used++;
   std::swap(c->u, c->u_next);

@@ -9,6 +9,7 @@
 #include <cstdio>
 #include "ader_internal.h"
 #include "pde.cuh"
+#include "step_scalars.cuh"
 
 namespace ader {
 
@@ -705,13 +706,30 @@ __device__ __forceinline__ void riemann_face(const StepArgs& A, const Tables& T,
   }
 }
 
+// Blocks of the Riemann solver: the directions one after the other in one launch (a step of a small
+// grid is a chain of launches: 27^2 cells, 48 steps in a graph, see launch_riemann_n).
+struct FaceBlocks {
+  unsigned end[3];       // first block after direction d's
+  long long off[3];      // offset of direction d's fluxes
+  __device__ __forceinline__ int dir(unsigned b, unsigned& first) const {
+    const int d = b < end[0] ? 0 : (b < end[1] ? 1 : 2);
+    first = d == 0 ? 0u : end[d - 1];
+    return d;
+  }
+};
+
 // One warp per face (all lanes of the warp take part).
 template <class P, int D, int N>
 __global__ void __launch_bounds__(128) k_riemann(const __grid_constant__ StepArgs A,
-                                                 const __grid_constant__ Tables T, int d,
-                                                 long long phi_off) {
-  riemann_face<P, D, N>(A, T, d, phi_off, (long long)blockIdx.x * 4 + (threadIdx.x >> 5),
-                        threadIdx.x & 31);
+                                                 const __grid_constant__ Tables T,
+                                                 const __grid_constant__ FaceBlocks B) {
+  unsigned first;
+  const int d = B.dir(blockIdx.x, first);
+  const long long f = (long long)(blockIdx.x - first) * 4 + (threadIdx.x >> 5);
+  // a compile-time direction in each branch
+  if (d == 0) riemann_face<P, D, N>(A, T, 0, B.off[0], f, threadIdx.x & 31);
+  if (d == 1) riemann_face<P, D, N>(A, T, 1, B.off[1], f, threadIdx.x & 31);
+  if (D == 3 && d == 2) riemann_face<P, D, N>(A, T, 2, B.off[2], f, threadIdx.x & 31);
 }
 
 // Faces with few nodes (NF <= 16): FPW faces per warp, one lane per (face, node), so that the
@@ -727,10 +745,9 @@ struct RiemannPack {
   static constexpr bool USE = P::CONS && !P::LINEAR && !P::NCP && FPW >= 2;
 };
 
-template <class P, int D, int N>
-__global__ void __launch_bounds__(128) k_riemann_packed(const __grid_constant__ StepArgs A,
-                                                        const __grid_constant__ Tables T, int d,
-                                                        long long phi_off) {
+template <class P, int D, int N, int d>
+__device__ __forceinline__ void riemann_packed(const StepArgs& A, const Tables& T, unsigned block,
+                                               long long phi_off) {
   using C = Cfg<P, D, N>;
   constexpr int NV = C::NV, NF = C::NF, FR = C::FR, NPHI = C::NPHI;
   constexpr int FPW = RiemannPack<P, D, N>::FPW;
@@ -739,7 +756,7 @@ __global__ void __launch_bounds__(128) k_riemann_packed(const __grid_constant__ 
   const Geometry& g = A.g;
   const int nd = g.n[d];
   const long long nfaces = (long long)(nd + 1) * FaceIdx::ntrans(g, d);
-  const long long f = ((long long)blockIdx.x * 4 + (threadIdx.x >> 5)) * FPW + slot;
+  const long long f = ((long long)block * 4 + (threadIdx.x >> 5)) * FPW + slot;
   const bool periodic = (g.bc[d][0] == BC_PERIODIC);
   bool on = slot < FPW && f < nfaces;
   int kf = 0;
@@ -768,14 +785,9 @@ __global__ void __launch_bounds__(128) k_riemann_packed(const __grid_constant__ 
       FL[v] = a[NF * NV + jp * NV + v];
       FRv[v] = b[NF * NV + jp * NV + v];
     }
-    // ghost states and speeds with a compile-time direction (the states stay in registers)
-#pragma unroll
-    for (int dd = 0; dd < D; ++dd) {
-      if (dd != d) continue;
-      if (!recL) ghost<P>(g.bc[dd][0], dd, qL, FL);
-      if (!recR) ghost<P>(g.bc[dd][1], dd, qR, FRv);
-      sp = fmax(P::speed(qL, A.p, dd), P::speed(qR, A.p, dd));
-    }
+    if (!recL) ghost<P>(g.bc[d][0], d, qL, FL);
+    if (!recR) ghost<P>(g.bc[d][1], d, qR, FRv);
+    sp = fmax(P::speed(qL, A.p, d), P::speed(qR, A.p, d));
   }
   // the face's speed: the maximum over its NF lanes (every lane takes part in the shuffles)
   double s = 0.0;
@@ -804,6 +816,22 @@ __global__ void __launch_bounds__(128) k_riemann_packed(const __grid_constant__ 
     }
   }
 }
+
+template <class P, int D, int N>
+__global__ void __launch_bounds__(128) k_riemann_packed(const __grid_constant__ StepArgs A,
+                                                        const __grid_constant__ Tables T,
+                                                        const __grid_constant__ FaceBlocks B) {
+  unsigned first;
+  const int d = B.dir(blockIdx.x, first);
+  if (d == 0) riemann_packed<P, D, N, 0>(A, T, blockIdx.x - first, B.off[0]);
+  if (d == 1) riemann_packed<P, D, N, 1>(A, T, blockIdx.x - first, B.off[1]);
+  if constexpr (D == 3)
+    if (d == 2) riemann_packed<P, D, N, 2>(A, T, blockIdx.x - first, B.off[2]);
+}
+
+// The time advance as a call: inlined, its FP64 addition would be issued, predicated off, by every
+// warp of the corrector (a seventh of its FP64 work).
+static __device__ __noinline__ void advance_call(DevScalars* s) { advance_one(s, 0); }
 
 // Corrector, face part of Eq. (6) in strong form:
 //   u_j -= dt sum_d [ (e1_{j_d}/(w_{j_d} h_d)) Phi_L(right face) - (e0_{j_d}/(w_{j_d} h_d)) Phi_R(left face) ]
@@ -861,12 +889,14 @@ __global__ void __launch_bounds__(256) k_corrector(const __grid_constant__ StepA
     sw[k][d][m] = A.dev->dt * (k ? A.cw1[d][m] : A.cw0[d][m]);
   }
   __syncthreads();
+  // no kernel of the step reads the time after the predictor: the advance needs no launch of its own
+  if (A.advance && blockIdx.x == 0 && threadIdx.x == 0) advance_call(A.dev);
   const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
   if (e >= A.g.ncells * C::NL) return;
   corrector_dof<P, D, N>(A, sw, off1, off2, e);
 }
 
-// Max signal speed of the state (Eq. (7)); NaN / Inf latches ST_NONFINITE.  Euler: one FP64
+// Max signal speed of the state and the time step (Eq. (7)); NaN / Inf latches ST_NONFINITE.  Euler: one FP64
 // division and one square root per node for all directions, on the nodes that the binary32
 // enclosures cannot rule out.
 template <class P, int D, int N>
@@ -1002,6 +1032,13 @@ __global__ void __launch_bounds__(256) k_cfl(const __grid_constant__ StepArgs A)
   if ((threadIdx.x & 31) == 0) {
     atomicMax(&A.dev->lam_bits, (unsigned long long)__double_as_longlong(lmax));
     if (bad) atomicOr(&A.dev->status, ST_NONFINITE);
+    __threadfence();
+  }
+  // the last block to finish forms dt from the maximum (the counter wraps to 0)
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicInc(&A.dev->cfl_blocks, gridDim.x - 1) == gridDim.x - 1) {
+    __threadfence();
+    dt_finalize_one(A);
   }
 }
 
@@ -1009,26 +1046,26 @@ __global__ void __launch_bounds__(256) k_cfl(const __grid_constant__ StepArgs A)
 template <class P, int D, int N>
 cudaError_t launch_riemann_n(const StepArgs& a, const Tables& t, cudaStream_t s) {
   using C = Cfg<P, D, N>;
-  long long off = 0;
+  const bool packed = RiemannPack<P, D, N>::USE && !a.fspeed;
+  const int fpb = packed ? 4 * RiemannPack<P, D, N>::FPW : 4;  // faces per block
+  FaceBlocks B{};
+  long long off = 0, blocks = 0;
   for (int d = 0; d < D; ++d) {
     const long long nf = (long long)(a.g.n[d] + 1) * (a.g.ncells / a.g.n[d]);
-    if constexpr (RiemannPack<P, D, N>::USE) {
-      if (!a.fspeed) {
-        constexpr int FPB = 4 * RiemannPack<P, D, N>::FPW;  // faces per block
-        k_riemann_packed<P, D, N><<<(unsigned)((nf + FPB - 1) / FPB), 128, 0, s>>>(a, t, d, off);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        off += nf * (long long)(C::NPHI * C::NF * C::NV);
-        continue;
-      }
-    }
-    const long long blocks = (nf + 3) / 4;
-    k_riemann<P, D, N><<<(unsigned)blocks, 128, 0, s>>>(a, t, d, off);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    blocks += (nf + fpb - 1) / fpb;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    B.end[d] = (unsigned)blocks;
+    B.off[d] = off;
     off += nf * (long long)(C::NPHI * C::NF * C::NV);
   }
-  return cudaSuccess;
+  if constexpr (RiemannPack<P, D, N>::USE) {
+    if (packed) {
+      k_riemann_packed<P, D, N><<<(unsigned)blocks, 128, 0, s>>>(a, t, B);
+      return cudaGetLastError();
+    }
+  }
+  k_riemann<P, D, N><<<(unsigned)blocks, 128, 0, s>>>(a, t, B);
+  return cudaGetLastError();
 }
 
 template <class P, int D, int N>
@@ -1047,7 +1084,11 @@ cudaError_t launch_corrector_n(const StepArgs& a, const Tables& t, cudaStream_t 
 
 template <class P, int D, int N>
 cudaError_t launch_cfl_n(const StepArgs& a, cudaStream_t s) {
-  k_cfl<P, D, N><<<152 * 8, 256, 0, s>>>(a);
+  using C = Cfg<P, D, N>;
+  // as many blocks as have a node (a cell, for the elastic material) each, up to 8 per SM
+  const long long items = P::NCP ? a.g.ncells : a.g.ncells * C::NS;
+  const long long want = (items + 255) / 256;
+  k_cfl<P, D, N><<<(unsigned)(want < 152 * 8 ? want : 152 * 8), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

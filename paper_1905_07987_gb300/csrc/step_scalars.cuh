@@ -1,5 +1,6 @@
-// Device-side time-step scalars shared by the per-context kernels (common.cu) and the ensemble's
-// persistent launches: the time-step finalisation of Eq. (7) and the time advance.
+// Device-side time-step scalars shared by the per-context kernels (the CFL kernel's last block, the
+// corrector; common.cu when the step is fixed or receivers record it) and the ensemble's persistent
+// launches: the time-step finalisation of Eq. (7) and the time advance.
 #pragma once
 #include "ader_internal.h"
 
@@ -12,7 +13,7 @@ __device__ __forceinline__ void dt_finalize_one(const StepArgs& A) {
   if (A.dt_fixed > 0.0) {
     dt = A.dt_fixed;
   } else {
-    const double lam = __longlong_as_double((long long)s->lam_bits);
+    const double lam = __longlong_as_double((long long)*(volatile unsigned long long*)&s->lam_bits);
     double hmin = A.g.h[0];
     for (int d = 1; d < A.g.dim; ++d) hmin = fmin(hmin, A.g.h[d]);
     dt = A.cfl / (double)(A.g.dim * (2 * A.g.order + 1)) * hmin / lam;
