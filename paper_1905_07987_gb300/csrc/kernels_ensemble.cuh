@@ -67,21 +67,15 @@ __global__ void __launch_bounds__(128) k_ens_riemann(const StepArgs* __restrict_
 }
 
 template <class P, int D, int N>
-__global__ void __launch_bounds__(256) k_ens_corrector(const StepArgs* __restrict__ R,
-                                                       const __grid_constant__ EnsTable E) {
-  constexpr int n = N + 1, NL = Cfg<P, D, N>::NL;
-  // dt e0 / (w h_d), dt e1 / (w h_d) of every run
-  __shared__ double sw[ENS_MAXR][2][3][n];
-  for (int i = threadIdx.x; i < E.nr * 2 * D * n; i += blockDim.x) {
-    const int r = i / (2 * D * n), k = (i / (D * n)) % 2, d = (i / n) % D, m = i % n;
-    sw[r][k][d][m] = R[r].dev->dt * (k ? R[r].cw1[d][m] : R[r].cw0[d][m]);
-  }
-  __syncthreads();
-  const long long total = E.cell0[E.nr] * NL;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int r = ens_find(E.cell0, E.nr, e / NL);
-    corrector_dof<P, D, N>(R[r], sw[r], E.phioff[1][r], E.phioff[2][r], e - E.cell0[r] * NL);
+__global__ void __launch_bounds__(CfgC<P, D, N>::TPB) k_ens_corrector(const StepArgs* __restrict__ R,
+                                                                     const __grid_constant__ EnsTable E) {
+  using X = CfgC<P, D, N>;
+  __shared__ SmemC<P, D, N, 1> S;
+  for (long long c = blockIdx.x; c < E.cell0[E.nr]; c += gridDim.x) {
+    const int r = ens_find(E.cell0, E.nr, c);
+    const int Ew = corrector_weights<D, N + 1>(R[r], S.w, threadIdx.x);
+    corrector_cells<P, D, N, 1, X::TPB>(R[r], S, Ew, E.phioff[1][r], E.phioff[2][r], c - E.cell0[r], 1,
+                                        threadIdx.x);
   }
 }
 
@@ -108,7 +102,7 @@ cudaError_t ens_step_n(const StepArgs* R, const EnsTable& E, const Tables& T, co
     k_ens_riemann<Elastic, 3, N><<<152 * 16, 128, 0, s>>>(R, E, T, d);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_ens_corrector<Elastic, 3, N><<<152 * 8, 256, 0, s>>>(R, E);
+  k_ens_corrector<Elastic, 3, N><<<152 * 8, CfgC<Elastic, 3, N>::TPB, 0, s>>>(R, E);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_ens_advance(R, E.nr, s);
 }
@@ -165,8 +159,7 @@ __global__ void __launch_bounds__(EnsCfg<N, MIXED>::TPB, EnsCfg<N, MIXED>::MINB)
                 GridBar* bar, long long limit) {
   using P = Elastic;
   constexpr int D = 3;
-  using C = Cfg<P, D, N>;
-  constexpr int n = N + 1, NL = C::NL, TPB = EnsCfg<N, MIXED>::TPB;
+  constexpr int n = N + 1, TPB = EnsCfg<N, MIXED>::TPB;
   extern __shared__ __align__(16) double fsm[];
   const unsigned nb = gridDim.x;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -192,17 +185,13 @@ __global__ void __launch_bounds__(EnsCfg<N, MIXED>::TPB, EnsCfg<N, MIXED>::MINB)
     }
     if (!(ok = grid_sync(bar, nb, limit))) break;
     {
-      // dt e0 / (w h_d), dt e1 / (w h_d) of every run, over the predictor's shared memory
-      double (*sw)[2][3][n] = reinterpret_cast<double (*)[2][3][n]>(fsm);
-      for (int i = threadIdx.x; i < E.nr * 2 * D * n; i += TPB) {
-        const int r = i / (2 * D * n), k = (i / (D * n)) % 2, d = (i / n) % D, m = i % n;
-        sw[r][k][d][m] = R[r].dev->dt * (k ? R[r].cw1[d][m] : R[r].cw0[d][m]);
-      }
-      __syncthreads();
-      const long long total = ncell * NL;
-      for (long long e = (long long)blockIdx.x * TPB + threadIdx.x; e < total; e += (long long)nb * TPB) {
-        const int r = ens_find(E.cell0, E.nr, e / NL);
-        corrector_dof<P, D, N>(R[r], sw[r], E.phioff[1][r], E.phioff[2][r], e - E.cell0[r] * NL);
+      // over the predictor's shared memory
+      SmemC<P, D, N, 1>& S = *reinterpret_cast<SmemC<P, D, N, 1>*>(fsm);
+      for (long long c = blockIdx.x; c < ncell; c += nb) {
+        const int r = ens_find(E.cell0, E.nr, c);
+        const int Ew = corrector_weights<D, n>(R[r], S.w, threadIdx.x);
+        corrector_cells<P, D, N, 1, TPB>(R[r], S, Ew, E.phioff[1][r], E.phioff[2][r], c - E.cell0[r], 1,
+                                         threadIdx.x);
       }
     }
     if (!(ok = grid_sync(bar, nb, limit))) break;
@@ -219,8 +208,8 @@ cudaError_t ens_fused_n(const StepArgs* R, const EnsTable& E, const Tables& T, c
                         int steps, GridBar* bar, long long limit, int blocks_per_sm,
                         cudaStream_t s) {
   using G = EnsCfg<N, MIXED>;
-  constexpr size_t SW = (size_t)ENS_MAXR * 2 * 3 * (N + 1) * sizeof(double);
-  constexpr size_t SMEM = G::SMEM > SW ? G::SMEM : SW;
+  constexpr size_t SC = sizeof(SmemC<Elastic, 3, N, 1>);  // the corrector's
+  constexpr size_t SMEM = G::SMEM > SC ? G::SMEM : SC;
   static int max_bps = 0;
   if (!max_bps) {
     cudaError_t e = cudaFuncSetAttribute(k_ens_fused<N, MIXED>,
