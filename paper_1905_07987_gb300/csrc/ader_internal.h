@@ -83,6 +83,8 @@ struct TablesE {
   fx3 od[MAXN / 2][MAXN / 2 + 1];
   fx3 mid[MAXN / 2];
   fx3 e[2][MAXN];
+  // the same derivative as binary32 (hi, lo) pairs, for the mixed form's levels
+  float2 evf[MAXN / 2][MAXN / 2], odf[MAXN / 2][MAXN / 2 + 1], midf[MAXN / 2];
   int kc;                                   // material coefficients are x 2^kc
   int ke;                                   // face values: r 2^(E + ke)
 };

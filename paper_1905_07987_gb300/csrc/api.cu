@@ -288,9 +288,16 @@ void build_tables_e(int order, const Tables& T, TablesE& X) {
   const int p = fx_scale(2 * H + 1, H + 1, P[0], MAXN);
   const int pe = std::min(fx_scale(1, n, T.e0, MAXN), fx_scale(1, n, T.e1, MAXN));
   for (int i = 0; i < H; ++i) {
-    for (int m = 0; m < H; ++m) X.ev[i][m] = fx_entry(P[i][m], p);
-    for (int m = 0; m <= H; ++m) X.od[i][m] = fx_entry(P[H + i][m], p);
+    for (int m = 0; m < H; ++m) {
+      X.ev[i][m] = fx_entry(P[i][m], p);
+      split_f(P[i][m], X.evf[i][m].x, X.evf[i][m].y);
+    }
+    for (int m = 0; m <= H; ++m) {
+      X.od[i][m] = fx_entry(P[H + i][m], p);
+      split_f(P[H + i][m], X.odf[i][m].x, X.odf[i][m].y);
+    }
     X.mid[i] = fx_entry(P[2 * H][i], p);
+    split_f(P[2 * H][i], X.midf[i].x, X.midf[i].y);
   }
   for (int i = 0; i < n; ++i) {
     X.e[0][i] = fx_entry(T.e0[i], pe);

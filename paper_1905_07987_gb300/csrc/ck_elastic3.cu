@@ -11,12 +11,12 @@ cudaError_t predictor_ck_elastic3(const StepArgs& a, const Tables& t, const Tabl
   if (prec == 3) return predictor_ck_tc_elastic3(a, t, s);
   if (prec == 1) {
     switch (a.g.order) {
-      case 1: return launch_predictor_ck_mixed_n<1, false>(a, t, f, s);
-      case 2: return launch_predictor_ck_mixed_n<2, false>(a, t, f, s);
-      case 3: return launch_predictor_ck_mixed_n<3, false>(a, t, f, s);
-      case 4: return launch_predictor_ck_mixed_n<4, false>(a, t, f, s);
-      case 5: return launch_predictor_ck_mixed_n<5, false>(a, t, f, s);
-      case 6: return launch_predictor_ck_mixed_n<6, false>(a, t, f, s);
+      case 1: return launch_predictor_elastic_mixed_n<1, false>(a, t, f, s);
+      case 2: return launch_predictor_elastic_mixed_n<2, false>(a, t, f, s);
+      case 3: return launch_predictor_elastic_mixed_n<3, false>(a, t, f, s);
+      case 4: return launch_predictor_elastic_mixed_n<4, false>(a, t, f, s);
+      case 5: return launch_predictor_elastic_mixed_n<5, false>(a, t, f, s);
+      case 6: return launch_predictor_elastic_mixed_n<6, false>(a, t, f, s);
     }
     return cudaErrorInvalidValue;
   }

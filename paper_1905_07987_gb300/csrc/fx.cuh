@@ -45,6 +45,16 @@ __device__ __forceinline__ double fx_out(long long r, int k) {
   return __longlong_as_double(z ? 0ll : (long long)(b | (g & 0x8000000000000000ull)));
 }
 
+// To and from binary32 by 32-bit conversions (the 64-bit ones run at the FP64 pipe's rate): r within
+// a few units of binary32's last place or 2^8, |x| < 2^62 within one.
+__device__ __forceinline__ float fx_float(long long r) {
+  return fmaf((float)(int)(r >> 32), 4294967296.0f, (float)(unsigned)r);
+}
+__device__ __forceinline__ long long fx_from_float(float x) {
+  const float h = rintf(x * 0x1p-32f);
+  return ((long long)(int)h << 32) + (long long)(int)fmaf(h, -4294967296.0f, x);
+}
+
 // The two words of X: X = h 2^32 + l.
 __device__ __forceinline__ fx2 fx_split(long long X) {
   const unsigned l = (unsigned)X;

@@ -729,28 +729,4 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
   }
 }
 
-template <int N, bool PIC>
-__global__ void __launch_bounds__(CfgCKM<N>::TPB, CfgCKM<N>::MINB)
-    k_predictor_ck_mixed(const __grid_constant__ StepArgs A, const __grid_constant__ Tables T,
-                         const __grid_constant__ TablesF F) {
-  predictor_ck_mixed_block<N, PIC>(A, T, F, (long long)blockIdx.x * CfgCKM<N>::CPB);
-}
-
-template <int N, bool PIC>
-cudaError_t launch_predictor_ck_mixed_n(const StepArgs& a, const Tables& t, const TablesF& f,
-                                        cudaStream_t s) {
-  using C = CfgCKM<N>;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(
-        k_predictor_ck_mixed<N, PIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
-  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
-  k_predictor_ck_mixed<N, PIC><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t, f);
-  return cudaGetLastError();
-}
-
 }  // namespace ader

@@ -65,21 +65,48 @@ __device__ __forceinline__ void fx_octet(long long (&x)[8]) {
       }
 }
 
+// The lines of thread j of a cell, the same in every level: place of the first node in the level (12
+// bits) and in the derivatives (13 bits) and the direction; -1: none.  Line id: q = 6 d + i (direction,
+// i-th of its six variables: the velocities, then sigma_{0d}, sigma_{1d}, sigma_{2d}).
+template <int N>
+struct FxeLines {
+  using C = CfgE<N>;
+  static constexpr int RND = (18 * C::NF + C::NS - 1) / C::NS;
+  int t[RND];
+  __device__ __forceinline__ explicit FxeLines(int j) {
+    constexpr int n = C::n, NF = C::NF;
+#pragma unroll
+    for (int k = 0; k < RND; ++k) {
+      const int id = j + k * C::NS, q = id / NF;
+      const int ln = id - q * NF, d = q / 6, i = q - d * 6, b = i - 3;
+      const int v = i < 3 ? i : (b == d ? 3 + d : 5 + b + d);
+      const int j0 = d == 0 ? ln * n : (d == 1 ? ln % n + (ln / n) * n * n : ln);
+      t[k] = id < 18 * NF ? (v * C::NSP + j0) | (q * C::NSP + j0) << 12 | d << 25 : -1;
+    }
+  }
+  // line k: places and stride
+  __device__ __forceinline__ bool get(int k, int& x, int& g, int& st) const {
+    constexpr int n = C::n;
+    x = t[k] & 0xfff;
+    g = (t[k] >> 12) & 0x1fff;
+    const int d = t[k] >> 25;
+    st = d == 0 ? 1 : (d == 1 ? n : n * n);
+    return t[k] >= 0;
+  }
+  static_assert(9 * C::NSP <= 4096 && 18 * C::NSP <= 8192, "places fit their bits");
+};
+
 // One application of r dt L to the level X: derivatives of every line into G.
 template <int N>
-__device__ __forceinline__ void fxe_lines(const TablesE& E, const fx2* X, fx2* G, int j) {
+__device__ __forceinline__ void fxe_lines(const TablesE& E, const fx2* X, fx2* G, const FxeLines<N>& L) {
   using C = CfgE<N>;
-  constexpr int n = C::n, NF = C::NF, NSP = C::NSP, H = C::H;
-  for (int id = j; id < 18 * NF; id += C::NS) {
-    const int q = id / NF, ln = id - q * NF;
-    const int d = q / 6, i = q - d * 6;
-    // variable of the line: the three velocities, then sigma_{0d}, sigma_{1d}, sigma_{2d}
-    const int b = i - 3;
-    const int v = i < 3 ? i : (b == d ? 3 + d : 5 + b + d);
-    const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
-    const int j0 = d == 0 ? ln * n : (d == 1 ? ln % n + (ln / n) * n * n : ln);
-    const fx2* x = X + v * NSP + j0;
-    fx2* g = G + q * NSP + j0;
+  constexpr int n = C::n, H = C::H;
+#pragma unroll
+  for (int r = 0; r < FxeLines<N>::RND; ++r) {
+    int px, pg, st;
+    if (!L.get(r, px, pg, st)) continue;
+    const fx2* x = X + px;
+    fx2* g = G + pg;
     fx2 a[n];
 #pragma unroll
     for (int m = 0; m < n; ++m) a[m] = x[m * st];
@@ -146,8 +173,77 @@ __device__ __forceinline__ void fxe_node(const fx2* G, const fx2* kc, int j, lon
   }
 }
 
-// The CPB cells from c0 (one block); false (for every thread) when the block needs the FP64 form.
-template <int N>
+// Binary32 derivatives of every line; LO: with the table's lo parts.
+template <int N, bool LO>
+__device__ __forceinline__ void fxe_lines_f(const TablesE& E, const float* X, float* G, const FxeLines<N>& L) {
+  using C = CfgE<N>;
+  constexpr int n = C::n, H = C::H;
+#pragma unroll
+  for (int r = 0; r < FxeLines<N>::RND; ++r) {
+    int px, pg, st;
+    if (!L.get(r, px, pg, st)) continue;
+    const float* x = X + px;
+    float* g = G + pg;
+    float a[n];
+#pragma unroll
+    for (int m = 0; m < n; ++m) a[m] = x[m * st];
+    const auto mac = [](float& h, float& l, float2 t, float y) {
+      h = fmaf(t.x, y, h);
+      if (LO) l = fmaf(t.y, y, l);
+    };
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      float ev = 0.f, od = 0.f, el = 0.f, ol = 0.f;
+#pragma unroll
+      for (int m = 0; m < H; ++m) {
+        mac(ev, el, E.evf[k][m], a[n - 1 - m]);
+        mac(od, ol, E.odf[k][m], a[m]);
+      }
+      if (C::ODD) mac(od, ol, E.odf[k][H], a[H]);
+      g[k * st] = LO ? ev + el : ev;
+      g[(n - 1 - k) * st] = LO ? od + ol : od;
+    }
+    if (C::ODD) {
+      float c = 0.f, cl = 0.f;
+#pragma unroll
+      for (int m = 0; m < H; ++m) mac(c, cl, E.midf[m], a[n - 1 - m]);
+      g[H * st] = LO ? c + cl : c;
+    }
+  }
+}
+
+// The material products in binary32 (k: dt times the coefficients as (hi, lo) pairs, r: the level's
+// factor).
+template <int N, bool LO>
+__device__ __forceinline__ void fxe_node_f(const float* G, const float2* k, float r, int j,
+                                           float (&out)[9]) {
+  constexpr int NSP = CfgE<N>::NSP;
+  const auto mac = [&](float& o, int c, float g) {
+    o = LO ? fmaf(k[c].x, g, fmaf(k[c].y, g, o)) : fmaf(k[c].x, g, o);
+  };
+  const auto g = [&](int d, int i) { return G[(d * 6 + i) * NSP + j]; };
+#pragma unroll
+  for (int i = 0; i < 9; ++i) out[i] = 0.f;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) mac(out[i], d * 4, g(d, 3 + i));
+    const float e = g(d, d);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) mac(out[3 + i], d * 4 + (i == d ? 1 : 2), e);
+#pragma unroll
+    for (int v = 6; v < 9; ++v) {
+      const int s = Elastic::src(d, v);
+      if (s >= 0) mac(out[v], d * 4 + 3, g(d, s));
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i) out[i] *= r;
+}
+
+// The CPB cells from c0 (one block); false (for every thread) when the block needs the other form.
+// MIXED: the levels after the first, of the size of the step squared and less, in binary32.
+template <int N, bool MIXED>
 __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const TablesE& E,
                                                      long long c0) {
   using C = CfgE<N>;
@@ -158,6 +254,7 @@ __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const Ta
   const long long sc = A.src.cell - c0;
   if (A.nfx <= 0 || (sc >= 0 && sc < ncb)) return false;
   __shared__ int s_e[CPB];
+  __shared__ float2 s_kf[MIXED ? CPB : 1][12];
   fx2(*s_k)[fxe_levels(N) + 1][12] =  // the levels' coefficients
       reinterpret_cast<fx2(*)[fxe_levels(N) + 1][12]>(reinterpret_cast<unsigned char*>(smem) + CPB * C::CELL);
   const int tid = threadIdx.x;
@@ -186,6 +283,10 @@ __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const Ta
       const int k = i / 12, q = i % 4, d = (i % 12) / 4;
       const double m = q == 0 ? s / rho : is * (q == 1 ? lam + 2.0 * mu : (q == 2 ? lam : mu));
       s_k[slot][k][i % 12] = fx_split(fx_in(dt * A.rfx[k] * A.g.inv_h[d] * m, 1082 - E.kc, over));
+      if (MIXED && k == K) {
+        const ff x = ff_split(dt * A.g.inv_h[d] * m);
+        s_kf[slot][i % 12] = make_float2(x.h, x.l);
+      }
     }
     // the cell's state, coalesced, and its largest exponent (stresses over 2^ez)
     int emax = 200;
@@ -228,9 +329,12 @@ __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const Ta
   long long S[NV];  // qbar: the sum of the levels at this node (parity index)
 #pragma unroll
   for (int v = 0; v < NV; ++v) S[v] = act ? fx_join(X[v * NSP + j]) : 0;
+  const FxeLines<N> L(j);
+  const int KI = MIXED ? 1 : K;  // levels in fixed point
+  float d32[MIXED ? NV : 1];     // the sum of the others
 #pragma unroll 1
-  for (int k = 0; k < K; ++k) {
-    if (act) fxe_lines<N>(E, X, G, j);
+  for (int k = 0; k < KI; ++k) {
+    if (act) fxe_lines<N>(E, X, G, L);
     __syncthreads();
     if (act) {
       long long b[NV];
@@ -238,10 +342,45 @@ __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const Ta
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         S[v] += b[v];
-        X[v * NSP + j] = fx_split(k == K - 1 ? S[v] : b[v]);
+        if constexpr (MIXED) {
+          d32[v] = 0.f;
+          if (K > 1) reinterpret_cast<float*>(X)[v * NSP + j] = fx_float(b[v]);
+          else X[v * NSP + j] = fx_split(S[v]);
+        } else {
+          X[v * NSP + j] = fx_split(k == K - 1 ? S[v] : b[v]);
+        }
       }
     }
     __syncthreads();
+  }
+  if constexpr (MIXED) {
+    float* Xf = reinterpret_cast<float*>(X);
+    float* Gf = reinterpret_cast<float*>(G);
+#pragma unroll 1
+    for (int k = 1; k < K; ++k) {
+      if (act) {
+        if (k == 1) fxe_lines_f<N, true>(E, Xf, Gf, L);
+        else fxe_lines_f<N, false>(E, Xf, Gf, L);
+      }
+      __syncthreads();
+      if (act) {
+        float b[NV];
+        if (k == 1) fxe_node_f<N, true>(Gf, s_kf[slot], (float)A.rfx[k], j, b);
+        else fxe_node_f<N, false>(Gf, s_kf[slot], (float)A.rfx[k], j, b);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          d32[v] += b[v];
+          if (k < K - 1) {
+            Xf[v * NSP + j] = b[v];
+          } else {
+            // (a sum outside the scale saturates and is caught with qbar)
+            S[v] += fx_from_float(fminf(fmaxf(d32[v], -0x1p61f), 0x1p61f));
+            X[v * NSP + j] = fx_split(S[v]);
+          }
+        }
+      }
+      __syncthreads();
+    }
   }
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
@@ -250,7 +389,7 @@ __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const Ta
   }
   // dt L qbar
   long long* W = reinterpret_cast<long long*>(G);  // [9][NSP]
-  if (act) fxe_lines<N>(E, X, G, j);
+  if (act) fxe_lines<N>(E, X, G, L);
   __syncthreads();
   {
     long long b[NV];
@@ -331,7 +470,72 @@ __device__ __noinline__ void predictor_ck_plain(const StepArgs& A, const Tables&
 template <int N, bool PIC>
 __device__ __forceinline__ void predictor_elastic_block(const StepArgs& A, const Tables& T,
                                                         const TablesE& E, long long c0) {
-  if (!predictor_elastic_fx<N>(A, E, c0)) predictor_ck_plain<N, PIC>(A, T, c0);
+  if (!predictor_elastic_fx<N, false>(A, E, c0)) predictor_ck_plain<N, PIC>(A, T, c0);
+}
+
+// The mixed predictor: u, the first level and the output in fixed point as above, the other levels in
+// binary32 (of the size of the step squared and less; the second level with float-float tables).
+// The node form (predictor_ck_mixed_block) keeps binary32 pairs for the first level and its FP64
+// pipe time is the base term, L qbar and the face values: 54 FP64 FMAs per node of order 5 per pass.
+//
+// The line: Picard from order 4, Cauchy-Kowalevski from order 5.  Predictor of a step, 64^3 cells, node form -> this one, ms.  Cauchy-
+// Kowalevski: order 5 16.46 -> 14.98, order 4 9.11 -> 9.09, order 3 3.88 -> 4.41, order 2 1.74 -> 2.38,
+// order 1 0.42 -> 0.56; order 6 at 48^3 17.35 -> 12.45.  Picard: order 5 21.33 -> 15.51, order 4 11.03
+// -> 9.36 (10^3 cells 0.0589 -> 0.0580), order 6 at 48^3 20.21 -> 12.90.  Below the conversion and the
+// change of basis cost what the FMAs that they save did, or more.  Warps: 24 an SM at order 4 (28:
+// 9.55, 21: 9.63), 28 above (24 and 21: 17.6 at order 5).  Error of a step against binary64: CK 5 to
+// 15 times less than the node form's, Picard 1.1 to 3 times.
+template <int N, bool PIC>
+struct CfgEM {
+  using C = CfgE<N>;
+  static constexpr bool FX = N >= (PIC ? 4 : 5);
+  static constexpr int TPB = C::TPB, CPB = C::CPB;
+  static constexpr int MINB = FX ? (N == 4 ? 768 : 896) / TPB : CfgCKM<N>::MINB;
+  static constexpr size_t SMEM =
+      FX && C::SMEM_X > CfgCKM<N>::SMEM ? C::SMEM_X : CfgCKM<N>::SMEM;
+  static_assert(TPB == CfgCKM<N>::TPB && CPB == CfgCKM<N>::CPB, "one launch shape for both forms");
+};
+
+// (not inlined: its registers do not add to the integer form's)
+template <int N, bool PIC>
+__device__ __noinline__ void predictor_ck_mixed_plain(const StepArgs& A, const Tables& T,
+                                                      const TablesF& F, long long c0) {
+  __syncthreads();
+  predictor_ck_mixed_block<N, PIC>(A, T, F, c0);
+}
+
+template <int N, bool PIC>
+__device__ __forceinline__ void predictor_elastic_mixed_block(const StepArgs& A, const Tables& T,
+                                                              const TablesF& F, long long c0) {
+  if constexpr (CfgEM<N, PIC>::FX) {
+    if (!predictor_elastic_fx<N, true>(A, F.el, c0)) predictor_ck_mixed_plain<N, PIC>(A, T, F, c0);
+  } else {
+    predictor_ck_mixed_block<N, PIC>(A, T, F, c0);
+  }
+}
+
+template <int N, bool PIC>
+__global__ void __launch_bounds__(CfgEM<N, PIC>::TPB, CfgEM<N, PIC>::MINB)
+    k_predictor_elastic_mixed(const __grid_constant__ StepArgs A, const __grid_constant__ Tables T,
+                              const __grid_constant__ TablesF F) {
+  predictor_elastic_mixed_block<N, PIC>(A, T, F, (long long)blockIdx.x * CfgEM<N, PIC>::CPB);
+}
+
+template <int N, bool PIC>
+cudaError_t launch_predictor_elastic_mixed_n(const StepArgs& a, const Tables& t, const TablesF& f,
+                                             cudaStream_t s) {
+  using C = CfgEM<N, PIC>;
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e = cudaFuncSetAttribute(
+        k_predictor_elastic_mixed<N, PIC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const long long blocks = (a.g.ncells + C::CPB - 1) / C::CPB;
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  k_predictor_elastic_mixed<N, PIC><<<(unsigned)blocks, C::TPB, C::SMEM, s>>>(a, t, f);
+  return cudaGetLastError();
 }
 
 template <int N, bool PIC>

@@ -23,12 +23,12 @@ __device__ __forceinline__ int ens_find(const long long* off, int nr, long long 
   return lo;
 }
 
-template <int N, bool MIXED>
+template <int N, bool MIXED, bool PIC>
 struct EnsCfg {
-  static constexpr int TPB = MIXED ? CfgCKM<N>::TPB : CfgE<N>::TPB;
-  static constexpr int MINB = MIXED ? CfgCKM<N>::MINB : CfgE<N>::MINB;
-  static constexpr int CPB = MIXED ? CfgCKM<N>::CPB : CfgE<N>::CPB;
-  static constexpr size_t SMEM = MIXED ? CfgCKM<N>::SMEM : CfgE<N>::SMEM;
+  static constexpr int TPB = MIXED ? CfgEM<N, PIC>::TPB : CfgE<N>::TPB;
+  static constexpr int MINB = MIXED ? CfgEM<N, PIC>::MINB : CfgE<N>::MINB;
+  static constexpr int CPB = MIXED ? CfgEM<N, PIC>::CPB : CfgE<N>::CPB;
+  static constexpr size_t SMEM = MIXED ? CfgEM<N, PIC>::SMEM : CfgE<N>::SMEM;
   static_assert(CPB == ck_cells_per_block(N), "the host counts the blocks of each run");
 };
 
@@ -38,14 +38,14 @@ __device__ __forceinline__ void ens_predictor_block(const StepArgs* R, const Ens
                                                     const Tables& T, const TablesF& F,
                                                     long long it) {
   const int r = ens_find(E.blk0, E.nr, it);
-  const long long c0 = (it - E.blk0[r]) * EnsCfg<N, MIXED>::CPB;
-  if constexpr (MIXED) predictor_ck_mixed_block<N, PIC>(R[r], T, F, c0);
+  const long long c0 = (it - E.blk0[r]) * EnsCfg<N, MIXED, PIC>::CPB;
+  if constexpr (MIXED) predictor_elastic_mixed_block<N, PIC>(R[r], T, F, c0);
   else predictor_elastic_block<N, PIC>(R[r], T, F.el, c0);
   __syncthreads();  // the next block of cells reuses the shared memory
 }
 
 template <int N, bool MIXED, bool PIC>
-__global__ void __launch_bounds__(EnsCfg<N, MIXED>::TPB, EnsCfg<N, MIXED>::MINB)
+__global__ void __launch_bounds__(EnsCfg<N, MIXED, PIC>::TPB, EnsCfg<N, MIXED, PIC>::MINB)
     k_ens_predictor(const StepArgs* __restrict__ R, const __grid_constant__ EnsTable E,
                     const __grid_constant__ Tables T, const __grid_constant__ TablesF F) {
   const long long total = E.blk0[E.nr];
@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(CfgC<P, D, N>::TPB) k_ens_corrector(const Step
 template <int N, bool MIXED, bool PIC>
 cudaError_t ens_step_n(const StepArgs* R, const EnsTable& E, const Tables& T, const TablesF& F,
                        long long blocks, cudaStream_t s) {
-  using G = EnsCfg<N, MIXED>;
+  using G = EnsCfg<N, MIXED, PIC>;
   static bool attr = false;
   if (!attr) {
     const cudaError_t e = cudaFuncSetAttribute(k_ens_predictor<N, MIXED, PIC>,
@@ -153,13 +153,13 @@ __device__ __forceinline__ bool grid_sync(GridBar* b, unsigned nblocks, long lon
 // the corrector over the concatenated degrees of freedom and the time advance, separated by
 // grid-wide barriers.  Rsteps: the runs' step arguments of each step ([steps][nr]).
 template <int N, bool MIXED>
-__global__ void __launch_bounds__(EnsCfg<N, MIXED>::TPB, EnsCfg<N, MIXED>::MINB)
+__global__ void __launch_bounds__(EnsCfg<N, MIXED, true>::TPB, EnsCfg<N, MIXED, true>::MINB)
     k_ens_fused(const StepArgs* __restrict__ Rsteps, const __grid_constant__ EnsTable E,
                 const __grid_constant__ Tables T, const __grid_constant__ TablesF F, int steps,
                 GridBar* bar, long long limit) {
   using P = Elastic;
   constexpr int D = 3;
-  constexpr int n = N + 1, TPB = EnsCfg<N, MIXED>::TPB;
+  constexpr int n = N + 1, TPB = EnsCfg<N, MIXED, true>::TPB;
   extern __shared__ __align__(16) double fsm[];
   const unsigned nb = gridDim.x;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -207,7 +207,7 @@ template <int N, bool MIXED>
 cudaError_t ens_fused_n(const StepArgs* R, const EnsTable& E, const Tables& T, const TablesF& F,
                         int steps, GridBar* bar, long long limit, int blocks_per_sm,
                         cudaStream_t s) {
-  using G = EnsCfg<N, MIXED>;
+  using G = EnsCfg<N, MIXED, true>;
   constexpr size_t SC = sizeof(SmemC<Elastic, 3, N, 1>);  // the corrector's
   constexpr size_t SMEM = G::SMEM > SC ? G::SMEM : SC;
   static int max_bps = 0;

@@ -9,12 +9,12 @@ cudaError_t predictor_picard_elastic3(const StepArgs& a, const Tables& t, const 
   if (!a.lin) return cudaErrorInvalidValue;
   if (prec == 1) {
     switch (a.g.order) {
-      case 1: return launch_predictor_ck_mixed_n<1, true>(a, t, f, s);
-      case 2: return launch_predictor_ck_mixed_n<2, true>(a, t, f, s);
-      case 3: return launch_predictor_ck_mixed_n<3, true>(a, t, f, s);
-      case 4: return launch_predictor_ck_mixed_n<4, true>(a, t, f, s);
-      case 5: return launch_predictor_ck_mixed_n<5, true>(a, t, f, s);
-      case 6: return launch_predictor_ck_mixed_n<6, true>(a, t, f, s);
+      case 1: return launch_predictor_elastic_mixed_n<1, true>(a, t, f, s);
+      case 2: return launch_predictor_elastic_mixed_n<2, true>(a, t, f, s);
+      case 3: return launch_predictor_elastic_mixed_n<3, true>(a, t, f, s);
+      case 4: return launch_predictor_elastic_mixed_n<4, true>(a, t, f, s);
+      case 5: return launch_predictor_elastic_mixed_n<5, true>(a, t, f, s);
+      case 6: return launch_predictor_elastic_mixed_n<6, true>(a, t, f, s);
     }
     return cudaErrorInvalidValue;
   }

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from cases import Case, rel_linf
+from paper_1905_07987_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -76,3 +77,22 @@ def test_non_finite():
     far = [k for k in range(25) if min(abs(k % 5 - b % 5) + abs(k // 5 - b // 5) for b in (0, 12)) > 1]
     assert rel_linf(out[far], ref[far]) < 1e-12
     assert not np.isfinite(out[12]).all() and not np.isfinite(out[0]).all()
+
+
+# the mixed elastic predictor: its lowest order in fixed point, the largest, odd and even numbers of
+# nodes; a block that is part full; 30 stable steps: levels past the room, the block in the node form
+@pytest.mark.parametrize("predictor", ["picard", "ck"])
+@pytest.mark.parametrize("order,stretch", [(3, 1), (4, 1), (5, 1), (6, 1), (4, 30), (5, 30)])
+def test_mixed_elastic(order, stretch, predictor):
+    nc = (3, 3, 3)
+    c = Case("elastic", 3, order, nc, hi=(1.3, 0.7, 1.0), predictor=predictor, precision="mixed",
+             material=synth.elastic_material(nc, seed=order))
+    s = sum(c.X)
+    # stresses of the size of the impedance times the velocities
+    u = np.stack([(3.0 if i >= 3 else 1.0) * np.sin(2 * np.pi * (s + 0.37 * i)) for i in range(9)], axis=-1)
+    dt = stretch * float(c.oracle.cfl_dt(torch.from_numpy(u)))
+    c.set(u)
+    c.ctx.step(dt)
+    ref = c.oracle_step(u, dt)
+    # the levels after the first carry binary32's rounding, 2^-24 each operation
+    assert np.abs(c.get() - ref).max() < 2e-6 * np.abs(ref - u).max()
