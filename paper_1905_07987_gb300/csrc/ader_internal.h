@@ -113,6 +113,8 @@ struct SubTables {
   double P1[MAXNS][MAXN];  // DG nodal values -> subcell averages
   double R1[MAXN][MAXNS];  // subcell averages -> DG (mean-preserving least squares)
   double Pf[MAXNS][MAXN];  // P1[s][m] / (w_m ns): subface flux -> nodal face flux weights
+  fx3 PX[MAXNS][MAXN];     // P1 in fixed point
+  int kx;                  // results r of dim passes over inputs of fx_in<4>: r 2^(E + kx)
 };
 
 // Arguments of the limiter kernels (Sec. 3.5).

@@ -418,7 +418,7 @@ bool solve_dense(int m, std::vector<double> A, std::vector<double>& B, int nrhs)
 // Subcell tables of the limiter (Sec. 3.5): P1[s][m] = mean of phi_m over subcell s, computed
 // from the monomial coefficients of phi_m (inverse Vandermonde) and exact antiderivatives;
 // R1 = the mean-preserving least-squares left inverse of P1 (KKT system).
-bool build_subtables(int order, const Tables& T, SubTables& S) {
+bool build_subtables(int order, int dim, const Tables& T, SubTables& S) {
   std::memset(&S, 0, sizeof(S));
   const int n = order + 1, ns = 2 * order + 1;
   // coefficients: phi_m(x) = sum_k a[k][m] x^k  <=>  V a = I with V[i][k] = x_i^k
@@ -461,6 +461,10 @@ bool build_subtables(int order, const Tables& T, SubTables& S) {
   if (!solve_dense(m, K, B, ns)) return false;
   for (int i = 0; i < n; ++i)
     for (int s = 0; s < ns; ++s) S.R1[i][s] = B[i * ns + s];
+  const int p = fx_scale(ns, n, S.P1[0], MAXN);
+  for (int s = 0; s < ns; ++s)
+    for (int i = 0; i < n; ++i) S.PX[s][i] = fx_entry(S.P1[s][i], p);
+  S.kx = dim * (60 - p) - 1079;
   return true;
 }
 
@@ -778,7 +782,7 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
     long long nsf = 1;
     for (int d = 0; d < cfg->dim; ++d) c->nss *= ns;
     for (int d = 1; d < cfg->dim; ++d) nsf *= ns;
-    if (!build_subtables(cfg->order, c->tab, c->sub)) e = cudaErrorInvalidValue;
+    if (!build_subtables(cfg->order, cfg->dim, c->tab, c->sub)) e = cudaErrorInvalidValue;
     const size_t nrep = (size_t)ncells * c->nss * c->nvar;
     if (e == cudaSuccess) e = cudaMalloc(&c->rep, nrep * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&c->rep_new, nrep * sizeof(double));

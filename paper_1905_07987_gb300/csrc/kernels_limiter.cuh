@@ -18,6 +18,7 @@
 // double-buffered across steps.
 #pragma once
 #include <climits>
+#include "fx.cuh"
 #include "kernels.cuh"
 
 namespace ader {
@@ -74,8 +75,74 @@ struct CfgL {
   static constexpr int T1 = ipow(ns, D - 1) * n * NV;
   static constexpr int T2 = D == 3 ? n * ns * ns * NV : 0;
   static constexpr size_t SMEM_P = (size_t)(NN * NV + T1 + T2 + NSS * NV) * sizeof(double);
+  // projection alone: in 3-D the first partial result lies where the subcell values go
+  static constexpr int T1P = D == 3 ? 0 : T1;
+  static constexpr size_t SMEM_D = (size_t)(NN * NV + T1P + T2 + NSS * NV) * sizeof(double);
   static constexpr size_t SMEM_FV = (size_t)(NH * NV + NC * NV + (ns + 1) * NSF * NV) * sizeof(double);
 };
+
+// Order-preserving map of a double to a 64-bit integer (both zeros to 0, negative values to
+// minus their magnitude bits); it is its own inverse.  For values that are not NaN,
+// x <= y exactly when okey(x) <= okey(y), so the bound tests and the min / max of the
+// limiter run on the integer pipes instead of the FP64 pipe.
+__device__ __forceinline__ long long okey(double x) {
+  const long long b = __double_as_longlong(x);
+  return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b);
+}
+__device__ __forceinline__ double okey_inv(long long k) {
+  return __longlong_as_double(k >= 0 ? k : (long long)(0x8000000000000000ull - (unsigned long long)k));
+}
+
+// Min or max of 32 lanes' keys: 32-bit reductions of the high words, then of the low words of the lanes
+// that have the winning one.
+__device__ __forceinline__ long long warp_min(long long k) {
+  const int h = (int)(k >> 32), m = __reduce_min_sync(0xffffffffu, h);
+  const unsigned l = __reduce_min_sync(0xffffffffu, h == m ? (unsigned)k : 0xffffffffu);
+  return (long long)m * 4294967296ll + l;
+}
+__device__ __forceinline__ long long warp_max(long long k) {
+  const int h = (int)(k >> 32), m = __reduce_max_sync(0xffffffffu, h);
+  const unsigned l = __reduce_max_sync(0xffffffffu, h == m ? (unsigned)k : 0u);
+  return (long long)m * 4294967296ll + l;
+}
+
+// Keys of the per-variable min / max of sub[NSS][NV] into key[2 NV]; red: smem scratch [2][NV][32].
+template <int NSS, int NV>
+__device__ void block_keys(const double* sub, long long* key, long long* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int v = 0; v < NV; ++v) {
+    long long lo = LLONG_MAX, hi = LLONG_MIN;
+    for (int s = threadIdx.x; s < NSS; s += blockDim.x) {
+      const long long k = okey(sub[s * NV + v]);
+      lo = min(lo, k);
+      hi = max(hi, k);
+    }
+    lo = warp_min(lo);
+    hi = warp_max(hi);
+    if (lane == 0) {
+      red[(0 * NV + v) * 32 + warp] = lo;
+      red[(1 * NV + v) * 32 + warp] = hi;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * NV) {
+    const int k = threadIdx.x;
+    long long r = red[k * 32];
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
+      r = k < NV ? min(r, red[k * 32 + w]) : max(r, red[k * 32 + w]);
+    key[k] = r;
+  }
+  __syncthreads();
+}
+
+// The same as values, into mm[2][NV].  Finite inputs give the same values as fmin / fmax (a zero
+// comes out as +0).
+template <int NSS, int NV>
+__device__ void block_minmax(const double* sub, double* mm, long long* red) {
+  __shared__ long long key[2 * NV];
+  block_keys<NSS, NV>(sub, key, red);
+  if (threadIdx.x < 2 * NV) mm[threadIdx.x] = okey_inv(key[threadIdx.x]);
+}
 
 // One axis of a sum-factorised tensor-product map: Y[o][q][i] = sum_p M[q][p] X[o][p][i] with
 // M = P1 (PROJ) or R1.  One thread per (o, i) column holds the LIN inputs in registers; the
@@ -100,11 +167,44 @@ __device__ __forceinline__ void contract_axis(const double* X, double* Y, const 
   }
 }
 
-// sub[s][v] = sum over nodes of prod_e P1[s_e][a_e] u[a][v] (sum factorisation, x first).
-// u: [NN][NV], out: [NSS][NV]; t1, t2 scratch.  All threads of the block participate.
+// The same in fixed point (fx.cuh), M = P1: nodal values of scale E in (FIRST); doubles out, to shared
+// memory and to the representation, with the smallest and the largest result of the thread (LAST).
+// Threads below `per`, a multiple of NV: each stays with one variable.
+template <int LIN, int LOUT, int OUTER, int INNER, int NV, bool FIRST, bool LAST>
+__device__ __forceinline__ void contract_axis_fx(const double* X, double* Y, double* rep, int per, int E,
+                                                 const SubTables& S, long long& lo, long long& hi) {
+  static_assert(INNER % NV == 0, "the variables are the fastest index");
+  if ((int)threadIdx.x >= per) return;
+  for (int it = threadIdx.x; it < OUTER * INNER; it += per) {
+    const int o = it / INNER, i = it - o * INNER;
+    const double* x = X + o * (LIN * INNER) + i;
+    int over = 0;
+    fx2 xv[LIN];
+#pragma unroll
+    for (int p = 0; p < LIN; ++p)
+      xv[p] = FIRST ? fx_split(fx_in<4>(x[p * INNER], E, over))
+                    : reinterpret_cast<const fx2*>(x)[p * INNER];
+    const int yo = o * (LOUT * INNER) + i;
+#pragma unroll
+    for (int q = 0; q < LOUT; ++q) {
+      const long long r = fx_dot<LIN, 4>(xv, S.PX[q]);
+      if (LAST) {
+        lo = min(lo, r);
+        hi = max(hi, r);
+        const double y = fx_out(r, E + S.kx);
+        Y[yo + q * INNER] = y;
+        rep[yo + q * INNER] = y;
+      } else {
+        reinterpret_cast<fx2*>(Y)[yo + q * INNER] = fx_split(r);
+      }
+    }
+  }
+}
+
+// sub[s][v] = sum over nodes of prod_e P1[s_e][a_e] u[a][v] (sum factorisation, x first), in FP64.
 template <int D, int N>
-__device__ void project_P(const double* u, double* t1, double* t2, double* out,
-                          const SubTables& S) {
+__device__ __noinline__ void project_P_plain(const double* u, double* t1, double* t2, double* out,
+                                             const SubTables& S) {
   using L = CfgL<D, N>;
   constexpr int n = L::n, ns = L::ns, NV = L::NV;
   if constexpr (D == 2) {
@@ -117,6 +217,79 @@ __device__ void project_P(const double* u, double* t1, double* t2, double* out,
     contract_axis<n, ns, n, ns * NV, true>(t1, t2, S);        // t2[z][sy][sx][v]
     __syncthreads();
     contract_axis<n, ns, 1, ns * ns * NV, true>(t2, out, S);  // out[sz][sy][sx][v]
+  }
+  __syncthreads();
+}
+
+// The same on the integer pipe, with a copy in rep (global) and the keys of the per-variable min and
+// max in key[2 NV].  u: [NN][NV], out: [NSS][NV]; t1 (in 3-D it may be out), t2 scratch, red
+// [2][NV][32] for the keys.  All threads of the block participate; a barrier comes before the first
+// read of u and one is last.
+//
+// The FP64 pipe (2 lane operations per clock and SM) was the bound: 13020 FMAs a cell at order 3 in
+// 3-D.  One scale per cell and variable, the power of two above its largest nodal value: values
+// below 2^57, rows of P1 of sum below 2 after the host's scaling, so nothing passes 2^60 in three
+// passes.  The conversion truncates at 2^-57 of the largest value and each pass rounds at 2^-57
+// to 2^-56 of it, where each FP64 FMA rounds at 2^-53 of its partial sum.  Min and max are taken of
+// the integers, whose order fx_out keeps.  Non-finite values and such near the end of binary64's
+// range: the FP64 form.
+//
+// Measured, 64^3 cells of order 3: k_lim_detect 8.8 -> 3.85 ms, k_lim_init 7.6 -> 2.97 ms (with the
+// integer contractions but min, max and the copy taken from shared memory afterwards 4.47 and 3.55).
+// What is left: half of the issue slots, and the barriers between the passes.
+template <int D, int N>
+__device__ __forceinline__ void project_P(const double* u, double* t1, double* t2, double* out,
+                                          double* rep, long long* key, long long* red,
+                                          const SubTables& S) {
+  using L = CfgL<D, N>;
+  constexpr int n = L::n, ns = L::ns, NV = L::NV, NN = L::NN, NSS = L::NSS;
+  constexpr int PER = L::TPB / NV * NV, RV = PER / NV;
+  static_assert(RV <= 32 && 2 * PER <= 2 * NV * 32, "one warp reduces a variable");
+  __shared__ int s_E[NV];
+  const int tid = threadIdx.x, v = tid % NV, lane = tid & 31;
+  if (tid < NV) s_E[tid] = 200;
+  __syncthreads();
+  if (tid < PER) {
+    int E = 200;
+    for (int e = tid; e < NN * NV; e += PER)
+      E = max(E, (int)(((unsigned)__double2hiint(u[e]) >> 20) & 0x7ffu));
+    atomicMax(&s_E[v], E);
+  }
+  __syncthreads();
+  bool big = false;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) big = big || s_E[i] > 1900;
+  if (big) {
+    project_P_plain<D, N>(u, t1, t2, out, S);
+    for (int e = tid; e < NSS * NV; e += L::TPB) rep[e] = out[e];
+    block_keys<NSS, NV>(out, key, red);
+    return;
+  }
+  const int E = s_E[v];
+  long long lo = LLONG_MAX, hi = LLONG_MIN;
+  if constexpr (D == 2) {
+    contract_axis_fx<n, ns, n, NV, NV, true, false>(u, t1, rep, PER, E, S, lo, hi);
+    __syncthreads();
+    contract_axis_fx<n, ns, 1, ns * NV, NV, false, true>(t1, out, rep, PER, E, S, lo, hi);
+  } else {
+    contract_axis_fx<n, ns, n * n, NV, NV, true, false>(u, t1, rep, PER, E, S, lo, hi);
+    __syncthreads();
+    contract_axis_fx<n, ns, n, ns * NV, NV, false, false>(t1, t2, rep, PER, E, S, lo, hi);
+    __syncthreads();
+    contract_axis_fx<n, ns, 1, ns * ns * NV, NV, false, true>(t2, out, rep, PER, E, S, lo, hi);
+  }
+  if (tid < PER) {
+    red[tid] = lo;
+    red[PER + tid] = hi;
+  }
+  __syncthreads();
+  for (int k = tid >> 5; k < 2 * NV; k += L::TPB / 32) {  // a warp per key
+    const bool mx = k >= NV;
+    const int i = mx ? k - NV : k;
+    long long r = mx ? LLONG_MIN : LLONG_MAX;
+    if (lane < RV) r = red[(mx ? PER : 0) + i + lane * NV];
+    r = mx ? warp_max(r) : warp_min(r);
+    if (lane == 0) key[k] = okey(fx_out(r, s_E[i] + S.kx));
   }
   __syncthreads();
 }
@@ -141,16 +314,8 @@ __device__ void reconstruct_R(const double* U, double* t1, double* t2, double* o
   __syncthreads();
 }
 
-// Order-preserving map of a double to a 64-bit integer (both zeros to 0, negative values to
-// minus their magnitude bits); it is its own inverse.  For values that are not NaN,
-// x <= y exactly when okey(x) <= okey(y), so the bound tests and the min / max of the
-// limiter run on the integer pipes instead of the FP64 pipe.
-__device__ __forceinline__ long long okey(double x) {
-  const long long b = __double_as_longlong(x);
-  return b >= 0 ? b : (long long)(0x8000000000000000ull - (unsigned long long)b);
-}
-__device__ __forceinline__ double okey_inv(long long k) {
-  return __longlong_as_double(k >= 0 ? k : (long long)(0x8000000000000000ull - (unsigned long long)k));
+__device__ __forceinline__ bool is_nan(double x) {
+  return (unsigned long long)(__double_as_longlong(x) & 0x7fffffffffffffffll) > 0x7ff0000000000000ull;
 }
 
 // rho > 0 and p > 0 with every value finite.  For rho > 0 and gamma > 1, p > 0 is
@@ -189,38 +354,6 @@ __device__ __forceinline__ bool admissible_f(const double* q, double floor, doub
 }
 
 
-// Per-variable min / max of sub[NSS][NV] into mm[2][NV]; red: smem scratch [2][NV][32].
-// Finite inputs give the same values as fmin / fmax (a zero comes out as +0).
-template <int NSS, int NV>
-__device__ void block_minmax(const double* sub, double* mm, long long* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int v = 0; v < NV; ++v) {
-    long long lo = LLONG_MAX, hi = LLONG_MIN;
-    for (int s = threadIdx.x; s < NSS; s += blockDim.x) {
-      const long long k = okey(sub[s * NV + v]);
-      lo = min(lo, k);
-      hi = max(hi, k);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if (lane == 0) {
-      red[(0 * NV + v) * 32 + warp] = lo;
-      red[(1 * NV + v) * 32 + warp] = hi;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < 2 * NV) {
-    const int k = threadIdx.x;
-    long long r = red[k * 32];
-    for (int w = 1; w < nw; ++w) r = (k < NV) ? min(r, red[k * 32 + w]) : max(r, red[k * 32 + w]);
-    mm[k] = okey_inv(r);
-  }
-  __syncthreads();
-}
-
 template <int D>
 __device__ __forceinline__ long long neighbor(const Geometry& g, long long c, int d, int side) {
   long long idx[3], rem = c;
@@ -245,11 +378,11 @@ __global__ void __launch_bounds__(128) k_lim_detect(const __grid_constant__ Step
   constexpr int NN = C::NN, NSS = C::NSS, NV = C::NV;
   extern __shared__ double sm[];
   double* us = sm;
-  double* t1 = us + NN * NV;
-  double* t2 = t1 + C::T1;
+  double* t2 = us + NN * NV + C::T1P;
   double* sub = t2 + C::T2;
+  double* t1 = D == 3 ? sub : us + NN * NV;
   __shared__ long long red[2 * NV * 32];
-  __shared__ long long bk[2][NV];
+  __shared__ long long bk[2][NV], key[2 * NV];
   const long long c = blockIdx.x;
   if (L.status) {
     // hybrid status: a cell with FV steps left, or next to one, computes with FV in this step
@@ -270,41 +403,38 @@ __global__ void __launch_bounds__(128) k_lim_detect(const __grid_constant__ Step
   for (int e = threadIdx.x; e < NN * NV; e += blockDim.x) us[e] = u[e];
   if (threadIdx.x < NV) {
     const int v = threadIdx.x;
-    double lo = L.mm[c * 2 * NV + v], hi = L.mm[c * 2 * NV + NV + v];
-    for (int d = 0; d < D; ++d)
-      for (int side = -1; side <= 1; side += 2) {
-        const long long nb = neighbor<D>(A.g, c, d, side);
-        if (nb >= 0) {
-          lo = fmin(lo, L.mm[nb * 2 * NV + v]);
-          hi = fmax(hi, L.mm[nb * 2 * NV + NV + v]);
-        }
-      }
+    // min and max over the cell and its neighbours, as keys; NaN is passed over
+    long long kl = LLONG_MAX, kh = LLONG_MIN;
+#pragma unroll
+    for (int i = 0; i <= 2 * D; ++i) {
+      const long long nb = i < 2 * D ? neighbor<D>(A.g, c, i >> 1, i & 1 ? 1 : -1) : c;
+      const double* m = L.mm + (nb >= 0 ? nb : c) * 2 * NV + v;
+      const double a = m[0], b = m[NV];
+      if (!is_nan(a)) kl = min(kl, okey(a));
+      if (!is_nan(b)) kh = max(kh, okey(b));
+    }
+    const double lo = okey_inv(kl), hi = kh == LLONG_MIN ? okey_inv(LLONG_MAX) : okey_inv(kh);
     // DMP band [lo - delta, hi + delta] as ordered keys (a NaN bound admits nothing)
     const double delta = fmax(L.eps * (hi - lo), L.delta0);
     const double bl = lo - delta, bh = hi + delta;
     bk[0][v] = bl == bl ? okey(bl) : LLONG_MAX;
     bk[1][v] = bh == bh ? okey(bh) : LLONG_MIN;
   }
-  __syncthreads();
-  project_P<D, N>(us, t1, t2, sub, S);
+  project_P<D, N>(us, t1, t2, sub, L.rep_new + c * (NSS * NV), key, red, S);
   bool ok = true;
-  for (int s = threadIdx.x; s < NSS; s += blockDim.x) {
-    const double* q = sub + s * NV;
-    ok = ok && admissible_f<D>(q, L.floor, A.p.gamma);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      const long long k = okey(q[v]);
-      ok = ok && (k >= bk[0][v]) && (k <= bk[1][v]);
-    }
-  }
+  for (int s = threadIdx.x; s < NSS; s += blockDim.x)
+    ok = ok && admissible_f<D>(sub + s * NV, L.floor, A.p.gamma);
   for (int j = threadIdx.x; j < NN; j += blockDim.x)
     ok = ok && admissible_f<D>(us + j * NV, L.floor, A.p.gamma);
+  if (threadIdx.x < 2 * NV) {
+    // every value lies in the band exactly when the smallest and the largest do
+    const int k = threadIdx.x;
+    const long long r = key[k];
+    L.mm_new[c * 2 * NV + k] = okey_inv(r);
+    ok = ok && (k < NV ? r >= bk[0][k] : r <= bk[1][k - NV]);
+  }
   const bool all_ok = __syncthreads_and(ok) != 0;
-  const bool troubled = L.force ? true : !all_ok;
-  double* rn = L.rep_new + c * (NSS * NV);
-  for (int e = threadIdx.x; e < NSS * NV; e += blockDim.x) rn[e] = sub[e];
-  block_minmax<NSS, NV>(sub, L.mm_new + c * 2 * NV, red);
-  if (threadIdx.x == 0) L.flags[c] = troubled ? 1 : 0;
+  if (threadIdx.x == 0) L.flags[c] = (L.force || !all_ok) ? 1 : 0;
 }
 
 // Troubled list by warp ballot: every lane votes with its cell's flag, lane 0 reserves the warp's
@@ -615,7 +745,7 @@ __global__ void __launch_bounds__(128) k_lim_fix(const __grid_constant__ StepArg
   double* t2 = t1 + C::T1;
   double* sub = t2 + C::T2;
   double* geff = sub + NSS * NV;  // [NF][NV]
-  __shared__ long long red[2 * NV * 32];
+  __shared__ long long red[2 * NV * 32], key[2 * NV];
   double* u = A.u_next + c * (NN * NV);
   for (int e = threadIdx.x; e < NN * NV; e += blockDim.x) us[e] = u[e];
   __syncthreads();
@@ -667,10 +797,8 @@ __global__ void __launch_bounds__(128) k_lim_fix(const __grid_constant__ StepArg
     }
   }
   for (int e = threadIdx.x; e < NN * NV; e += blockDim.x) u[e] = us[e];
-  project_P<D, N>(us, t1, t2, sub, S);
-  double* rn = L.rep_new + c * (NSS * NV);
-  for (int e = threadIdx.x; e < NSS * NV; e += blockDim.x) rn[e] = sub[e];
-  block_minmax<NSS, NV>(sub, L.mm_new + c * 2 * NV, red);
+  project_P<D, N>(us, t1, t2, sub, L.rep_new + c * (NSS * NV), key, red, S);
+  if (threadIdx.x < 2 * NV) L.mm_new[c * 2 * NV + threadIdx.x] = okey_inv(key[threadIdx.x]);
 }
 
 // rep = P(u) for every cell (reset of the limiter history); flagged cells keep the given U_sub
@@ -686,24 +814,23 @@ __global__ void __launch_bounds__(128) k_lim_init(double* u, const double* Usub,
   double* t1 = us + NN * NV;
   double* t2 = t1 + C::T1;
   double* sub = t2 + C::T2;
-  __shared__ long long red[2 * NV * 32];
+  __shared__ long long red[2 * NV * 32], key[2 * NV];
   const long long c = blockIdx.x;
   double* uc = u + c * (NN * NV);
   const bool fl = flags && flags[c];
+  double* r = rep + c * (NSS * NV);
   if (fl) {
     const double* U = Usub + c * (NSS * NV);
-    for (int e = threadIdx.x; e < NSS * NV; e += blockDim.x) sub[e] = U[e];
+    for (int e = threadIdx.x; e < NSS * NV; e += blockDim.x) r[e] = sub[e] = U[e];
     __syncthreads();
     reconstruct_R<D, N>(sub, t1, t2, us, S);
     for (int e = threadIdx.x; e < NN * NV; e += blockDim.x) uc[e] = us[e];
+    block_keys<NSS, NV>(sub, key, red);
   } else {
     for (int e = threadIdx.x; e < NN * NV; e += blockDim.x) us[e] = uc[e];
-    __syncthreads();
-    project_P<D, N>(us, t1, t2, sub, S);
+    project_P<D, N>(us, t1, t2, sub, r, key, red, S);
   }
-  double* r = rep + c * (NSS * NV);
-  for (int e = threadIdx.x; e < NSS * NV; e += blockDim.x) r[e] = sub[e];
-  block_minmax<NSS, NV>(sub, mm + c * 2 * NV, red);
+  if (threadIdx.x < 2 * NV) mm[c * 2 * NV + threadIdx.x] = okey_inv(key[threadIdx.x]);
 }
 
 // ---- launchers -----------------------------------------------------------------------------
@@ -728,7 +855,7 @@ struct LimLaunch {
     static bool attr = false;
     if (!attr) {
       cudaError_t e = cudaFuncSetAttribute(k_lim_detect<D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)C::SMEM_P);
+                                           (int)C::SMEM_D);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_lim_fv<D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)C::SMEM_FV);
@@ -739,7 +866,7 @@ struct LimLaunch {
       attr = true;
     }
     const unsigned nc = (unsigned)a.g.ncells;
-    k_lim_detect<D, N><<<nc, C::TPB, C::SMEM_P, s>>>(a, l, S);
+    k_lim_detect<D, N><<<nc, C::TPB, C::SMEM_D, s>>>(a, l, S);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (l.status) {  // hybrid status: widen the flags before the compaction

@@ -324,3 +324,30 @@ def test_host_batch_with_the_limiter_equals_the_step_loop():
         c.ctx.set_time(0.0)
         c.ctx.step()
         assert np.array_equal(c.get().reshape(-1), outs[k].numpy()), k
+
+
+# the projection in fixed point against its FP64 form, which takes what lies near the end of the range:
+# the same data scaled by a power of two
+@pytest.mark.parametrize("exponent", [0, -200])
+@pytest.mark.parametrize("dim,order", [(2, 1), (2, 2), (2, 3), (2, 4), (3, 1), (3, 2), (3, 3), (3, 4)])
+def test_projection(dim, order, exponent):
+    ncell = (3, 2, 4)[:dim]
+    c = Case("euler", dim, order, ncell, limiter=1)
+    lim = Limiter(c.oracle)
+    rng = np.random.default_rng(order)
+    u = rng.standard_normal(c.shape) * 10.0 ** rng.uniform(-3, 3, (c.ctx.cells,) + (1,) * dim + (c.ctx.nvar,))
+    u[1, ..., 0] = 0.0
+    u[2, 0, 0, ..., 1] = np.nan
+
+    def project(x):
+        gpu_set(c, x, np.zeros((c.ctx.cells,) + (lim.ns,) * dim + (c.ctx.nvar,)), np.zeros(c.ctx.cells, dtype=bool))
+        return gpu_rep(c, lim)
+
+    got = np.ldexp(project(np.ldexp(u, exponent)), -exponent)
+    ref = np.ldexp(project(np.ldexp(u, 960)), -960)
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    assert rel_linf(np.nan_to_num(got), np.nan_to_num(lim.project(torch.from_numpy(u)).numpy())) <= TOL
+    # dim passes of at most 5 products, rounded at 2^-53 (fixed point: less), rows of sum below 2
+    top = np.abs(u).max(axis=tuple(range(1, dim + 1)), keepdims=True)
+    ok = ~np.isnan(ref)
+    assert (np.abs(got - ref) <= 3 * 5 * 2 ** 3 * 2.0 ** -53 * np.broadcast_to(top, ref.shape))[ok].all()
