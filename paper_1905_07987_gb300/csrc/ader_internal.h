@@ -333,7 +333,6 @@ int limiter_max_order3();
 cudaError_t launch_dt_finalize(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_ens_dt(const StepArgs* runs, int nr, cudaStream_t s);
 cudaError_t launch_ens_advance(const StepArgs* runs, int nr, cudaStream_t s);
-cudaError_t launch_advance(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_advance_rec(const StepArgs& a, int receivers_on, cudaStream_t s);
 cudaError_t launch_receivers(const StepArgs& a, const Receivers& r, int nodes, int nvar,
                              cudaStream_t s);

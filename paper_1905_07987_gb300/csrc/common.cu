@@ -199,8 +199,6 @@ cudaError_t launch_advance_rec(const StepArgs& a, int receivers_on, cudaStream_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_advance(const StepArgs& a, cudaStream_t s) { return launch_advance_rec(a, 0, s); }
-
 cudaError_t launch_receivers(const StepArgs& a, const Receivers& r, int nodes, int nvar,
                              cudaStream_t s) {
   if (r.nrec <= 0) return cudaSuccess;

@@ -1,8 +1,8 @@
 // FP64 kernels of one ADER-DG step (Sec. 3.3-3.4), templated on the PDE system, the dimension
 // and the order.  One thread block per cell for the predictor (the work is FP64-pipe bound on
 // GB300: every cell is an independent dense small contraction problem), one warp per face for
-// the Riemann solver, one thread per degree of freedom for the corrector, grid-stride tiles for
-// the CFL maximum (Euler: FP64 evaluation only on the nodes that binary32 enclosures cannot rule
+// the Riemann solver (or several faces of few nodes), a thread per z line (3-D, order 3 and up) or
+// per degree of freedom for the corrector, grid-stride tiles for the CFL maximum (Euler: FP64 evaluation only on the nodes that binary32 enclosures cannot rule
 // out).  The Riemann solver also serves the mixed-precision form (wave speeds evaluated by its
 // predictor).
 #pragma once

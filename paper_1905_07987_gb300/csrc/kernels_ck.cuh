@@ -34,7 +34,7 @@
 // 18n + 24 FMA per node and application.  The Taylor coefficients ping-pong between two
 // shared-memory buffers of padded node records, 10 doubles per node, read in 16-byte pairs.
 //
-// Mixed-precision form (k_predictor_ck_mixed): only the O(1) base term L u carries the size of the
+// Mixed-precision form (predictor_ck_mixed_block): only the O(1) base term L u carries the size of the
 // solution; it is formed once in float-float (hi + lo binary32 pairs, about 44 bits) and serves
 // both a_1 = dt (L u + g s_0) and the volume term.  a_1 is float-float; a_2 .. a_N (O(dt^2) and
 // smaller) and L applied to the increment of the time average run in binary32.  The time average
