@@ -38,12 +38,15 @@ FP64_SMS, FP64_FMA_PER_CLK, SM_MAX_MHZ = 152, 2, 2070.0
 # DRAM bytes (read + write) per cell of the predictor kernels, from one ncu capture of the same
 # kernels on 40^3 cells, scaled to a launch by the number of cells (the traffic is per cell:
 # state in, next state and face records out; the mixed form also writes the face wave speeds).
-# FP64: k_predictor<Euler<3>,3,4> on 64 000 cells, read 331.102464 MB, write 1031.607040 MB;
+# FP64 (the FP64-pipe form; the fixed-point form moves the same state and records): 64 000 cells, read 331.102464 MB, write 1031.607040 MB;
 # mixed (the kernel with the continuous extension Runge-Kutta stages, captured with that guess):
 # read 320.445184 MB, write 1103.791872 MB.
 TRAFFIC_PER_CELL = {"fp64": (331.102464e6 + 1031.607040e6) / 64000,
                     "mixed": (320.445184e6 + 1103.791872e6) / 64000}
 FP64_PEAK = FP64_SMS * FP64_FMA_PER_CLK * 2 * SM_MAX_MHZ * 1e6  # FLOP/s
+# the FP64 predictors run their products in 64-bit fixed point: four 32 x 32 + 64-bit integer
+# multiply-adds each, 64 of those per clock and SM
+FX_PEAK = FP64_SMS * 64 / 4 * 2 * SM_MAX_MHZ * 1e6  # FLOP/s, a multiply-add of the model = 2
 
 
 def predictor_flops_per_cell(pde, D, N, iters):
@@ -1155,16 +1158,18 @@ def main():
         pred_ms = r["phases"]["predictor"] / nrec
         achieved = flops_model / (pred_ms * 1e-3) / 1e12
         key = "fp64" if prec == "fp64" else "fp32"
-        derived = (FP64_PEAK if prec == "fp64" else FP32_PEAK) / 1e12
-        if peaks and peaks.get(key):
+        derived = (FX_PEAK if prec == "fp64" else FP32_PEAK) / 1e12
+        if prec == "fp64":
+            peak, src = derived, "derived: 152 SMs x 64 integer multiply-adds/clk / 4 per product x 2 flop x 2070 MHz"
+        elif peaks and peaks.get(key):
             peak, src = peaks[key], "measured in this run (%s FMA throughput, libpeaks)" % key.upper()
         else:
-            peak, src = derived, "derived: 152 SMs x %d FMA/clk x 2 flop x 2070 MHz" % (
-                2 if prec == "fp64" else 128)
-        kname = "k_predictor (FP64)" if prec == "fp64" else \
+            peak, src = derived, "derived: 152 SMs x 128 FMA/clk x 2 flop x 2070 MHz"
+        kname = "k_predictor_fx (FP64 results, 64-bit fixed-point contractions on the integer pipe)" if prec == "fp64" else \
             "k_predictor_mixed (binary32 Picard iterations and flux remainders; float-float base terms, time averages and contractions; FP64 face wave speeds)"
         if FORMS[form][1] == "cerk":
             kname += ", continuous extension Runge-Kutta guess + %d iteration(s)" % FORMS[form][2]
+        fp64 = (peaks or {}).get("fp64") or FP64_PEAK / 1e12
         return {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": TRAFFIC_PER_CELL.get(prec, 0) * cells if TRAFFIC_PER_CELL.get(prec) else None,
@@ -1173,7 +1178,7 @@ def main():
                 "kernel_count_flops_per_cell": flops_kernel / cells,
                 "frac_kernel_count": flops_kernel / (pred_ms * 1e-3) / 1e12 / peak,
                 "frac_of_derived_peak": achieved / derived, "derived_peak": derived,
-                "ms_per_launch": pred_ms,
+                "over_fp64_peak": achieved / fp64, "ms_per_launch": pred_ms,
                 "phase_ms_per_step": {k: v / nrec for k, v in r["phases"].items()}}
 
     roof = roofline(args.prec)
@@ -1187,7 +1192,7 @@ def main():
             if k != "fp64" and r["err"]:
                 forms_out[k]["l2_error_over_fp64"] = r["err"]["l2_rho"] / res["fp64"]["err"]["l2_rho"]
                 forms_out[k]["speedup_over_fp64"] = r["value"] / res["fp64"]["value"]
-    launches_per_step = 1 + 1 + 1 + D + 1 + 1
+    launches_per_step = 4  # CFL with dt, predictor, Riemann of all directions, corrector with the time
     # the FP64 form of the same workload (the scheme's reference arithmetic), with its error
     fp64_entry = None
     if "fp64" in res:

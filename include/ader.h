@@ -72,7 +72,9 @@ typedef enum { ADER_PDE_ADVECTION = 0, ADER_PDE_EULER = 1, ADER_PDE_ELASTIC = 2,
 typedef enum { ADER_BC_PERIODIC = 0, ADER_BC_WALL = 1, ADER_BC_ABSORBING = 2 } ader_bc;
 
 /* Arithmetic of the step:
- *  FP64  - everything in binary64;
+ *  FP64  - everything in binary64 or, where a cell's values share a scale, in 64-bit fixed point
+ *          relative to the cell's largest value (rounding 2^-57 of it; non-finite values and
+ *          magnitudes near the ends of the range are computed in binary64);
  *  MIXED - predictor iterations on the increment q - u^n in binary32 with float-float base
  *          terms, time averages and contractions.  Pressure / sound speed and eigenvalues, the
  *          Riemann flux, the corrector and the limiter stay binary64 (for Euler the face wave
@@ -100,7 +102,8 @@ typedef enum { ADER_PREC_FP64 = 0, ADER_PREC_MIXED = 1, ADER_PREC_MIXED_TF32X3 =
  *           its degree-N interpolant at the step's Gauss-Legendre time nodes.  Built for the
  *           3-D elastic family (others: ADER_EUNSUPPORTED), with ADER_PREC_FP64 and with
  *           ADER_PREC_MIXED (the O(1) base term L u and the first Taylor coefficient in
- *           float-float, the higher coefficients in binary32, the update u + dt vol in FP64).
+ *           float-float or, from order 5, in 64-bit fixed point, the higher coefficients in
+ *           binary32, the update u + dt vol in FP64).
  *           Differentiated (orders 1-5): the adjoint entry points take the FP64 adjoint of the
  *           Taylor recursion. */
 typedef enum { ADER_PREDICTOR_PICARD = 0, ADER_PREDICTOR_CK = 1 } ader_predictor;
@@ -270,8 +273,8 @@ ader_status ader_run_graph(ader_ctx* ctx, int steps, int replays, double dt, dou
  * and accumulates  grad_mat[c][0..2] += d/d(rho, lambda, mu)_c of (lambda^{n+1})^T u^{n+1}  and
  * grad_M[0..5] += d/dM of the same, evaluated at the forward state u_n = u^n with the step
  * starting at time t_n.  With the Picard predictor this is the adjoint of the FP64 step (a MIXED
- * context too).  With the Cauchy-Kowalevski predictor an FP64 context gets the adjoint of its
- * FP64 step, a MIXED or TF32X3 context a mixed-precision adjoint: the base term F + dt L^T lambda
+ * context too), as the adjoint of the polynomial in dt L that the iterates are.  With the
+ * Cauchy-Kowalevski predictor an FP64 context gets the adjoint of its FP64 step, a MIXED or TF32X3 context a mixed-precision adjoint: the base term F + dt L^T lambda
  * in float-float, the level corrections dt L^T mu in binary32, lambda + mu_0 in FP64 (within a
  * few binary32 roundoffs, relative to the largest value, of the FP64 adjoint).  The wave speed max(vp_L, vp_R) of a face takes the left value at
  * ties.  The gradient sums are formed in a fixed order: repeated calls give identical bits.
@@ -285,8 +288,9 @@ ader_status ader_adjoint_step(ader_ctx* ctx, double t_n, double dt, const double
                               const double* dJdu, double* grad_mat, double* grad_M);
 
 /* Same result as ader_adjoint_step, but this call allocates no memory: its work buffers (the
- * forward Picard iterates kept per thread block (none with the Cauchy-Kowalevski predictor), the
- * face adjoints and the per-face material gradients) live in one fixed 64 MiB array of device memory that the library defines, so no
+ * forward Picard iterates kept per thread block (none with the Cauchy-Kowalevski predictor, nor
+ * with the Picard predictor where the buffers of the polynomial form fit), the face adjoints and
+ * the per-face material gradients) live in one fixed 64 MiB array of device memory that the library defines, so no
  * cudaMalloc, cudaFree or other allocating call is made.  It exists for callers that cannot
  * allocate device memory at the time of the call: for example code whose device memory is
  * owned by another allocator (a framework's memory pool that has reserved the GPU), processes
