@@ -116,6 +116,51 @@ __device__ __forceinline__ void ck_dmat_R(const double (&P)[9], const double (&n
   gm[2] = fma(imu, s, gm[2]);
 }
 
+// What the rows of L multiply by the material at node j: E_i = sum_d d sigma_{id} / dx_d (velocity
+// rows), E_{3+d} = dv_d / dx_d, and the shear rows' sums of two velocity derivatives.
+template <int N>
+__device__ __forceinline__ void ck_strains(const double* X, int j, const double (&Dr)[3][N + 1],
+                                           const double* inv_h, double (&E)[9]) {
+#pragma unroll
+  for (int v = 0; v < 9; ++v) E[v] = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double ih = inv_h[d];
+    double dv[3], ds[3];
+    ck_derivs<N>(X, j, d, Dr[d], dv, ds);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) E[i] = fma(ih, ds[i], E[i]);
+    E[3 + d] = ih * dv[d];
+#pragma unroll
+    for (int v = 6; v < 9; ++v) {
+      const int s = Elastic::src(d, v);
+      if (s >= 0) E[v] = fma(ih, dv[s], E[v]);
+    }
+  }
+}
+
+// R = f L a at one node from the strains E of a.
+__device__ __forceinline__ void ck_rows(const double (&E)[9], double f, double irho, double lam,
+                                        double mu, double (&R)[9]) {
+  const double fr = f * irho, fm = f * mu, lt = f * lam * (E[3] + E[4] + E[5]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    R[i] = fr * E[i];
+    R[3 + i] = fma(2.0 * fm, E[3 + i], lt);
+    R[6 + i] = fm * E[6 + i];
+  }
+}
+
+// gm += f nu^T (dL/d(rho, lam, mu)) a at one node from the strains E of a: no division, so a fluid
+// (mu = 0) or 3 lam + 2 mu = 0 is as exact as any material.
+__device__ __forceinline__ void ck_dmat_E(const double* E, const double (&nu)[9], double f,
+                                          double irho, double (&gm)[3]) {
+  gm[0] = fma(-f * irho * irho, fma(nu[0], E[0], fma(nu[1], E[1], nu[2] * E[2])), gm[0]);
+  gm[1] = fma(f * (E[3] + E[4] + E[5]), nu[3] + nu[4] + nu[5], gm[1]);
+  const double s = fma(nu[3], E[3], fma(nu[4], E[4], nu[5] * E[5]));
+  gm[2] = fma(f, fma(2.0, s, fma(nu[6], E[6], fma(nu[7], E[7], nu[8] * E[8]))), gm[2]);
+}
+
 template <int N>
 __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     k_adj_cell_ck(const __grid_constant__ StepArgs A, const __grid_constant__ AdjArgs J,
@@ -412,6 +457,9 @@ __global__ void __launch_bounds__(256) k_adj_face_sum(const __grid_constant__ St
 //   ab_k = w_k F + f_k L^T nu_{k+1},   nu_{k+1} = (w_k / phi_k) lambda + ab_{k+1},   ab_{K+1} = 0,
 //   lambda^n = lambda + ab_0 (the levels of u),   material sum_k f_k nu_{k+1}^T (dL/dm) a_k,
 //   moment dt sbar lambda^T (dg/dM) + dt ab_0^T (dg/dM) (the levels of the source).
+// The material gradient pairs nu with the strains of a_k, kept from the forward levels: (L a_k would
+// have to be divided by mu and 3 lam + 2 mu, which a fluid and lam = -2/3 mu make zero; 1e-12 off at
+// mu = 1e-6 lam.  Same time, 5.8 ms for the gradient below.)
 // K + 1 applications of L and of L^T replace the recomputation and reversal of K iterations over
 // n time nodes (k_adj_cell, kept for the grids and iteration counts whose buffers do not fit: the
 // K + 2 records of a block's cells in shared memory, lambda's projections in the fixed array of
@@ -421,50 +469,55 @@ __global__ void __launch_bounds__(256) k_adj_face_sum(const __grid_constant__ St
 // Forward and reverse levels of one sequence whose first level is in the record 0 of `base` ([K + 2]
 // records).  w(k): weight of level k.  Adds sum_k w_k a_k to qb and the material terms to gm; ab
 // returns ab_0.  All threads of the block; act: the thread has a node of the sequence.
+// A level that every neighbour has read gives its record to its strains, which nu is paired with;
+// the last level's record, whose strains are paired at once, becomes nu's second buffer.
 template <int N, class W>
 __device__ __forceinline__ void adj_lin_levels(double* base, int K, bool act, int j, double dt,
                                                const double* phi, W w, const double (&Dr)[3][N + 1],
                                                const double (&DT)[3][N + 1],
-                                               const double (&cf)[3][4], double irho, double lam,
-                                               double ik, double imu, const double (&lam_j)[9],
-                                               const double (&Fj)[9], double (&qb)[9],
-                                               double (&gm)[3], double (&ab)[9]) {
+                                               const double (&cf)[3][4], const double* inv_h,
+                                               double irho, double lam, double mu,
+                                               const double (&lam_j)[9], const double (&Fj)[9],
+                                               double (&qb)[9], double (&gm)[3], double (&ab)[9]) {
   using C = CfgCKA<N>;
   constexpr int NV = C::NV, NVP = C::NVP, REC = C::REC;
-  double* const spare = base + (K + 1) * REC;
+  double* const last = base + K * REC;
+  double* const spare = last + REC;
 #pragma unroll 1
   for (int k = 0; k <= K; ++k) {
+    double E[NV];
     if (act) {
       const double* r = base + k * REC + j * NVP;
       const double wk = w(k);
 #pragma unroll
       for (int v = 0; v < NV; ++v) qb[v] = fma(wk, r[v], qb[v]);
-      double R[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) R[v] = 0.0;
-      ck_apply<N>(base + k * REC, j, Dr, cf, R);
+      ck_strains<N>(base + k * REC, j, Dr, inv_h, E);
       const double f = dt * (k < K ? phi[k] : 0.5);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) R[v] *= f;
       if (k < K) {
+        double R[NV];
+        ck_rows(E, f, irho, lam, mu, R);
 #pragma unroll
         for (int v = 0; v < NV; ++v) base[(k + 1) * REC + j * NVP + v] = R[v];
       } else {
-        // the last level's f_K L a_K (phi_K = 1/2), with nu_{K+1} = 2 w_K lambda
+        // the last level (phi_K = 1/2), with nu_{K+1} = 2 w_K lambda
         double nu[NV];
         double* o = spare + j * NVP;
 #pragma unroll
         for (int v = 0; v < NV; ++v) o[v] = nu[v] = 2.0 * wk * lam_j[v];
         o[9] = nu[3] + nu[4] + nu[5];
-        ck_dmat_R(R, nu, irho, lam, ik, imu, gm);
+        ck_dmat_E(E, nu, f, irho, gm);
       }
     }
     __syncthreads();
+    if (act && k < K) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) base[k * REC + j * NVP + v] = E[v];
+    }
   }
 #pragma unroll 1
   for (int k = K; k >= 0; --k) {
-    const double* Yin = ((K - k) & 1) ? base : spare;
-    double* Yout = ((K - k) & 1) ? spare : base;
+    const double* Yin = ((K - k) & 1) ? last : spare;
+    double* Yout = ((K - k) & 1) ? spare : last;
     if (act) {
       double Tt[NV];
 #pragma unroll
@@ -474,17 +527,14 @@ __device__ __forceinline__ void adj_lin_levels(double* base, int K, bool act, in
 #pragma unroll
       for (int v = 0; v < NV; ++v) ab[v] = fma(f, Tt[v], wk * Fj[v]);
       if (k > 0) {
-        // nu_k, and its pairing with f_{k-1} L a_{k-1} = a_k
+        // nu_k, and its pairing with the strains of a_{k-1}
         const double wl = w(k - 1) / phi[k - 1];
-        double nu[NV], P[NV];
+        double nu[NV];
         double* o = Yout + j * NVP;
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          o[v] = nu[v] = fma(wl, lam_j[v], ab[v]);
-          P[v] = base[k * REC + j * NVP + v];
-        }
+        for (int v = 0; v < NV; ++v) o[v] = nu[v] = fma(wl, lam_j[v], ab[v]);
         o[9] = nu[3] + nu[4] + nu[5];
-        ck_dmat_R(P, nu, irho, lam, ik, imu, gm);
+        ck_dmat_E(base + (k - 1) * REC + j * NVP, nu, dt * phi[k - 1], irho, gm);
       }
     }
     __syncthreads();
@@ -530,7 +580,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
   }
   const bool srcc = srcb && act && sc == slot;  // this thread's cell holds the source
   double Dr[3][n], DT[3][n], cf[3][4];
-  double irho = 0.0, lam = 0.0, ik = 0.0, imu = 0.0;
+  double irho = 0.0, lam = 0.0, mu = 0.0;
   if (act) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -543,9 +593,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     }
     irho = 1.0 / A.mat[c * 3 + 0];
     lam = A.mat[c * 3 + 1];
-    const double mu = A.mat[c * 3 + 2];
-    ik = 1.0 / (3.0 * lam + 2.0 * mu);
-    imu = 1.0 / mu;
+    mu = A.mat[c * 3 + 2];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const double ih = A.g.inv_h[d];
@@ -584,7 +632,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     __syncthreads();
     const double* sm = s_smp;
     adj_lin_levels<N>(base, K - 1, srcc, j, dt, phi, [&](int k) { return lin_gamma<N>(A, sm, k); }, Dr,
-                      DT, cf, irho, lam, ik, imu, lam_j, Fj, qb, gm, ab);
+                      DT, cf, A.g.inv_h, irho, lam, mu, lam_j, Fj, qb, gm, ab);
     if (srcc) {
 #pragma unroll
       for (int a = 0; a < 6; ++a) gM[a] = -ph * dt * fma(s_sbar, lam_j[3 + a], ab[3 + a]);
@@ -596,8 +644,8 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     smem[(size_t)s * NBUF * REC + (r / NV) * NVP + r % NV] = J.u_n[c0 * NL + e];
   }
   __syncthreads();
-  adj_lin_levels<N>(base, K, act, j, dt, phi, [&](int k) { return A.lin[k]; }, Dr, DT, cf, irho, lam,
-                    ik, imu, lam_j, Fj, qb, gm, ab);
+  adj_lin_levels<N>(base, K, act, j, dt, phi, [&](int k) { return A.lin[k]; }, Dr, DT, cf,
+                    A.g.inv_h, irho, lam, mu, lam_j, Fj, qb, gm, ab);
 
   // qbar (for the forward face data) into record 0, lambda^n = lambda + ab_0 into record 1, the
   // gradient terms of the nodes into record 2 (K >= 1), for coalesced stores and fixed-order sums

@@ -88,44 +88,48 @@ __device__ __forceinline__ double lin_gamma(const StepArgs& A, const double* s, 
   return g;
 }
 
+// Derivatives along direction d at node j of the cell record X ([NS][NVP]), times h_d: of the
+// velocities (dv) and of the stresses sigma_{id}, i = 0..2 (ds).  Dr[m] = D[j_d][m].
+template <int N>
+__device__ __forceinline__ void ck_derivs(const double* X, int j, int d, const double (&Dr)[N + 1],
+                                          double (&dv)[3], double (&ds)[3]) {
+  constexpr int n = N + 1, NVP = CfgCK<N>::NVP;
+  const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
+  const int jd = (j / st) % n;
+  const double* b = X + (j - jd * st) * NVP;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) dv[i] = ds[i] = 0.0;
+#pragma unroll
+  for (int m = 0; m < n; ++m) {
+    const double2* p = reinterpret_cast<const double2*>(b + m * st * NVP);
+    double r[NVP];
+#pragma unroll
+    for (int i = 0; i < NVP / 2; ++i) {
+      const double2 v = p[i];
+      r[2 * i] = v.x;
+      r[2 * i + 1] = v.y;
+    }
+    const double c = Dr[m];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      dv[i] = fma(c, r[i], dv[i]);
+      ds[i] = fma(c, r[Elastic::sig(i, d)], ds[i]);
+    }
+  }
+}
+
 // R[v] += row v of -sum_d (1/h_d) B_d D_d X at node j of the cell record X ([NS][NVP]).
 // Dr[d][m] = D[j_d][m];  cf[d] = {1/(rho h_d), (lam + 2 mu)/h_d, lam/h_d, mu/h_d}.
 template <int N>
 __device__ __forceinline__ void ck_apply(const double* X, int j, const double (&Dr)[3][N + 1],
                                          const double (&cf)[3][4], double (&R)[9]) {
-  constexpr int n = N + 1, NVP = CfgCK<N>::NVP;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
-    const int jd = (j / st) % n;
-    const double* b = X + (j - jd * st) * NVP;
-    // stress components sigma_{id}, i = 0..2
-    const int s0 = Elastic::sig(0, d), s1 = Elastic::sig(1, d), s2 = Elastic::sig(2, d);
-    double dv0 = 0.0, dv1 = 0.0, dv2 = 0.0, ds0 = 0.0, ds1 = 0.0, ds2 = 0.0;
+    double dv[3], ds[3];
+    ck_derivs<N>(X, j, d, Dr[d], dv, ds);
+    // velocities: (1/rho) d sigma_{id} / dx_d; normal stresses: (lam + 2 mu [i == d]) dv_d / dx_d
 #pragma unroll
-    for (int m = 0; m < n; ++m) {
-      const double2* p = reinterpret_cast<const double2*>(b + m * st * NVP);
-      double r[NVP];
-#pragma unroll
-      for (int i = 0; i < NVP / 2; ++i) {
-        const double2 v = p[i];
-        r[2 * i] = v.x;
-        r[2 * i + 1] = v.y;
-      }
-      const double c = Dr[d][m];
-      dv0 = fma(c, r[0], dv0);
-      dv1 = fma(c, r[1], dv1);
-      dv2 = fma(c, r[2], dv2);
-      ds0 = fma(c, r[s0], ds0);
-      ds1 = fma(c, r[s1], ds1);
-      ds2 = fma(c, r[s2], ds2);
-    }
-    const double dv[3] = {dv0, dv1, dv2};
-    // velocities: (1/rho) d sigma_{id} / dx_d
-    R[0] = fma(cf[d][0], ds0, R[0]);
-    R[1] = fma(cf[d][0], ds1, R[1]);
-    R[2] = fma(cf[d][0], ds2, R[2]);
-    // normal stresses: (lam + 2 mu [i == d]) dv_d / dx_d
+    for (int i = 0; i < 3; ++i) R[i] = fma(cf[d][0], ds[i], R[i]);
 #pragma unroll
     for (int i = 0; i < 3; ++i) R[3 + i] = fma(i == d ? cf[d][1] : cf[d][2], dv[d], R[3 + i]);
     // shear stresses: mu dv_s / dx_d with s = Elastic::src(d, v)
