@@ -17,11 +17,10 @@
 //   material   sum_{k=0..N} f_k nu_{k+1}^T (dL/dm) a_k
 //   moment     dt sbar lambda^T (dg/dM) + sum_{k<N} f_k s_k mu_{k+1}^T (dg/dM).
 // (dL/dm) a needs no contraction of its own: at a node, L a is the material coefficients times
-// ten derivative quantities (velocity rows (1/rho) S_i, normal-stress rows lam theta + 2 mu e_i,
-// shear rows mu gamma_v), so the derivatives with respect to (rho, lam, mu) follow from R = L a
-// itself: -R_i / rho; theta = sum_i R_{3+i} / (3 lam + 2 mu); 2 e_i = (R_{3+i} - lam theta) / mu;
-// gamma_v = R_v / mu.  For k < N, f_k L a_k = a_{k+1} - f_k s_k g is already at hand; L a_N costs
-// one application.
+// nine derivative quantities, the strains of a (velocity rows (1/rho) S_i, normal-stress rows
+// lam (e_0 + e_1 + e_2) + 2 mu e_i, shear rows mu gamma_v), from which the forward recursion forms
+// L a_k; they are kept for the reverse one (dividing L a by the material instead fails for a
+// fluid, mu = 0, and for 3 lam + 2 mu = 0).  L a_N costs one application.
 //
 // The forward face data the face terms' material gradient needs come from this kernel too (qbar
 // and its extrapolations, as the predictor forms them): the face adjoints, which need lambda and
@@ -29,9 +28,9 @@
 // gradients after it (MODE 2), so no forward predictor launch precedes the adjoint.
 //
 // One thread per node, the cells of a block (several at low order) each keep a_0 .. a_N in
-// shared memory ((N+2) padded records of 10 doubles per node; the record of a_0 and a spare one
-// hold the adjoint nu during the reverse sweep, the tenth double of a nu record its sum
-// nu_3 + nu_4 + nu_5), no global scratch.  Work per node: N+1 applications of L (the forward
+// shared memory ((N+2) padded records of 10 doubles per node; a level's strains take its record
+// once the neighbours have read it, the record of a_N and a spare one hold the adjoint nu during
+// the reverse sweep, the tenth double of a nu record its sum nu_3 + nu_4 + nu_5), no global scratch.  Work per node: N+1 applications of L (the forward
 // recursion and L a_N) and N+1 of L^T; the Picard adjoint recomputes and reverses N+1 iterations
 // over n time nodes.  The gradient sums are reduced in a fixed order (no atomics), so repeated
 // runs give identical bits.
@@ -52,7 +51,7 @@ struct CfgCKA {
   static constexpr int TPB = (CPB * NS + 31) / 32 * 32;
   static constexpr int NF = n * n;
   static constexpr int REC = NS * NVP;
-  static constexpr int NBUF = N + 2;  // a_0 (then nu) .. a_N, one more nu buffer
+  static constexpr int NBUF = N + 2;  // a_0 .. a_N (then nu), one more nu buffer
   static constexpr size_t SMEM = (size_t)CPB * NBUF * REC * sizeof(double);
 };
 
@@ -100,20 +99,6 @@ __device__ __forceinline__ void ck_apply_T(const double* Y, int j, const double 
     Out[Elastic::src(d, va)] = fma(cf[d][3], tsa, Out[Elastic::src(d, va)]);
     Out[Elastic::src(d, vb)] = fma(cf[d][3], tsb, Out[Elastic::src(d, vb)]);
   }
-}
-
-// gm += nu^T (dL/d(rho, lam, mu)) a at one node, given P = w L a there (any weight w: the result
-// carries the same factor).  irho = 1/rho, ik = 1/(3 lam + 2 mu), imu = 1/mu.
-__device__ __forceinline__ void ck_dmat_R(const double (&P)[9], const double (&nu)[9], double irho,
-                                          double lam, double ik, double imu, double (&gm)[3]) {
-  gm[0] = fma(-irho, fma(nu[0], P[0], fma(nu[1], P[1], nu[2] * P[2])), gm[0]);
-  const double theta = (P[3] + P[4] + P[5]) * ik;
-  const double nsum = nu[3] + nu[4] + nu[5];
-  gm[1] = fma(theta, nsum, gm[1]);
-  double s = fma(nu[3], P[3], fma(nu[4], P[4], nu[5] * P[5]));
-  s = fma(-lam * theta, nsum, s);
-  s = fma(nu[6], P[6], fma(nu[7], P[7], fma(nu[8], P[8], s)));
-  gm[2] = fma(imu, s, gm[2]);
 }
 
 // What the rows of L multiply by the material at node j: E_i = sum_d d sigma_{id} / dx_d (velocity
@@ -180,6 +165,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
   const long long c = c0 + slot;
   double* base = smem + (size_t)(act ? slot : 0) * NBUF * REC;  // a_k at base + k * REC
   double* const spare = base + (N + 1) * REC;
+  double* const last = base + N * REC;
   const double dt = A.dev->dt;
   const double tn = A.dev->t;
 
@@ -212,7 +198,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
   }
   const bool srcc = srcb && act && sc == slot;  // this thread's cell holds the source
   double Dr[3][n], DT[3][n], cf[3][4];
-  double irho = 0.0, lam = 0.0, ik = 0.0, imu = 0.0;
+  double irho = 0.0, lam = 0.0, mu = 0.0;
   if (act) {
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -225,9 +211,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     }
     irho = 1.0 / A.mat[c * 3 + 0];
     lam = A.mat[c * 3 + 1];
-    const double mu = A.mat[c * 3 + 2];
-    ik = 1.0 / (3.0 * lam + 2.0 * mu);
-    imu = 1.0 / mu;
+    mu = A.mat[c * 3 + 2];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const double ih = A.g.inv_h[d];
@@ -244,45 +228,77 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
   for (int a = 0; a < 6; ++a) mphi[a] = srcc ? -A.src.M[a] * phi : 0.0;
   __syncthreads();
 
-  // ---- forward recursion: a_1 .. a_N; then P = f_N L a_N at this node ------------------------
+  // ---- forward recursion: a_1 .. a_N and their strains; qbar = sum_k a_k / (k+1) at this node, summed
+  // in the predictor's order ---------------------------------------------------------------------
+  double qb[NV], E[NV];
+  if (act) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) qb[v] = base[j * NVP + v];
+  }
 #pragma unroll
   for (int k = 0; k < N; ++k) {
     if (act) {
       double R[NV];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) R[v] = 0.0;
-      ck_apply<N>(base + k * REC, j, Dr, cf, R);
+      const double f = dt * (1.0 / (k + 1)), wk = 1.0 / (k + 2);
+      ck_strains<N>(base + k * REC, j, Dr, A.g.inv_h, E);
+      ck_rows(E, f, irho, lam, mu, R);
       if (srcc) {
 #pragma unroll
-        for (int v = 3; v < NV; ++v) R[v] = fma(mphi[v - 3], s_sk[k], R[v]);
+        for (int v = 3; v < NV; ++v) R[v] = fma(mphi[v - 3], f * s_sk[k], R[v]);
       }
-      const double f = dt * (1.0 / (k + 1));
 #pragma unroll
-      for (int v = 0; v < NV; ++v) base[(k + 1) * REC + j * NVP + v] = f * R[v];
+      for (int v = 0; v < NV; ++v) {
+        base[(k + 1) * REC + j * NVP + v] = R[v];
+        qb[v] = fma(wk, R[v], qb[v]);
+      }
     }
     __syncthreads();
-  }
-  // forward face data of the step (the predictor's epilogue): qbar = sum_k a_k / (k+1) at this
-  // node, summed in the predictor's order, into the record of a_0 (each thread reads and writes
-  // its own node only), then extrapolated to both ends of every direction
-  if (act) {
-    double qb[NV];
+    if (act) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) qb[v] = base[j * NVP + v];
-#pragma unroll
-    for (int k = 1; k <= N; ++k) {
-      const double wk = 1.0 / (k + 1);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) qb[v] = fma(wk, base[k * REC + j * NVP + v], qb[v]);
+      for (int v = 0; v < NV; ++v) base[k * REC + j * NVP + v] = E[v];
     }
+  }
+  double lam_j[NV], Fj[NV];
+  double gm[3] = {0.0, 0.0, 0.0}, gM[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  if (act) {
+    // lambda at this node; its stress sum into the tenth slot of the record; its pairing with the
+    // strains of a_N
+    double* lr = spare + j * NVP;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) base[j * NVP + v] = qb[v];
+    for (int v = 0; v < NV; ++v) lam_j[v] = lr[v];
+    lr[9] = lam_j[3] + lam_j[4] + lam_j[5];
+    ck_strains<N>(last, j, Dr, A.g.inv_h, E);
+    ck_dmat_E(E, lam_j, dt * (1.0 / (N + 1)), irho, gm);
+    // F: the face adjoints carried back to the nodes (transposed extrapolation)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Fj[v] = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
+      const int jd = (j / st) % n;
+      const int jp = (j % st) + (j / (st * n)) * st;
+      const double* af = J.adjf + (c * 3 + d) * 2 * (long long)(NF * NV) + jp * NV;
+      const double e0 = T.e0[jd], e1 = T.e1[jd];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Fj[v] = fma(e0, af[v], fma(e1, af[NF * NV + v], Fj[v]));
+    }
+  }
+  if (srcc) {
+#pragma unroll
+    for (int a = 0; a < 6; ++a) gM[a] = -phi * dt * s_sbar * lam_j[3 + a];
+  }
+  __syncthreads();  // a_N is read; lambda's stress sums are read by the neighbours below
+  // forward face data of the step (the predictor's epilogue): qbar extrapolated to both ends of every
+  // direction
+  if (act) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) last[j * NVP + v] = qb[v];
   }
   __syncthreads();
   for (int e = tid; e < ncb * NF * NV; e += TPB) {
     const int s = e / (NF * NV), r = e - s * (NF * NV);
     const int v = r % NV, jp = r / NV;
-    const double* Xs = smem + (size_t)s * NBUF * REC;
+    const double* Xs = smem + (size_t)s * NBUF * REC + N * REC;
     double* fc = A.face + (c0 + s) * (3 * 2 * NF * NV) + jp * NV + v;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
@@ -299,67 +315,29 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
       fc[(d * 2 + 1) * NF * NV] = q1;
     }
   }
-  double P[NV];  // f_k L a_k at this node, for the level being reversed
-  double lam_j[NV], Fj[NV];
-  if (act) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) P[v] = 0.0;
-    ck_apply<N>(base + N * REC, j, Dr, cf, P);
-    const double fN = dt * (1.0 / (N + 1));
-#pragma unroll
-    for (int v = 0; v < NV; ++v) P[v] *= fN;
-    // lambda at this node; its stress sum into the tenth slot of the record
-    double* lr = spare + j * NVP;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) lam_j[v] = lr[v];
-    lr[9] = lam_j[3] + lam_j[4] + lam_j[5];
-    // F: the face adjoints carried back to the nodes (transposed extrapolation)
-#pragma unroll
-    for (int v = 0; v < NV; ++v) Fj[v] = 0.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
-      const int jd = (j / st) % n;
-      const int jp = (j % st) + (j / (st * n)) * st;
-      const double* af = J.adjf + (c * 3 + d) * 2 * (long long)(NF * NV) + jp * NV;
-      const double e0 = T.e0[jd], e1 = T.e1[jd];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Fj[v] = fma(e0, af[v], fma(e1, af[NF * NV + v], Fj[v]));
-    }
-  }
-  double gm[3] = {0.0, 0.0, 0.0}, gM[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  if (srcc) {
-#pragma unroll
-    for (int a = 0; a < 6; ++a) gM[a] = -phi * dt * s_sbar * lam_j[3 + a];
-  }
-  __syncthreads();  // lambda's stress sums are read by the neighbours below
+  __syncthreads();  // the record becomes a nu buffer
 
   // ---- reverse recursion on nu_k = lambda + mu_k ---------------------------------------------
-  // nu_{k+1} is read from Yin: the spare record at k = N, then alternately the record of a_0 and
-  // the spare one (a_0 is not read after the forward recursion).
+  // nu_{k+1} is read from Yin: the spare record at k = N, then alternately the record of a_N and
+  // the spare one.
   double nu_c[NV];  // nu_{k+1} at this node
 #pragma unroll
   for (int v = 0; v < NV; ++v) nu_c[v] = lam_j[v];
 #pragma unroll
   for (int k = N; k >= 0; --k) {
-    const double* Yin = ((N - k) & 1) ? base : spare;
-    double* Yout = ((N - k) & 1) ? spare : base;
+    const double* Yin = ((N - k) & 1) ? last : spare;
+    double* Yout = ((N - k) & 1) ? spare : last;
     if (act) {
-      // material: f_k nu_{k+1}^T (dL/dm) a_k, from P = f_k L a_k at this node
-      if (k < N) {
+      if (k < N) {  // material: f_k nu_{k+1}^T (dL/dm) a_k from the strains of a_k
         const double f = dt * (1.0 / (k + 1));
-#pragma unroll
-        for (int v = 0; v < NV; ++v) P[v] = base[(k + 1) * REC + j * NVP + v];
+        ck_dmat_E(base + k * REC + j * NVP, nu_c, f, irho, gm);
         if (srcc) {
+          // moment: f_k s_k mu_{k+1}^T (dg/dM), mu_{k+1} = nu_{k+1} - lambda
 #pragma unroll
-          for (int a = 0; a < 6; ++a) {
-            P[3 + a] = fma(-f * s_sk[k], mphi[a], P[3 + a]);
-            // moment: f_k s_k mu_{k+1}^T (dg/dM), mu_{k+1} = nu_{k+1} - lambda
+          for (int a = 0; a < 6; ++a)
             gM[a] = fma(-phi * f * s_sk[k], nu_c[3 + a] - lam_j[3 + a], gM[a]);
-          }
         }
       }
-      ck_dmat_R(P, nu_c, irho, lam, ik, imu, gm);
       double Tt[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) Tt[v] = 0.0;
@@ -376,8 +354,8 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     }
     if (k > 0) __syncthreads();
   }
-  // lambda^n = nu_0 (+ dJ/du^n), staged in the record of a_1 for a coalesced store (a_1 is last
-  // read at level 0, before the barrier below)
+  // lambda^n = nu_0 (+ dJ/du^n), staged in record 1 for a coalesced store (its strains are last read
+  // at level 1, before the barrier below)
   __syncthreads();
   if (act) {
 #pragma unroll
@@ -457,9 +435,8 @@ __global__ void __launch_bounds__(256) k_adj_face_sum(const __grid_constant__ St
 //   ab_k = w_k F + f_k L^T nu_{k+1},   nu_{k+1} = (w_k / phi_k) lambda + ab_{k+1},   ab_{K+1} = 0,
 //   lambda^n = lambda + ab_0 (the levels of u),   material sum_k f_k nu_{k+1}^T (dL/dm) a_k,
 //   moment dt sbar lambda^T (dg/dM) + dt ab_0^T (dg/dM) (the levels of the source).
-// The material gradient pairs nu with the strains of a_k, kept from the forward levels: (L a_k would
-// have to be divided by mu and 3 lam + 2 mu, which a fluid and lam = -2/3 mu make zero; 1e-12 off at
-// mu = 1e-6 lam.  Same time, 5.8 ms for the gradient below.)
+// The material gradient pairs nu with the strains of a_k as above (L a_k divided by the material was
+// 1e-12 off at mu = 1e-6 lam; the time is the same, 5.8 ms for the gradient below).
 // K + 1 applications of L and of L^T replace the recomputation and reversal of K iterations over
 // n time nodes (k_adj_cell, kept for the grids and iteration counts whose buffers do not fit: the
 // K + 2 records of a block's cells in shared memory, lambda's projections in the fixed array of

@@ -48,3 +48,9 @@ def check(order, lam, mu, predictor, source, static):
 @pytest.mark.parametrize("order", [1, 2, 3, 4, 5])
 def test_picard(order, lam, mu):
     check(order, lam, mu, "picard", source=order % 2 == 1, static=order == 2)
+
+
+@pytest.mark.parametrize("lam,mu", MATERIALS)
+@pytest.mark.parametrize("order", [1, 2, 3, 4, 5])
+def test_ck(order, lam, mu):
+    check(order, lam, mu, "ck", source=order % 2 == 1, static=order == 2)
