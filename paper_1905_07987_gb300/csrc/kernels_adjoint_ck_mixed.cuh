@@ -135,8 +135,8 @@ __device__ __forceinline__ void ck_apply_T_f(const float* Y, int j, const float2
   }
 }
 
-// Binary32 form of ck_dmat_R: the three sums of nu^T (dL/d(rho, lam, mu)) a before the material
-// factors, g[0] = sum_i nu_i P_i, g[1] = theta (nu_3 + nu_4 + nu_5) with theta = (P_3 + P_4 +
+// The three sums of nu^T (dL/d(rho, lam, mu)) a before the material factors, from P = w L a (any
+// weight w: the result carries the same factor), in binary32: g[0] = sum_i nu_i P_i, g[1] = theta (nu_3 + nu_4 + nu_5) with theta = (P_3 + P_4 +
 // P_5) ik, g[2] = sum nu_v P_v - lam theta (nu_3 + nu_4 + nu_5) over the stress rows.
 __device__ __forceinline__ void ck_dmat_R_f(const float (&P)[9], const float (&nu)[9], float lam,
                                             float ik, float (&g)[3]) {
@@ -165,6 +165,55 @@ __device__ __forceinline__ void ck_dmat_R_ff(const ff (&P)[9], const ff (&nu)[9]
   g[2] = ff_sub(s, lt);
 }
 
+// P divided by the material is off by lam / mu, and by (lam + 2 mu) / (3 lam + 2 mu), times the rounding,
+// and a fluid (mu = 0) divides by zero: cells where either is above 64 form the sums from the strains
+// of a (ck_strains), one more application of the derivatives per level, in S.  X: the level's
+// records, STRIDE values a node.  gm += f nu^T (dL/d(rho, lam, mu)) a.  Not inlined: its registers
+// do not add to the other cells'.
+__device__ __forceinline__ bool ck_divides(double lam, double mu) {
+  const double m = 0.015625 * (lam + 2.0 * mu);
+  return mu >= m && fabs(3.0 * lam + 2.0 * mu) >= m;
+}
+template <int N, class S, int STRIDE>
+__device__ __noinline__ void ck_dmat_strains(const S* X, int j, const Tables& T, const double* inv_h,
+                                             const S* nu, double f, double irho, double* gm) {
+  constexpr int n = N + 1;
+  S E[9];
+#pragma unroll
+  for (int v = 0; v < 9; ++v) E[v] = 0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int st = d == 0 ? 1 : (d == 1 ? n : n * n);
+    const int jd = (j / st) % n;
+    const S* b = X + (j - jd * st) * STRIDE;
+    const S ih = (S)inv_h[d];
+    S dv[3] = {0, 0, 0}, ds[3] = {0, 0, 0};
+    for (int m = 0; m < n; ++m) {
+      const S c = (S)T.D[jd][m];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        dv[i] += c * b[m * st * STRIDE + i];
+        ds[i] += c * b[m * st * STRIDE + Elastic::sig(i, d)];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) E[i] += ih * ds[i];
+    E[3 + d] = ih * dv[d];
+#pragma unroll
+    for (int v = 6; v < 9; ++v) {
+      const int s = Elastic::src(d, v);
+      if (s >= 0) E[v] += ih * dv[s];
+    }
+  }
+  const S r = nu[0] * E[0] + nu[1] * E[1] + nu[2] * E[2];
+  const S l = (nu[3] + nu[4] + nu[5]) * (E[3] + E[4] + E[5]);
+  const S s = nu[3] * E[3] + nu[4] * E[4] + nu[5] * E[5];
+  const S m = 2 * s + nu[6] * E[6] + nu[7] * E[7] + nu[8] * E[8];
+  gm[0] = fma(-f * irho * irho, (double)r, gm[0]);
+  gm[1] = fma(f, (double)l, gm[1]);
+  gm[2] = fma(f, (double)m, gm[2]);
+}
+
 template <int N>
 __global__ void __launch_bounds__(CfgCKAM<N>::TPB, CfgCKAM<N>::MINB)
     k_adj_cell_ck_mixed(const __grid_constant__ StepArgs A, const __grid_constant__ AdjArgs J,
@@ -175,6 +224,7 @@ __global__ void __launch_bounds__(CfgCKAM<N>::TPB, CfgCKAM<N>::MINB)
   extern __shared__ __align__(16) unsigned char smem_am[];  // [CPB][CELL] + g
   __shared__ ff s_cf[CPB][3][4];
   __shared__ double s_mat[CPB][4];  // 1/rho, lam, 1/(3 lam + 2 mu), 1/mu
+  __shared__ bool s_div[CPB];       // the material gradient from L a divided by the material
   __shared__ ff s_skf[n], s_sbarf;
   __shared__ double s_sk[n], s_sbar;
   __shared__ int s_slot;
@@ -219,6 +269,7 @@ __global__ void __launch_bounds__(CfgCKAM<N>::TPB, CfgCKAM<N>::MINB)
     s_mat[tid][1] = lam;
     s_mat[tid][2] = 1.0 / (3.0 * lam + 2.0 * mu);
     s_mat[tid][3] = 1.0 / mu;
+    s_div[tid] = ck_divides(lam, mu);
   }
   const long long sc = A.src.cell - c0;
   const bool srcb = sc >= 0 && sc < ncb;
@@ -386,6 +437,25 @@ __global__ void __launch_bounds__(CfgCKAM<N>::TPB, CfgCKAM<N>::MINB)
   double gm[3] = {0.0, 0.0, 0.0}, gM[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   const double irho = act ? s_mat[slot][0] : 0.0, lamd = act ? s_mat[slot][1] : 0.0;
   const double ikd = act ? s_mat[slot][2] : 0.0, imud = act ? s_mat[slot][3] : 0.0;
+  const bool divides = act && s_div[slot];
+  // level k from the strains of a_k, its records of S at X (see ck_dmat_strains)
+  const auto strains = [&](int k, const float* X, const ff (&nu)[NV]) {
+    double g[3] = {0.0, 0.0, 0.0};
+    const double f = dt * (1.0 / (k + 1));
+    if (k == 0) {
+      double x[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) x[v] = ff_to_d(nu[v]);
+      ck_dmat_strains<N, double, NV>(J.u_n + c * NL, j, T, A.g.inv_h, x, f, irho, g);
+    } else {
+      float x[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) x[v] = nu[v].h;
+      ck_dmat_strains<N, float, NVF>(X, j, T, A.g.inv_h, x, f, irho, g);
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) gm[q] += g[q];
+  };
   const float lamf = (float)lamd, ikf = (float)ikd;
   const ff lamff = ff_split(lamd), ikff = ff_split(ikd);
   const double phi = srcc ? A.src.phi[j] : 0.0;
@@ -398,13 +468,17 @@ __global__ void __launch_bounds__(CfgCKAM<N>::TPB, CfgCKAM<N>::MINB)
 #pragma unroll
     for (int v = 0; v < NV; ++v) B[v] = ff_add(Fj[v], ff_mul(dtf, LT[v]));
     // level N: f_N lambda^T (dL/dm) a_N
-    float nu[NV], g[3];
+    if (divides) {
+      float nu[NV], g[3];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) nu[v] = lj[v].h;
-    ck_dmat_R_f(PN, nu, lamf, ikf, g);
-    gm[0] = -irho * (double)g[0];
-    gm[1] = (double)g[1];
-    gm[2] = imud * (double)g[2];
+      for (int v = 0; v < NV; ++v) nu[v] = lj[v].h;
+      ck_dmat_R_f(PN, nu, lamf, ikf, g);
+      gm[0] = -irho * (double)g[0];
+      gm[1] = (double)g[1];
+      gm[2] = imud * (double)g[2];
+    } else {
+      strains(N, Arec + (N - 1) * NS * NVF, lj);
+    }
     if (srcc) {
 #pragma unroll
       for (int a = 0; a < 6; ++a) gM[a] = -phi * dt * s_sbar * ff_to_d(lj[3 + a]);
@@ -427,7 +501,12 @@ __global__ void __launch_bounds__(CfgCKAM<N>::TPB, CfgCKAM<N>::MINB)
     if (act) {
       const double f = dt * (1.0 / (k + 1));
       // material: f_k (lambda + mu_{k+1})^T (dL/dm) a_k
-      if (k == 0) {
+      if (!divides) {
+        ff nu[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) nu[v] = ff_add(lj[v], mu_c[v]);
+        strains(k, Arec + (k - 1) * NS * NVF, nu);
+      } else if (k == 0) {
         // float-float from a_1 and lambda + mu_1, the material factors in FP64
         ff P[NV], nu[NV];
 #pragma unroll

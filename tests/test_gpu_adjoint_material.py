@@ -18,12 +18,13 @@ def device(a):
     return torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).cuda()
 
 
-def check(order, lam, mu, predictor, source, static):
+def check(order, lam, mu, predictor, source, static, precision="fp64", tol=1e-12):
     nc = (3, 2, 2)
     mat = synth.elastic_material(nc, seed=order)
     mat[::2, 1] = lam  # the other cells keep an ordinary material
     mat[::2, 2] = mu
-    c = Case("elastic", 3, order, nc, hi=(1.5, 1.0, 1.0), bc="absorbing", material=mat, predictor=predictor)
+    c = Case("elastic", 3, order, nc, hi=(1.5, 1.0, 1.0), bc="absorbing", material=mat, predictor=predictor,
+             precision=precision)
     if source:
         c.point_source([0.3, 0.2, 0.3], synth.moment_tensor(5), 2.0, 0.4)
     rng = np.random.default_rng(order)
@@ -38,7 +39,9 @@ def check(order, lam, mu, predictor, source, static):
     out = (lam_d.cpu().numpy(), gm.cpu().numpy(), gM.cpu().numpy())
     for a, b in zip(out, ref):
         b = b.numpy().reshape(-1)
-        assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+        assert np.abs(a - b).max() <= tol * np.abs(b).max()
+    if precision != "fp64":
+        return
     # each material parameter by its own size too
     a, b = gm.cpu().numpy().reshape(-1, 3), ref[1].numpy()
     assert (np.abs(a - b).max(axis=0) <= 1e-12 * np.abs(b).max(axis=0)).all()
@@ -54,3 +57,10 @@ def test_picard(order, lam, mu):
 @pytest.mark.parametrize("order", [1, 2, 3, 4, 5])
 def test_ck(order, lam, mu):
     check(order, lam, mu, "ck", source=order % 2 == 1, static=order == 2)
+
+
+# binary32 levels: a few of its roundings relative to the largest value, on states that are not smooth
+@pytest.mark.parametrize("lam,mu", MATERIALS)
+@pytest.mark.parametrize("order", [1, 2, 3, 4, 5])
+def test_ck_mixed(order, lam, mu):
+    check(order, lam, mu, "ck", source=order % 2 == 1, static=order == 2, precision="mixed", tol=2e-6)
