@@ -904,7 +904,8 @@ __global__ void __launch_bounds__(256) k_corrector(const __grid_constant__ StepA
 // The 6 n^2 fluxes of a cell and variable share a power of two (their largest exponent), are
 // converted once, each used by the n nodes of its line, and the six products of a node are summed
 // as integers (2^-56 of the largest flux times the largest weight, far below the rounding of
-// u); FP64 adds the sum to u.  A variable with a non-finite flux takes the FP64 form.
+// u); FP64 adds the sum to u.  A variable with a non-finite flux, or whose sum could pass binary64's
+// range (six products below 2^(E + Ew - 2044)), takes the FP64 form, where it overflows to infinity.
 // A thread has the n degrees of freedom of a line along z: the x and y weights and the two z
 // fluxes stay in its registers, and the line's index also names one value of every face, so the
 // same thread loads and converts these six.
@@ -1019,7 +1020,7 @@ __device__ __forceinline__ void corrector_cells(const StepArgs& A, SmemC<P, D, N
         const fx2 t = S.w[(side * D + d) * n + m];
         return fx3{t.h, t.l, 0};
       };
-      if (CfgC<P, D, N>::FX && E != 0x7ff) {
+      if (CfgC<P, D, N>::FX && E != 0x7ff && E + Ew <= 3060) {
         const fx3 x0 = w(0, 0, a), x1 = w(1, 0, a), y0 = w(0, 1, b), y1 = w(1, 1, b);
         const fx2* px = &S.phi[s][0][b * NV + v];
         const fx2* py = &S.phi[s][2][a * NV + v];
