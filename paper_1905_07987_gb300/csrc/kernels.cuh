@@ -904,8 +904,9 @@ __global__ void __launch_bounds__(256) k_corrector(const __grid_constant__ StepA
 // The 6 n^2 fluxes of a cell and variable share a power of two (their largest exponent), are
 // converted once, each used by the n nodes of its line, and the six products of a node are summed
 // as integers (2^-56 of the largest flux times the largest weight, far below the rounding of
-// u); FP64 adds the sum to u.  A variable with a non-finite flux, or whose sum could pass binary64's
-// range (six products below 2^(E + Ew - 2044)), takes the FP64 form, where it overflows to infinity.
+// u); FP64 adds the sum to u.  A variable with a non-finite flux takes the FP64 form, and one whose six
+// products, below 2^(E + Ew - 2044) and summed in units of 2^(E + Ew - 2104), could pass binary64's
+// range or fall out of it below (or all of its fluxes are below 2^-822; zeros stay).
 // A thread has the n degrees of freedom of a line along z: the x and y weights and the two z
 // fluxes stay in its registers, and the line's index also names one value of every face, so the
 // same thread loads and converts these six.
@@ -963,6 +964,7 @@ struct SmemC {
   fx2 w[2 * D * (N + 1)];
   const double* face[CPB][2 * D];
   int e[CPB][P::NV];
+  int tiny[CPB][P::NV];  // every flux is below 2^-822, and not all are zero (or subnormal)
 };
 
 // Cells c0 .. c0 + ncb - 1 of a context (ncb <= CPB), all NT threads of the block, after
@@ -974,7 +976,10 @@ __device__ __forceinline__ void corrector_cells(const StepArgs& A, SmemC<P, D, N
   using C = Cfg<P, D, N>;
   constexpr int n = C::n, NV = C::NV, NL = C::NL, LINES = CfgC<P, D, N>::LINES;
   constexpr int RND = (CPB * LINES + NT - 1) / NT;  // lines per thread
-  for (int i = tid; i < ncb * NV; i += NT) (&S.e[0][0])[i] = 200;
+  for (int i = tid; i < ncb * NV; i += NT) {
+    (&S.e[0][0])[i] = 200;
+    (&S.tiny[0][0])[i] = 0;
+  }
   for (int i = tid; i < ncb * 2 * D; i += NT)
     (&S.face[0][0])[i] = face_flux<P, D, N>(A, c0 + i / (2 * D), i % (2 * D), off1, off2);
   __syncthreads();
@@ -1005,6 +1010,7 @@ __device__ __forceinline__ void corrector_cells(const StepArgs& A, SmemC<P, D, N
         const fx2 p = fx_split(fx_in(x[k][f], E, over));
         if (f < 4) S.phi[s][f][q] = p;
         else z[k][f - 4] = p;
+        if (E == 200 && (__double2hiint(x[k][f]) & 0x7ff00000)) S.tiny[s][q % NV] = 1;
       }
     }
   }
@@ -1020,7 +1026,8 @@ __device__ __forceinline__ void corrector_cells(const StepArgs& A, SmemC<P, D, N
         const fx2 t = S.w[(side * D + d) * n + m];
         return fx3{t.h, t.l, 0};
       };
-      if (CfgC<P, D, N>::FX && E != 0x7ff && E + Ew <= 3060) {
+      const bool fit = E != 0x7ff && (unsigned)(E + Ew - 1100) <= 1960u && !(E == 200 && S.tiny[s][v]);
+      if (CfgC<P, D, N>::FX && fit) {
         const fx3 x0 = w(0, 0, a), x1 = w(1, 0, a), y0 = w(0, 1, b), y1 = w(1, 1, b);
         const fx2* px = &S.phi[s][0][b * NV + v];
         const fx2* py = &S.phi[s][2][a * NV + v];

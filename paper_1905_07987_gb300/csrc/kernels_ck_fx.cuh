@@ -16,7 +16,8 @@
 // Scale: one power of two per cell, velocities and stresses related by the power of two nearest
 // the impedance rho vp: nodal values below 2^57, parity values (sums of eight) below 2^60.  The
 // levels shrink at stable time steps; a value that leaves 2^60, a coefficient that does not fit, a
-// non-finite value, and the cell with the point source send the block to the FP64 form.  Rounding:
+// non-finite value, a cell of values near an end of binary64's range (all below 2^-722, but not all
+// zero), and the cell with the point source send the block to the FP64 form.  Rounding:
 // 2^-57 of the cell's largest value in the conversion, less in each level (every product takes its
 // low words too), where FP64 rounds each operation at 2^-53.
 //
@@ -63,6 +64,13 @@ __device__ __forceinline__ void fx_octet(long long (&x)[8]) {
         x[i] = a + b;
         x[i | s] = a - b;
       }
+}
+
+// Negative when a cell's values, all small, are not all zero (or subnormal): a quiet cell stays.
+static __device__ __noinline__ int fxe_tiny(const double* x, int j, int n, int step) {
+  int t = 0;
+  for (int r = j; r < n; r += step) t |= __double2hiint(x[r]) & 0x7ff00000;
+  return -t;
 }
 
 // The lines of thread j of a cell, the same in every level: place of the first node in the level (12
@@ -302,7 +310,9 @@ __device__ __forceinline__ bool predictor_elastic_fx(const StepArgs& A, const Ta
   }
   __syncthreads();
   const int Ec = s_e[act ? slot : 0];
-  if (Ec > 1900) over = -1;  // results near the end of binary64's range
+  if (Ec > 1900) over = -1;  // results near an end of binary64's range
+  // (the mixed form's node form loses values below 2^-126, as its float-float pairs do)
+  if (!MIXED && act && Ec < 300) over |= fxe_tiny(stage, j, NL, NS);
   // octets of mirrored nodes: into fixed point and the parity basis
   if (act) {
     for (int g = j; g < NV * M * M * M; g += NS) {

@@ -231,8 +231,8 @@ __device__ __noinline__ void project_P_plain(const double* u, double* t1, double
 // below 2^57, rows of P1 of sum below 2 after the host's scaling, so nothing passes 2^60 in three
 // passes.  The conversion truncates at 2^-57 of the largest value and each pass rounds at 2^-57
 // to 2^-56 of it, where each FP64 FMA rounds at 2^-53 of its partial sum.  Min and max are taken of
-// the integers, whose order fx_out keeps.  Non-finite values and such near the end of binary64's
-// range: the FP64 form.
+// the integers, whose order fx_out keeps.  Non-finite values and such near an end of binary64's
+// range (a variable whose values are all below 2^-822, but not all zero): the FP64 form.
 //
 // Measured, 64^3 cells of order 3: k_lim_detect 8.8 -> 3.85 ms, k_lim_init 7.6 -> 2.97 ms (with the
 // integer contractions but min, max and the copy taken from shared memory afterwards 4.47 and 3.55).
@@ -247,10 +247,10 @@ __device__ __forceinline__ void project_P(const double* u, double* t1, double* t
   static_assert(RV <= 32 && 2 * PER <= 2 * NV * 32, "one warp reduces a variable");
   __shared__ int s_E[NV];
   const int tid = threadIdx.x, v = tid % NV, lane = tid & 31;
-  if (tid < NV) s_E[tid] = 200;
+  if (tid < NV) s_E[tid] = 0;
   __syncthreads();
   if (tid < PER) {
-    int E = 200;
+    int E = 0;
     for (int e = tid; e < NN * NV; e += PER)
       E = max(E, (int)(((unsigned)__double2hiint(u[e]) >> 20) & 0x7ffu));
     atomicMax(&s_E[v], E);
@@ -258,14 +258,14 @@ __device__ __forceinline__ void project_P(const double* u, double* t1, double* t
   __syncthreads();
   bool big = false;
 #pragma unroll
-  for (int i = 0; i < NV; ++i) big = big || s_E[i] > 1900;
+  for (int i = 0; i < NV; ++i) big = big || s_E[i] > 1900 || (unsigned)(s_E[i] - 1) < 199u;
   if (big) {
     project_P_plain<D, N>(u, t1, t2, out, S);
     for (int e = tid; e < NSS * NV; e += L::TPB) rep[e] = out[e];
     block_keys<NSS, NV>(out, key, red);
     return;
   }
-  const int E = s_E[v];
+  const int E = max(s_E[v], 200);
   long long lo = LLONG_MAX, hi = LLONG_MIN;
   if constexpr (D == 2) {
     contract_axis_fx<n, ns, n, NV, NV, true, false>(u, t1, rep, PER, E, S, lo, hi);
@@ -289,7 +289,7 @@ __device__ __forceinline__ void project_P(const double* u, double* t1, double* t
     long long r = mx ? LLONG_MIN : LLONG_MAX;
     if (lane < RV) r = red[(mx ? PER : 0) + i + lane * NV];
     r = mx ? warp_max(r) : warp_min(r);
-    if (lane == 0) key[k] = okey(fx_out(r, s_E[i] + S.kx));
+    if (lane == 0) key[k] = okey(fx_out(r, max(s_E[i], 200) + S.kx));
   }
   __syncthreads();
 }
