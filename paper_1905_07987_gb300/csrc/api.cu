@@ -315,17 +315,19 @@ void build_tables_e(int order, const Tables& T, TablesE& X) {
 // G_{k+1} <- Kw G_k, G_0 <- Kw.  So after `iters` iterations the first `iters` levels are powers of
 // Kw and the guess's own coefficients follow, multiplied by Kw^iters.  Stored: the time averages
 // of the coefficients of the scaled levels a_k = (prod_{i<k} phi_i) Lambda^k u with phi_0 = 1 and
-// phi_k = 1/2 after it (the spectral radius of Kw is below 0.41: the scaled weights fall).
-std::vector<double> build_linear_levels(int order, const Tables& T, int iters, bool cerk) {
+// phi_k = 1/2 after it (the spectral radius of Kw is below 0.41: the scaled weights fall).  The
+// scaling is part of the recursion, Kw / phi_k, so that any number of iterations stays in range, and
+// the levels end where every weight left is below 2^-1000.  `levels`: their number.
+std::vector<double> build_linear_levels(int order, const Tables& T, int iters, bool cerk, int* levels) {
   const int n = order + 1, ns = n + 3;
   typedef std::vector<double> Vec;
   const auto phi = [](int k) { return k == 0 ? 1.0 : 0.5; };
-  const auto times_kw = [&](const Vec& a) {  // a[t][..] -> sum_m Kw[t][m] a[m][..]
+  const auto times_kw = [&](const Vec& a, double f) {  // a[t][..] -> sum_m Kw[t][m] a[m][..] / f
     const size_t w = a.size() / n;
     Vec b(a.size(), 0.0);
     for (int t = 0; t < n; ++t)
       for (int m = 0; m < n; ++m)
-        for (size_t i = 0; i < w; ++i) b[t * w + i] += T.Kw[t][m] * a[m * w + i];
+        for (size_t i = 0; i < w; ++i) b[t * w + i] += T.Kw[t][m] / f * a[m * w + i];
     return b;
   };
   // the guess: coefficients of u (C0[k][t]) and of the source (G0[k][t][m])
@@ -352,42 +354,53 @@ std::vector<double> build_linear_levels(int order, const Tables& T, int iters, b
       }
     }
   }
-  // levels of q after the iterations
-  const size_t K = (size_t)iters + C0.size() - 1;
-  std::vector<double> out(2 * K + 1 + K * ns, 0.0);
-  double scale = 1.0;  // 1 / prod phi
   const auto average = [&](const Vec& a, size_t w, size_t i) {
     double s = 0.0;
     for (int t = 0; t < n; ++t) s += T.w[t] * a[t * w + i];
     return s;
+  };
+  const auto gone = [](const Vec& a) {
+    for (double x : a)
+      if (std::fabs(x) >= 0x1p-1000) return false;
+    return true;
+  };
+  const auto all_gone = [&](const std::vector<Vec>& v) {
+    for (const Vec& a : v)
+      if (!gone(a)) return false;
+    return true;
   };
   Vec c(n, 1.0), g((size_t)n * ns, 0.0);
   for (int t = 0; t < n; ++t)
     for (int m = 0; m < n; ++m) g[(size_t)t * ns + m] = T.Kw[t][m];
   // the guess's levels carry Kw^iters times what follows Lambda^iters
   std::vector<Vec> Ct = C0, Gt = G0;
-  for (int it = 0; it < iters; ++it) {
-    for (Vec& a : Ct) a = times_kw(a);
-    for (Vec& a : Gt) a = times_kw(a);
+  for (int it = 0; it < iters && !(all_gone(Ct) && all_gone(Gt)); ++it) {
+    for (Vec& a : Ct) a = times_kw(a, phi(it));
+    for (Vec& a : Gt) a = times_kw(a, phi(it));
   }
+  // levels of q after the iterations
+  const size_t it = (size_t)iters;
+  size_t K = it + C0.size() - 1;
+  Vec wk, wg;          // weights of the levels, of the samples
+  double scale = 1.0;  // 1 / prod phi from level `iters` on
   for (size_t k = 0; k <= K; ++k) {
-    if (k < (size_t)iters) {
-      out[k] = scale * average(c, 1, 0);
-      c = times_kw(c);
-    } else {
-      out[k] = scale * average(Ct[k - iters], 1, 0);
-    }
+    wk.push_back(k < it ? average(c, 1, 0) : scale * average(Ct[k - it], 1, 0));
+    if (k < it && k > 0 && gone(c) && gone(g) && all_gone(Ct) && all_gone(Gt)) K = k;
     if (k == K) break;
-    out[K + 1 + k] = phi((int)k);
-    if (k < (size_t)iters) {
-      for (int m = 0; m < ns; ++m) out[2 * K + 1 + k * ns + m] = scale * average(g, ns, m);
-      g = times_kw(g);
-    } else if (k - iters < Gt.size()) {
-      for (int m = 0; m < ns; ++m) out[2 * K + 1 + k * ns + m] = scale * average(Gt[k - iters], ns, m);
+    for (int m = 0; m < ns; ++m)
+      wg.push_back(k < it ? average(g, ns, m)
+                          : (k - it < Gt.size() ? scale * average(Gt[k - it], ns, m) : 0.0));
+    if (k < it) {
+      c = times_kw(c, phi((int)k));
+      g = times_kw(g, phi((int)k));
+    } else {
+      scale /= phi((int)k);
     }
-    scale /= phi((int)k);
   }
-  return out;
+  *levels = (int)K;
+  for (size_t k = 0; k < K; ++k) wk.push_back(phi((int)k));
+  wk.insert(wk.end(), wg.begin(), wg.end());
+  return wk;
 }
 
 // Solve A x = b for several right-hand sides (Gauss-Jordan, partial pivoting); A is m x m.
@@ -749,12 +762,11 @@ ader_status ader_create(const ader_config* cfg, void* stream, ader_ctx** out) {
   if (cfg->pde == ADER_PDE_ELASTIC && cfg->predictor == ADER_PREDICTOR_CK)
     for (int k = 0; k < cfg->order; ++k) rfx.push_back(1.0 / (k + 2));
   if (e == cudaSuccess && cfg->pde == ADER_PDE_ELASTIC && cfg->predictor == ADER_PREDICTOR_PICARD) {
-    // (a host allocation that fails for an absurd number of iterations is ADER_ENOMEM)
+    // (a host allocation that fails is ADER_ENOMEM)
     try {
       const int it = cfg->picard_iters > 0 ? cfg->picard_iters : cfg->order + 1;
       const bool cerk = cfg->initial_guess == ADER_GUESS_CERK;
-      const std::vector<double> lv = build_linear_levels(cfg->order, c->tab, it, cerk);
-      c->nlev = it + (cerk ? 4 : 0);
+      const std::vector<double> lv = build_linear_levels(cfg->order, c->tab, it, cerk, &c->nlev);
       e = cudaMalloc(&c->lin, lv.size() * sizeof(double));
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(c->lin, lv.data(), lv.size() * sizeof(double), cudaMemcpyHostToDevice,

@@ -40,6 +40,14 @@ def test_mixed(order, iters, guess):
     assert np.abs(out - ref).max() < 2e-6 * np.abs(ref - u).max()
 
 
+# iterations enough for the last weights to leave the range: the levels end before
+@pytest.mark.parametrize("guess", ["constant", "cerk"])
+@pytest.mark.parametrize("iters", [1021, 1024, 1025, 1100])
+def test_many_iterations(iters, guess):
+    out, ref, _ = run(1, iters, guess, "fp64")
+    assert rel_linf(out, ref) < 1e-12
+
+
 def device(a):
     return torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).cuda()
 
