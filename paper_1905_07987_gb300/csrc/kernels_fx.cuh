@@ -12,8 +12,8 @@
 // level, q^0 = u, so its right-hand side is formed once.
 //
 // Scale: one power of two per cell and quantity, one to two bits above its largest magnitude at
-// u^n: velocities s = |v| + c, momenta rho s, H (shallow water: s, h s, and |h + b| for the
-// surface); a flux has the product's scale.  An iterate above it, a non-finite value or magnitudes
+// u^n: velocities s = |v| + c, momenta rho s, H (shallow water: s, h s, and the larger of |h + b| and
+// h for the surface); a flux has the product's scale.  An iterate above it, a non-finite value or magnitudes
 // outside 2^-100 .. 2^100 end the attempt, and the cell is recomputed by the FP64 form
 // (predictor_cell), whose results for such values are kept as they were.  A contraction's rounding
 // is 2^-58 of the scale times the table's row sum: below the rounding of the FP64 FMA chain,
@@ -130,7 +130,7 @@ __device__ __forceinline__ bool fx_scales(const PdeParams& pp, const double* q, 
                                           FxScale& E, int tid) {
   using C = Cfg<P, D, N>;
   using X = FxCell<P, D, N>;
-  unsigned m[3] = {0u, 0u, 0u};  // Euler rho, H, s; shallow water h, |h + b|, s
+  unsigned m[3] = {0u, 0u, 0u};  // Euler rho, H, s; shallow water h, max(|h + b|, h), s
   for (int k = tid; k < C::NS; k += C::TPB) {
     const double* qn = q + k * C::NV;
     double v[D];
@@ -153,6 +153,10 @@ __device__ __forceinline__ bool fx_scales(const PdeParams& pp, const double* q, 
       m[i] = b > m[i] ? b : m[i];
     }
   }
+  // the surface may lie at the datum (still water with b = -h), and leave it by any factor in a step;
+  // h and b are rounded at 2^-53 of h themselves.  Water at rest, 256^2 cells, order 3: 4.0 ms in the
+  // FP64 form, 1.2 here.
+  if (!X::EULER && m[0] > m[1]) m[1] = m[0];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     const unsigned w = __reduce_max_sync(0xffffffffu, m[i]);
