@@ -66,17 +66,35 @@ __global__ void __launch_bounds__(128) k_ens_riemann(const StepArgs* __restrict_
   }
 }
 
-template <class P, int D, int N>
-__global__ void __launch_bounds__(CfgC<P, D, N>::TPB) k_ens_corrector(const StepArgs* __restrict__ R,
-                                                                     const __grid_constant__ EnsTable E) {
-  using X = CfgC<P, D, N>;
-  __shared__ SmemC<P, D, N, 1> S;
-  for (long long c = blockIdx.x; c < E.cell0[E.nr]; c += gridDim.x) {
-    const int r = ens_find(E.cell0, E.nr, c);
-    const int Ew = corrector_weights<D, N + 1>(R[r], S.w, threadIdx.x);
-    corrector_cells<P, D, N, 1, X::TPB>(R[r], S, Ew, E.phioff[1][r], E.phioff[2][r], c - E.cell0[r], 1,
-                                        threadIdx.x);
+// The corrector of all runs in groups of CPB concatenated cells, as the per-context kernel's blocks; a
+// group that spans runs is taken run by run.  A run's weights are formed when a block comes to it.
+// (One cell at a time left half to seven eighths of the threads idle at orders 1 to 4.)
+template <int N, int CPB, int NT>
+__device__ __forceinline__ void ens_corrector(const StepArgs* R, const EnsTable& E,
+                                              SmemC<Elastic, 3, N, CPB>& S) {
+  const long long total = E.cell0[E.nr];
+  int run = -1, Ew = 0;
+  for (long long b = (long long)blockIdx.x * CPB; b < total; b += (long long)gridDim.x * CPB) {
+    const long long end = b + CPB < total ? b + CPB : total;
+    for (long long c = b; c < end;) {
+      const int r = ens_find(E.cell0, E.nr, c);
+      const long long e = CPB == 1 || E.cell0[r + 1] > end ? end : E.cell0[r + 1];
+      // (with groups of one cell keeping the weights gains nothing)
+      if (CPB == 1 || r != run) Ew = corrector_weights<3, N + 1>(R[r], S.w, threadIdx.x);
+      run = r;
+      corrector_cells<Elastic, 3, N, CPB, NT>(R[r], S, Ew, E.phioff[1][r], E.phioff[2][r],
+                                              c - E.cell0[r], (int)(e - c), threadIdx.x);
+      c = e;
+    }
   }
+}
+
+template <int N>
+__global__ void __launch_bounds__(CfgC<Elastic, 3, N>::TPB)
+    k_ens_corrector(const StepArgs* __restrict__ R, const __grid_constant__ EnsTable E) {
+  using X = CfgC<Elastic, 3, N>;
+  __shared__ SmemC<Elastic, 3, N, X::CPB> S;
+  ens_corrector<N, X::CPB, X::TPB>(R, E, S);
 }
 
 // One step of every run: dt, predictor (`blocks` of them), Riemann per direction, corrector, time
@@ -102,7 +120,7 @@ cudaError_t ens_step_n(const StepArgs* R, const EnsTable& E, const Tables& T, co
     k_ens_riemann<Elastic, 3, N><<<152 * 16, 128, 0, s>>>(R, E, T, d);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_ens_corrector<Elastic, 3, N><<<152 * 8, CfgC<Elastic, 3, N>::TPB, 0, s>>>(R, E);
+  k_ens_corrector<N><<<152 * 8, CfgC<Elastic, 3, N>::TPB, 0, s>>>(R, E);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return launch_ens_advance(R, E.nr, s);
 }
@@ -148,9 +166,15 @@ __device__ __forceinline__ bool grid_sync(GridBar* b, unsigned nblocks, long lon
   return __syncthreads_and(ok) != 0;
 }
 
+// Cells of a group of the fused launch's corrector: a round of the predictor's threads.
+template <int N>
+__host__ __device__ constexpr int ens_fused_corrector_cells(int threads) {
+  return threads < 2 * CfgC<Elastic, 3, N>::LINES ? 1 : threads / CfgC<Elastic, 3, N>::LINES;
+}
+
 // `steps` steps of every run in one launch: per step the time-step finalisation, the predictor
 // over the concatenated cells, the Riemann solver over the concatenated faces of all directions,
-// the corrector over the concatenated degrees of freedom and the time advance, separated by
+// the corrector over groups of the concatenated cells and the time advance, separated by
 // grid-wide barriers.  Rsteps: the runs' step arguments of each step ([steps][nr]).
 template <int N, bool MIXED>
 __global__ void __launch_bounds__(EnsCfg<N, MIXED, true>::TPB, EnsCfg<N, MIXED, true>::MINB)
@@ -159,11 +183,10 @@ __global__ void __launch_bounds__(EnsCfg<N, MIXED, true>::TPB, EnsCfg<N, MIXED, 
                 GridBar* bar, long long limit) {
   using P = Elastic;
   constexpr int D = 3;
-  constexpr int n = N + 1, TPB = EnsCfg<N, MIXED, true>::TPB;
+  constexpr int TPB = EnsCfg<N, MIXED, true>::TPB;
   extern __shared__ __align__(16) double fsm[];
   const unsigned nb = gridDim.x;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const long long ncell = E.cell0[E.nr];
   bool ok = true;
   for (int s = 0; s < steps && ok; ++s) {
     const StepArgs* R = Rsteps + (long long)s * E.nr;
@@ -186,13 +209,8 @@ __global__ void __launch_bounds__(EnsCfg<N, MIXED, true>::TPB, EnsCfg<N, MIXED, 
     if (!(ok = grid_sync(bar, nb, limit))) break;
     {
       // over the predictor's shared memory
-      SmemC<P, D, N, 1>& S = *reinterpret_cast<SmemC<P, D, N, 1>*>(fsm);
-      for (long long c = blockIdx.x; c < ncell; c += nb) {
-        const int r = ens_find(E.cell0, E.nr, c);
-        const int Ew = corrector_weights<D, n>(R[r], S.w, threadIdx.x);
-        corrector_cells<P, D, N, 1, TPB>(R[r], S, Ew, E.phioff[1][r], E.phioff[2][r], c - E.cell0[r], 1,
-                                         threadIdx.x);
-      }
+      constexpr int CPB = ens_fused_corrector_cells<N>(TPB);
+      ens_corrector<N, CPB, TPB>(R, E, *reinterpret_cast<SmemC<P, D, N, CPB>*>(fsm));
     }
     if (!(ok = grid_sync(bar, nb, limit))) break;
     if (blockIdx.x == 0 && (int)threadIdx.x < E.nr) advance_one(R[threadIdx.x].dev, 0);
@@ -208,7 +226,7 @@ cudaError_t ens_fused_n(const StepArgs* R, const EnsTable& E, const Tables& T, c
                         int steps, GridBar* bar, long long limit, int blocks_per_sm,
                         cudaStream_t s) {
   using G = EnsCfg<N, MIXED, true>;
-  constexpr size_t SC = sizeof(SmemC<Elastic, 3, N, 1>);  // the corrector's
+  constexpr size_t SC = sizeof(SmemC<Elastic, 3, N, ens_fused_corrector_cells<N>(G::TPB)>);
   constexpr size_t SMEM = G::SMEM > SC ? G::SMEM : SC;
   static int max_bps = 0;
   if (!max_bps) {

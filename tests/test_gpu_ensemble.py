@@ -75,6 +75,26 @@ def test_ensemble_graph_equals_separate_runs(branches, spg, bps, prec):
     ens.close()
 
 
+# the corrector's groups of cells span runs and end in part-filled ones (1, 8, 27 cells)
+@pytest.mark.parametrize("order", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("launch", [(0, 2, 1), (-1, 2, 1)])
+def test_small_runs_in_the_shared_launches(order, launch):
+    sides = [1, 2, 1, 3, 1]
+    ens = ader.Ensemble(member_configs(sides, order))
+    singles = [ader.Context(c) for c in member_configs(sides, order)]
+    for i, s in enumerate(sides):
+        setup_member(ens.runs[i], s, order, seed=i)
+        setup_member(singles[i], s, order, seed=i)
+    ens.set_launch(*launch)
+    ens.step(4, dt=1e-3)
+    ens.sync()
+    for c in singles:
+        c.run(4, dt=1e-3)
+    for a, b in zip(states(ens.runs), states(singles)):
+        assert np.array_equal(a, b)
+    ens.close()
+
+
 @pytest.mark.parametrize("sides,order,launch", [([2, 3], 3, None), ([8, 10, 9], 3, None),
                                                 ([8, 10, 9], 3, (0, 2, 2)), ([12, 8], 4, (0, 2, 1)),
                                                 ([12, 8, 10], 4, (-1, 2, 1))])
