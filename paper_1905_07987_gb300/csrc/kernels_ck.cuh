@@ -77,6 +77,16 @@ __device__ __forceinline__ double ck_ricker(const StepArgs& A, const Tables& T, 
   return (1.0 - 2.0 * a) * exp(-a);
 }
 
+// The first M of them, to every lane of a warp: a lane forms one (a block's source costs a wavelet, not
+// M after one another).
+template <int N, int M>
+__device__ __forceinline__ void ck_samples(const StepArgs& A, const Tables& T, double tn, double dt,
+                                           double (&ric)[M]) {
+  const double r = ck_ricker<N>(A, T, (int)(threadIdx.x & 31) < M ? threadIdx.x & 31 : 0, tn, dt);
+#pragma unroll
+  for (int t = 0; t < M; ++t) ric[t] = __shfl_sync(0xffffffffu, r, t);
+}
+
 // gam_k of the Picard form's source levels from the samples s[n + 3].
 template <int N>
 __device__ __forceinline__ double lin_gamma(const StepArgs& A, const double* s, int k) {
@@ -175,10 +185,9 @@ __device__ __forceinline__ void predictor_ck_block(const StepArgs& A, const Tabl
   __shared__ int s_slot;
   const long long sc = A.src.cell - c0;
   const bool srcb = sc >= 0 && sc < ncb;  // uniform over the block
-  if (srcb && tid == 0) {
+  if (srcb && tid < 32) {
     double ric[PIC ? n + 3 : n], sbar = 0.0;
-#pragma unroll
-    for (int t = 0; t < (PIC ? n + 3 : n); ++t) ric[t] = ck_ricker<N>(A, T, t, tn, dt);
+    ck_samples<N>(A, T, tn, dt, ric);
 #pragma unroll
     for (int t = 0; t < n; ++t) sbar = fma(T.w[t], ric[t], sbar);
     if constexpr (PIC) {
@@ -523,10 +532,9 @@ __device__ __forceinline__ void predictor_ck_mixed_block(const StepArgs& A, cons
   __shared__ int s_slot;
   const long long sc = A.src.cell - c0;
   const bool srcb = sc >= 0 && sc < ncb;
-  if (srcb && tid == 0) {
+  if (srcb && tid < 32) {
     double ric[PIC ? n + 3 : n], sbar = 0.0;
-#pragma unroll
-    for (int t = 0; t < (PIC ? n + 3 : n); ++t) ric[t] = ck_ricker<N>(A, T, t, tn, dt);
+    ck_samples<N>(A, T, tn, dt, ric);
 #pragma unroll
     for (int t = 0; t < n; ++t) sbar = fma(T.w[t], ric[t], sbar);
     if constexpr (PIC) {
