@@ -1288,25 +1288,36 @@ ader_status ader_adjoint_step(ader_ctx* c, double t_n, double dt, const double* 
   if (!adjoint_supported(c)) return ADER_EUNSUPPORTED;
   if (!c->mat_set) return ADER_ESTATE;
   const bool ck = c->cfg.predictor == ADER_PREDICTOR_CK;
-  // levels: the adjoint of a polynomial of L (Cauchy-Kowalevski, or Picard when its levels fit)
-  const bool levels = ck || c->fam->adj_lin_fits(c->cfg.order, c->nlev);
+  // levels: the adjoint of a polynomial of L (Cauchy-Kowalevski, or Picard when its levels and
+  // lambda's projections, as large as the face adjoints, fit)
+  bool levels = ck || (c->dev_adj ? c->adj_spb == 0 : c->fam->adj_lin_fits(c->cfg.order, c->nlev));
   const int iters = c->cfg.picard_iters > 0 ? c->cfg.picard_iters : c->cfg.order + 1;
   if (!c->dev_adj) {
     int dev = 0, sms = 0;
     CUDA_OK(cudaGetDevice(&dev));
     CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // the adjoint of the levels keeps its cell in shared memory: no iterate slabs
-    c->adj_blocks = levels ? 0 : sms * c->fam->adj_blocks_per_sm(c->cfg.order);
-    c->adj_spb = levels ? 0 : c->fam->adj_scratch_per_block(c->cfg.order, iters);
     long long nfaces = 0;
     for (int d = 0; d < 3; ++d) nfaces += (long long)(c->g.n[d] + 1) * (c->g.ncells / c->g.n[d]);
     cudaError_t e = cudaMalloc(&c->dev_adj, sizeof(DevScalars));
     if (e == cudaSuccess) e = cudaMalloc(&c->adjf, (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&c->gface, (size_t)nfaces * 6 * sizeof(double));
-    // lambda's projections onto the cells' faces, or the iterate slabs
-    const size_t scratch = levels ? (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar
-                              : (size_t)c->adj_blocks * c->adj_spb;
-    if (e == cudaSuccess) e = cudaMalloc(&c->adj_scratch, scratch * sizeof(double));
+    // lambda's projections onto the cells' faces (the adjoint of the levels keeps its cell in shared
+    // memory), or the iterate slabs
+    c->adj_blocks = 0;
+    c->adj_spb = 0;
+    if (e == cudaSuccess && levels) {
+      e = cudaMalloc(&c->adj_scratch, (size_t)c->g.ncells * 3 * 2 * c->nf * c->nvar * sizeof(double));
+      if (e == cudaErrorMemoryAllocation && !ck) {
+        cudaGetLastError();
+        e = cudaSuccess;
+        levels = false;
+      }
+    }
+    if (e == cudaSuccess && !levels) {
+      c->adj_blocks = sms * c->fam->adj_blocks_per_sm(c->cfg.order);
+      c->adj_spb = c->fam->adj_scratch_per_block(c->cfg.order, iters);
+      e = cudaMalloc(&c->adj_scratch, (size_t)c->adj_blocks * c->adj_spb * sizeof(double));
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
       cudaFree(c->dev_adj);
