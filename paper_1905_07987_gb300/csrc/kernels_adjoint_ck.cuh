@@ -136,12 +136,13 @@ __device__ __forceinline__ void ck_rows(const double (&E)[9], double f, double i
   }
 }
 
-// gm += f nu^T (dL/d(rho, lam, mu)) a at one node from the strains E of a: no division, so a fluid
-// (mu = 0) or 3 lam + 2 mu = 0 is as exact as any material.
-__device__ __forceinline__ void ck_dmat_E(const double* E, const double (&nu)[9], double f,
-                                          double irho, double (&gm)[3]) {
-  gm[0] = fma(-f * irho * irho, fma(nu[0], E[0], fma(nu[1], E[1], nu[2] * E[2])), gm[0]);
-  gm[1] = fma(f * (E[3] + E[4] + E[5]), nu[3] + nu[4] + nu[5], gm[1]);
+// gm += f nu^T (dL/d(1/rho, lam, mu)) a at one node from the strains E of a (nsum = nu_3 + nu_4 + nu_5):
+// no division, so a fluid (mu = 0) or 3 lam + 2 mu = 0 is as exact as any material.  The sum over
+// the levels times -1/rho^2 is rho's.
+__device__ __forceinline__ void ck_dmat_E(const double* E, const double (&nu)[9], double nsum,
+                                          double f, double (&gm)[3]) {
+  gm[0] = fma(f, fma(nu[0], E[0], fma(nu[1], E[1], nu[2] * E[2])), gm[0]);
+  gm[1] = fma(f * nsum, E[3] + E[4] + E[5], gm[1]);
   const double s = fma(nu[3], E[3], fma(nu[4], E[4], nu[5] * E[5]));
   gm[2] = fma(f, fma(2.0, s, fma(nu[6], E[6], fma(nu[7], E[7], nu[8] * E[8]))), gm[2]);
 }
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
       for (int v = 0; v < NV; ++v) base[k * REC + j * NVP + v] = E[v];
     }
   }
-  double lam_j[NV], Fj[NV];
+  double lam_j[NV], Fj[NV], nsum = 0.0;  // nsum: nu_{k+1}'s stresses
   double gm[3] = {0.0, 0.0, 0.0}, gM[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   if (act) {
     // lambda at this node; its stress sum into the tenth slot of the record; its pairing with the
@@ -266,9 +267,9 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     double* lr = spare + j * NVP;
 #pragma unroll
     for (int v = 0; v < NV; ++v) lam_j[v] = lr[v];
-    lr[9] = lam_j[3] + lam_j[4] + lam_j[5];
+    lr[9] = nsum = lam_j[3] + lam_j[4] + lam_j[5];
     ck_strains<N>(last, j, Dr, A.g.inv_h, E);
-    ck_dmat_E(E, lam_j, dt * (1.0 / (N + 1)), irho, gm);
+    ck_dmat_E(E, lam_j, nsum, dt * (1.0 / (N + 1)), gm);
     // F: the face adjoints carried back to the nodes (transposed extrapolation)
 #pragma unroll
     for (int v = 0; v < NV; ++v) Fj[v] = 0.0;
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
     if (act) {
       if (k < N) {  // material: f_k nu_{k+1}^T (dL/dm) a_k from the strains of a_k
         const double f = dt * (1.0 / (k + 1));
-        ck_dmat_E(base + k * REC + j * NVP, nu_c, f, irho, gm);
+        ck_dmat_E(base + k * REC + j * NVP, nu_c, nsum, f, gm);
         if (srcc) {
           // moment: f_k s_k mu_{k+1}^T (dg/dM), mu_{k+1} = nu_{k+1} - lambda
 #pragma unroll
@@ -349,7 +350,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
         double* o = Yout + j * NVP;
 #pragma unroll
         for (int v = 0; v < NV; ++v) o[v] = nu_c[v];
-        o[9] = nu_c[3] + nu_c[4] + nu_c[5];
+        o[9] = nsum = nu_c[3] + nu_c[4] + nu_c[5];
       }
     }
     if (k > 0) __syncthreads();
@@ -377,6 +378,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
   // before the barrier that follows it): [9][NS]
   double* red = spare;
   if (act) {
+    gm[0] *= -irho * irho;
 #pragma unroll
     for (int q = 0; q < 3; ++q) red[q * NS + j] = gm[q];
     if (srcc)
@@ -445,7 +447,8 @@ __global__ void __launch_bounds__(256) k_adj_face_sum(const __grid_constant__ St
 
 // Forward and reverse levels of one sequence whose first level is in the record 0 of `base` ([K + 2]
 // records).  w(k): weight of level k.  Adds sum_k w_k a_k to qb and the material terms to gm; ab
-// returns ab_0.  All threads of the block; act: the thread has a node of the sequence.
+// returns ab_0.  (gm[0] is that of 1/rho.)  All threads of the block; act: the thread has a node of
+// the sequence.
 // A level that every neighbour has read gives its record to its strains, which nu is paired with;
 // the last level's record, whose strains are paired at once, becomes nu's second buffer.
 template <int N, class W>
@@ -481,8 +484,9 @@ __device__ __forceinline__ void adj_lin_levels(double* base, int K, bool act, in
         double* o = spare + j * NVP;
 #pragma unroll
         for (int v = 0; v < NV; ++v) o[v] = nu[v] = 2.0 * wk * lam_j[v];
-        o[9] = nu[3] + nu[4] + nu[5];
-        ck_dmat_E(E, nu, f, irho, gm);
+        const double nsum = nu[3] + nu[4] + nu[5];
+        o[9] = nsum;
+        ck_dmat_E(E, nu, nsum, f, gm);
       }
     }
     __syncthreads();
@@ -510,8 +514,9 @@ __device__ __forceinline__ void adj_lin_levels(double* base, int K, bool act, in
         double* o = Yout + j * NVP;
 #pragma unroll
         for (int v = 0; v < NV; ++v) o[v] = nu[v] = fma(wl, lam_j[v], ab[v]);
-        o[9] = nu[3] + nu[4] + nu[5];
-        ck_dmat_E(base + (k - 1) * REC + j * NVP, nu, dt * phi[k - 1], irho, gm);
+        const double nsum = nu[3] + nu[4] + nu[5];
+        o[9] = nsum;
+        ck_dmat_E(base + (k - 1) * REC + j * NVP, nu, nsum, dt * phi[k - 1], gm);
       }
     }
     __syncthreads();
@@ -633,6 +638,7 @@ __global__ void __launch_bounds__(CfgCKA<N>::TPB)
       base[j * NVP + v] = qb[v];
       base[REC + j * NVP + v] = lam_j[v] + ab[v];
     }
+    gm[0] *= -irho * irho;
 #pragma unroll
     for (int q = 0; q < 3; ++q) red[q * NS + j] = gm[q];
     if (srcc)
