@@ -44,9 +44,9 @@ FP64_SMS, FP64_FMA_PER_CLK, SM_MAX_MHZ = 152, 2, 2070.0
 TRAFFIC_PER_CELL = {"fp64": (331.102464e6 + 1031.607040e6) / 64000,
                     "mixed": (320.445184e6 + 1103.791872e6) / 64000}
 FP64_PEAK = FP64_SMS * FP64_FMA_PER_CLK * 2 * SM_MAX_MHZ * 1e6  # FLOP/s
-# the FP64 predictors run their products in 64-bit fixed point: four 32 x 32 + 64-bit integer
-# multiply-adds each, 64 of those per clock and SM
-FX_PEAK = FP64_SMS * 64 / 4 * 2 * SM_MAX_MHZ * 1e6  # FLOP/s, a multiply-add of the model = 2
+# 32 x 32 + 64-bit integer multiply-adds per second: the FP64 predictors' contractions are in 64-bit fixed
+# point
+MAD_PEAK = FP64_SMS * 64 * SM_MAX_MHZ * 1e6
 
 
 def predictor_flops_per_cell(pde, D, N, iters):
@@ -172,10 +172,26 @@ def model_flops_per_cell(D, N, nv, iters, cF=30):
     return iters * it + epi
 
 
+def fx_multiply_adds_per_cell(D, N, iters, cerk):
+    """Integer multiply-adds of the FP64 Euler predictor for one cell (k_predictor_fx): three per
+    product of the derivatives and of the flux (momentum or H times velocity), four per product of the
+    time solve, the time averages, the face values and the volume sum.  From the constant guess the
+    first iteration has one time level and no time solve; the Runge-Kutta guess has four."""
+    n, nv = N + 1, D + 2
+    nodes, lines = n ** D, n ** (D - 1) * nv
+    levels = 4 + iters * n if cerk else 1 + (iters - 1) * n
+    solves = iters if cerk else iters - 1
+    flux = D * nodes * (nv - 1) * 3           # of one time level
+    derivatives = D * nodes * nv * n * 3
+    epilogue = n * flux + 4 * D * (nodes * nv * n + 2 * lines * n + nodes * nv * (n + 2))
+    return levels * (derivatives + flux) + solves * nodes * nv * n * n * 4 + epilogue
+
+
 def measure_fma_peaks(stream):
-    """FP64 and binary32 FMA throughput of this GPU measured now (libpeaks.so: 8 independent FMA
-    chains per thread, 8 blocks of 256 threads per SM, CUDA events on the bench stream); returns
-    {"fp64": TFLOP/s, "fp32": TFLOP/s, ...} or None if the library is missing."""
+    """FP64 and binary32 FMA and integer multiply-add throughput of this GPU measured now (libpeaks.so:
+    8 independent chains per thread, 8 blocks of 256 threads per SM, CUDA events on the bench
+    stream); returns {"fp64": TFLOP/s, "fp32": TFLOP/s, "mad": 10^12 multiply-adds/s, ...} or None if
+    the library is missing."""
     import ctypes
     import torch
     path = os.path.join(ROOT, "paper_1905_07987_gb300", "peaks", "libpeaks.so")
@@ -192,20 +208,20 @@ def measure_fma_peaks(stream):
     out = {"method": "8 independent FMA chains per thread, %d blocks x 256 threads, best of 3 "
                      "CUDA-event timed launches" % blocks}
     sink = torch.empty(blocks * 256, dtype=torch.float64, device="cuda")
-    for name, fp64, iters in (("fp64", 1, 4000), ("fp32", 0, 60000)):
+    for name, kind, iters in (("fp64", 1, 4000), ("fp32", 0, 60000), ("mad", 2, 60000)):
         with torch.cuda.stream(stream):
-            L.peaks_fma_launch(fp64, sink.data_ptr(), blocks, 200, stream.cuda_stream)  # warm-up
+            L.peaks_fma_launch(kind, sink.data_ptr(), blocks, 200, stream.cuda_stream)  # warm-up
             best = None
             for _ in range(3):
                 e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                 e0.record(stream)
-                if L.peaks_fma_launch(fp64, sink.data_ptr(), blocks, iters, stream.cuda_stream) != 0:
+                if L.peaks_fma_launch(kind, sink.data_ptr(), blocks, iters, stream.cuda_stream) != 0:
                     return None
                 e1.record(stream)
                 torch.cuda.synchronize()
                 ms = e0.elapsed_time(e1)
                 best = ms if best is None else min(best, ms)
-        out[name] = L.peaks_fma_flops(blocks, iters) / (best * 1e-3) / 1e12
+        out[name] = L.peaks_fma_flops(blocks, iters) / (best * 1e-3) / 1e12 / (2 if kind == 2 else 1)
         out[name + "_ms"] = best
     return out
 
@@ -1158,9 +1174,15 @@ def main():
         pred_ms = r["phases"]["predictor"] / nrec
         achieved = flops_model / (pred_ms * 1e-3) / 1e12
         key = "fp64" if prec == "fp64" else "fp32"
-        derived = (FX_PEAK if prec == "fp64" else FP32_PEAK) / 1e12
+        derived = FP32_PEAK / 1e12
         if prec == "fp64":
-            peak, src = derived, "derived: 152 SMs x 64 integer multiply-adds/clk / 4 per product x 2 flop x 2070 MHz"
+            # the model flops at which the multiply-adds alone would take the kernel's time
+            mads = fx_multiply_adds_per_cell(D, N, FORMS[form][2] or N + 1, FORMS[form][1] == "cerk")
+            derived = flops_model / (mads * cells) * MAD_PEAK / 1e12
+            peak = derived * peaks["mad"] * 1e12 / MAD_PEAK if peaks else derived
+            src = "model flops over %d integer multiply-adds a cell at %s a second" % (
+                mads, "the %.3g 10^12 measured in this run (libpeaks)" % peaks["mad"] if peaks else
+                "152 SMs x 64/clk x 2070 MHz (derived)")
         elif peaks and peaks.get(key):
             peak, src = peaks[key], "measured in this run (%s FMA throughput, libpeaks)" % key.upper()
         else:
