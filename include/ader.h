@@ -73,13 +73,16 @@ typedef enum { ADER_BC_PERIODIC = 0, ADER_BC_WALL = 1, ADER_BC_ABSORBING = 2 } a
 
 /* Arithmetic of the step:
  *  FP64  - everything in binary64 or, where a cell's values share a scale, in 64-bit fixed point
- *          relative to the cell's largest value (rounding 2^-57 of it; non-finite values and
- *          magnitudes near the ends of the range are computed in binary64);
+ *          relative to the cell's largest value of the quantity (rounding 2^-57 of it, so a value
+ *          far below it keeps fewer bits of its own; non-finite values and magnitudes near the
+ *          ends of the range are computed in binary64);
  *  MIXED - predictor iterations on the increment q - u^n in binary32 with float-float base
  *          terms, time averages and contractions.  Pressure / sound speed and eigenvalues, the
- *          Riemann flux, the corrector and the limiter stay binary64 (for Euler the face wave
- *          speeds are evaluated by the predictor, and the CFL maximum only on the nodes that a
- *          binary32 enclosure cannot rule out; dt equals the FP64 form's on the same state);
+ *          Riemann flux, the corrector and the limiter are those of the FP64 form: binary64, the
+ *          corrector's sums in 3-D from order 3 and the limiter's projections in 64-bit fixed
+ *          point (for Euler the face wave speeds are evaluated by the predictor, and the CFL
+ *          maximum only on the nodes that a binary32 enclosure cannot rule out; dt equals the FP64
+ *          form's on the same state);
  *  MIXED_TF32X3 - the Cauchy-Kowalevski predictor of the elastic family (orders 1, 3, 5) with
  *          every contraction on the tensor cores (tcgen05.mma kind::tf32): the derivatives of the
  *          Taylor coefficients and the face extrapolation of the time average as products with
@@ -104,8 +107,8 @@ typedef enum { ADER_PREC_FP64 = 0, ADER_PREC_MIXED = 1, ADER_PREC_MIXED_TF32X3 =
  *           ADER_PREC_MIXED (the O(1) base term L u and the first Taylor coefficient in
  *           float-float or, from order 5, in 64-bit fixed point, the higher coefficients in
  *           binary32, the update u + dt vol in FP64).
- *           Differentiated (orders 1-5): the adjoint entry points take the FP64 adjoint of the
- *           Taylor recursion. */
+ *           Differentiated (orders 1-5): the adjoint entry points take the adjoint of the
+ *           Taylor recursion (its precision: see ader_adjoint_step). */
 typedef enum { ADER_PREDICTOR_PICARD = 0, ADER_PREDICTOR_CK = 1 } ader_predictor;
 
 /* Initial guess of the Picard predictor (Sec. 5):
@@ -273,11 +276,14 @@ ader_status ader_run_graph(ader_ctx* ctx, int steps, int replays, double dt, dou
  * and accumulates  grad_mat[c][0..2] += d/d(rho, lambda, mu)_c of (lambda^{n+1})^T u^{n+1}  and
  * grad_M[0..5] += d/dM of the same, evaluated at the forward state u_n = u^n with the step
  * starting at time t_n.  With the Picard predictor this is the adjoint of the FP64 step (a MIXED
- * context too), as the adjoint of the polynomial in dt L that the iterates are.  With the
- * Cauchy-Kowalevski predictor an FP64 context gets the adjoint of its FP64 step, a MIXED or TF32X3 context a mixed-precision adjoint: the base term F + dt L^T lambda
- * in float-float, the level corrections dt L^T mu in binary32, lambda + mu_0 in FP64 (within a
- * few binary32 roundoffs, relative to the largest value, of the FP64 adjoint).  The wave speed max(vp_L, vp_R) of a face takes the left value at
- * ties.  The gradient sums are formed in a fixed order: repeated calls give identical bits.
+ * context too), as the adjoint of the polynomial in dt L that the iterates are (where its work
+ * buffers do not fit the device, of the iterates themselves).  With the Cauchy-Kowalevski predictor
+ * an FP64 context gets the adjoint of its FP64 step, a MIXED or TF32X3 context a mixed-precision
+ * adjoint: the base term F + dt L^T lambda in float-float, the level corrections dt L^T mu in
+ * binary32, lambda + mu_0 in FP64 (within a few binary32 roundoffs, relative to the largest value,
+ * of the FP64 adjoint).  The wave speed max(vp_L, vp_R) of a face takes the left value at ties.  The
+ * material may be any that the step accepts, a fluid (mu = 0) and 3 lambda + 2 mu = 0 among them.
+ * The gradient sums are formed in a fixed order: repeated calls give identical bits.
  * All pointers are device memory of the context's device ([cells][nodes][9] for u_n, lam, dJdu;
  * [cells][3]; [6]); dJdu may be NULL.  Uses the context's material, point source and order; the
  * context's own state and time are not touched.  Stream-ordered, no synchronisation.  The first
@@ -290,7 +296,8 @@ ader_status ader_adjoint_step(ader_ctx* ctx, double t_n, double dt, const double
 /* Same result as ader_adjoint_step, but this call allocates no memory: its work buffers (the
  * forward Picard iterates kept per thread block (none with the Cauchy-Kowalevski predictor, nor
  * with the Picard predictor where the buffers of the polynomial form fit), the face adjoints and
- * the per-face material gradients) live in one fixed 64 MiB array of device memory that the library defines, so no
+ * the per-face material gradients) live in one fixed 64 MiB array of device memory that the
+ * library defines, so no
  * cudaMalloc, cudaFree or other allocating call is made.  It exists for callers that cannot
  * allocate device memory at the time of the call: for example code whose device memory is
  * owned by another allocator (a framework's memory pool that has reserved the GPU), processes
@@ -340,8 +347,9 @@ ader_status ader_misfit_gradient(ader_ctx* ctx, const double* u0, double t0, dou
                                  double* grad_M);
 
 /* Per-phase device timing.  While enabled, every ader_step records CUDA events on the context's
- * stream around its phases: 0 CFL speed reduction, 1 dt finalisation, 2 predictor, 3 Riemann,
- * 4 corrector, 5 limiter, 6 receivers and time advance.  ader_phase_times synchronises, writes
+ * stream around its phases: 0 CFL speed reduction and the dt from it, 1 a fixed dt, 2 predictor,
+ * 3 Riemann, 4 corrector (advances the time when there are no receivers), 5 limiter, 6 receivers and
+ * the time advance with them.  ader_phase_times synchronises, writes
  * the summed milliseconds of each phase over the recorded steps to ms[7], the number of recorded
  * steps to *steps, and clears the record.  Timing adds no synchronisation between steps. */
 ader_status ader_enable_timing(ader_ctx* ctx, int on);

@@ -911,8 +911,8 @@ __global__ void __launch_bounds__(256) k_corrector(const __grid_constant__ StepA
 // fluxes stay in its registers, and the line's index also names one value of every face, so the
 // same thread loads and converts these six.
 // The results depend on the cell's data alone: every kernel that calls this gives the same bits.
-// Measured, 64^3 cells: elastic order 5 5.80 -> 3.67 ms, order 3 1.77 -> 1.12; Euler order 4 1.78 ->
-// 1.07, order 3 0.91 -> 0.63 (order 2: 0.39 and 0.40; elastic order 1 0.21 and 0.23, so orders 1
+// Measured, 64^3 cells: elastic order 5 5.80 -> 3.42 ms, order 3 1.77 -> 1.06; Euler order 4 1.78 ->
+// 1.00, order 3 0.91 -> 0.60 (order 2: 0.39 and 0.40; elastic order 1 0.21 and 0.23, so orders 1
 // and 2 keep the FP64 form).  A step's error against binary64 falls with it (1.6e-16 -> 1.3e-16 of
 // the state, Euler order 4): one rounding of u in place of six.
 template <class P, int D, int N>
